@@ -153,6 +153,7 @@ sph_status sph_create(sph_ctx **out, int32_t dim, int64_t max_particles, int32_t
   c->need_walk = ctx_alloc<int32_t>(c, 1, ok);
   c->csr_total = ctx_alloc<int64_t>(c, 1, ok);
   c->hflags = ctx_alloc<int32_t>(c, kMaxHIter + 3, ok);
+  c->vol = ctx_alloc<double>(c, N, ok);
   c->T = ctx_alloc<double>(c, 8 * N, ok);
   c->zeta = ctx_alloc<double>(c, 8 * N, ok);
   c->cs = ctx_alloc<double>(c, N, ok);
@@ -326,7 +327,8 @@ double velocity_scale(const MatTable &mt) {
 }
 }  // namespace sph
 
-static void set_materials(sph_ctx *c, const MatTable *mt) {
+static void set_materials(sph_ctx *c, const MatTable *mt, const sph_params *p = nullptr) {
+  c->pk.vol = p && p->precision == SPH_FP64 ? c->vol : nullptr;
   if (mt) {
     c->mt = *mt;
     c->vscale = velocity_scale(*mt);
@@ -514,7 +516,7 @@ sph_status sph_rhs(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t n
   if (s->n > 0 && s->S && !out->dS) return fail(c, SPH_ERR_INVALID, "dS output required when S is given");
   if (s->n > 0 && s->dmg && !out->ddmg) return fail(c, SPH_ERR_INVALID, "ddmg output required when dmg is given");
   cudaStream_t st = (cudaStream_t)stream;
-  set_materials(c, &mt);
+  set_materials(c, &mt, p);
   rhs_all(c, s, mt, *p, *out, st);
   return finish(c, p, st, "sph_rhs");
 }
@@ -598,7 +600,7 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
   if ((r = check_params(c, s, mats, nmat, p, mt)) != SPH_OK) return r;
   if (nsteps < 0) return fail(c, SPH_ERR_INVALID, "nsteps < 0");
   cudaStream_t st = (cudaStream_t)stream;
-  set_materials(c, &mt);
+  set_materials(c, &mt, p);
   StepBufs &B = c->st;
   const int ninst = s->ninst > 0 ? s->ninst : 1;
   // predicted state shares m, h, mat, id, flaws and instances with s
@@ -728,7 +730,7 @@ sph_status sph_step_rk3(sph_ctx *c, sph_state *s, const sph_material *mats, int3
   if ((r = check_params(c, s, mats, nmat, p, mt)) != SPH_OK) return r;
   if (nsteps < 0 || !dt || !(eps_des > 0.0)) return fail(c, SPH_ERR_INVALID, "need dt, eps_des > 0, nsteps >= 0");
   cudaStream_t st = (cudaStream_t)stream;
-  set_materials(c, &mt);
+  set_materials(c, &mt, p);
   StepBufs &B = c->st;
   const int ninst = s->ninst > 0 ? s->ninst : 1;
   // stage states share m, h, mat, id, flaws and instances with s
@@ -815,7 +817,7 @@ sph_status sph_rhs_adjoint(sph_ctx *c, sph_state *s, const sph_material *mats, i
     if (!sbar->rho || !sbar->u || (s->S && !sbar->S)) return fail(c, SPH_ERR_INVALID, "state_bar rho, u, S required");
   }
   cudaStream_t st = (cudaStream_t)stream;
-  set_materials(c, &mt);
+  set_materials(c, &mt, p);
   sph_params q = *p;
   // forward evaluation in the requested precision: partner lists, T = sigma /
   // rho^2 and c_s (FP64 arrays, or the FP32 code-unit views of the mixed form)

@@ -30,6 +30,7 @@ __device__ __forceinline__ void pack_particle(const PackedF32 &pk, int64_t i, in
   pk.pxl(i) = make_float4(xl[0], xl[1], xl[2], mf);
   pk.pv(i) = make_float4(vh[0], vh[1], vh[2], rf);
   pk.pvl(i) = make_float4(vl[0], vl[1], vl[2], __fdiv_rn(mf, rf));
+  if (pk.vol) pk.vol[i] = m / rho;
 }
 
 }  // namespace sph

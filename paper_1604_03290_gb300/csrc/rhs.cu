@@ -32,6 +32,7 @@
 #include <type_traits>
 
 #include "eos.cuh"
+#include "fp64fast.cuh"
 #include "fpbits.cuh"
 #include "sph_internal.cuh"
 
@@ -63,16 +64,7 @@ struct RhsArgs {
   int32_t *err;
 };
 
-template <class R>
-__device__ __forceinline__ R rsqrt_or_zero(R r2);
-template <>
-__device__ __forceinline__ float rsqrt_or_zero<float>(float r2) {
-  return r2 > 0.f ? rsqrtf(r2) : 0.f;
-}
-template <>
-__device__ __forceinline__ double rsqrt_or_zero<double>(double r2) {
-  return r2 > 0.0 ? 1.0 / sqrt(r2) : 0.0;
-}
+__device__ __forceinline__ float rsqrt_or_zero(float r2) { return r2 > 0.f ? rsqrtf(r2) : 0.f; }
 
 // Resident blocks per SM the neighbour passes are compiled for (register
 // budget).  Measured on GB300 with the partner prefetch below: pass A is
@@ -100,17 +92,14 @@ __device__ __forceinline__ double rcp_rn<double>(double x) {
   return __drcp_rn(x);
 }
 
-// Reciprocal and quotient inside the pair loops.  Mixed: the hardware's
+// Reciprocal and quotient inside the mixed pair loops: the hardware's
 // approximations (relative error below 2^-22, a few FP32 roundings of a pair
 // term, well inside the mixed tolerance; operands are in code units, far from
-// the subnormal range).  FP64: correctly rounded, as everywhere else.
+// the subnormal range).
 #ifndef SPH_FAST_PAIR_MATH
 #define SPH_FAST_PAIR_MATH 1
 #endif
-template <class R>
-__device__ __forceinline__ R pair_rcp(R x);
-template <>
-__device__ __forceinline__ float pair_rcp<float>(float x) {
+__device__ __forceinline__ float pair_rcp(float x) {
 #if SPH_FAST_PAIR_MATH
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -119,23 +108,12 @@ __device__ __forceinline__ float pair_rcp<float>(float x) {
   return __frcp_rn(x);
 #endif
 }
-template <>
-__device__ __forceinline__ double pair_rcp<double>(double x) {
-  return __drcp_rn(x);
-}
-template <class R>
-__device__ __forceinline__ R pair_div(R a, R b);
-template <>
-__device__ __forceinline__ float pair_div<float>(float a, float b) {
+__device__ __forceinline__ float pair_div(float a, float b) {
 #if SPH_FAST_PAIR_MATH
   return __fdividef(a, b);
 #else
   return a / b;
 #endif
-}
-template <>
-__device__ __forceinline__ double pair_div<double>(double a, double b) {
-  return a / b;
 }
 
 // ---------------------------------------------------------------------------
@@ -146,38 +124,11 @@ struct Own;
 
 template <>
 struct Own<false> {
-  double x[3], v[3], h, rho, m;
+  double h, rho, m;
   __device__ void load(const RhsArgs &A, int64_t a) {
-    for (int ax = 0; ax < 3; ++ax) {
-      x[ax] = ax < A.dim ? A.x[ax][a] : 0.0;
-      v[ax] = ax < A.dim ? A.v[ax][a] : 0.0;
-    }
     h = A.h[a];
     rho = A.rho[a];
     m = A.m[a];
-  }
-  // d = x_a - x_b, w = v_a - v_b
-  __device__ __forceinline__ void pair(const RhsArgs &A, int32_t b, double d[3], double w[3], double &hb,
-                                       double &rhob, double &mb, double &vol) const {
-    for (int ax = 0; ax < 3; ++ax) {
-      d[ax] = ax < A.dim ? x[ax] - A.x[ax][b] : 0.0;
-      w[ax] = ax < A.dim ? v[ax] - A.v[ax][b] : 0.0;
-    }
-    hb = A.h[b];
-    rhob = A.rho[b];
-    mb = A.m[b];
-    vol = mb / rhob;
-  }
-  // the same split into the loads of b (issued ahead) and the arithmetic
-  struct Raw {
-    int32_t b;
-  };
-  using RawPos = Raw;
-  __device__ __forceinline__ Raw fetch(const RhsArgs &, int32_t b) const { return Raw{b}; }
-  __device__ __forceinline__ Raw fetch_pos(const RhsArgs &, int32_t b) const { return Raw{b}; }
-  __device__ __forceinline__ void from(const RhsArgs &A, const Raw &r, double d[3], double w[3], double &hb,
-                                       double &rhob, double &mb, double &vol) const {
-    pair(A, r.b, d, w, hb, rhob, mb, vol);
   }
 };
 
@@ -291,6 +242,50 @@ struct PartnerCursor {
 };
 
 // ---------------------------------------------------------------------------
+// FP64 pair sums.  Bound by the FP64 unit, so each pair is written in as few
+// FP64 instructions as its terms need: reciprocals from fp64fast.cuh, V_b read
+// from an array (one gather instead of a division), powers of 1/h_ab kept
+// while h_b stays the same from partner to partner (a bit test), the kernel
+// slope as one product of two linear factors whose coefficients are selected
+// by the branch, and the kernel norm applied to the sums.
+// ---------------------------------------------------------------------------
+template <int DIM>
+struct Support64 {
+  double ha, hab, hinv, hD, hD1;  // h_a, h_ab, 1/h_ab, its powers D and D + 1
+  uint64_t last;                  // bits of the h_b these belong to
+  __device__ __forceinline__ void set(double hb) {
+    last = dbits(hb);
+    hab = 0.5 * (ha + hb);
+    hinv = rcp64(hab);
+    const double i2 = hinv * hinv;
+    hD = DIM == 3 ? i2 * hinv : i2;
+    hD1 = hD * hinv;
+  }
+  __device__ __forceinline__ void start(double h) {
+    ha = h;
+    set(h);
+  }
+  __device__ __forceinline__ void partner(double hb) {
+    if (dbits(hb) != last) set(hb);
+  }
+};
+
+// q < 1/2 for q >= 0, from the bits
+__device__ __forceinline__ bool below_half(double q) { return __double2hiint(q) < 0x3fe00000; }
+
+// (h^(D+1) / 6 sigma) dW/dr at q = r/h: q (3q - 2), or -(1 - q)^2 from q = 1/2
+__device__ __forceinline__ double slope64(double q) {
+  const bool in = below_half(q);
+  const double a1 = in ? 1.0 : -1.0, b1 = in ? 0.0 : 1.0, c1 = in ? 3.0 : 1.0, d1 = in ? -2.0 : -1.0;
+  return fma(a1, q, b1) * fma(c1, q, d1);
+}
+// (h^D / sigma) W: 1 + 6 q^2 (q - 1), or 2 (1 - q)^3
+__device__ __forceinline__ double value64(double q) {
+  const double t = below_half(q) ? q : 1.0 - q, t2 = t * t;
+  return below_half(q) ? fma(6.0 * t2, t - 1.0, 1.0) : 2.0 * t2 * t;
+}
+
+// ---------------------------------------------------------------------------
 // Density by kernel sum (Eq. density_by_kernel_sum) including m_a W(0; h_a).
 // ---------------------------------------------------------------------------
 template <bool MIXED, int DIM>
@@ -309,14 +304,32 @@ __global__ void __launch_bounds__(128) k_density_sum(RhsArgs A) {
   }
   const int32_t *list;
   const int cnt = partner_list(A, a, list);
-  for (int k = 0; k < cnt; ++k) {
-    const int32_t b = list[(int64_t)k * A.ld];
-    R d[3], w[3], hb, rhob, mb, vol;
-    o.pair(A, b, d, w, hb, rhob, mb, vol);
-    R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    R r = r2 * rsqrt_or_zero(r2);
-    R hinv = pair_rcp(R(0.5) * ((R)o.h + hb));
-    sum.add(mb * kern_W(r * hinv, sig * hpow(hinv, dim)));
+  if constexpr (!MIXED) {
+    Support64<DIM> H;
+    H.start(o.h);
+    double w = 0.0;
+    for (int k = 0; k < cnt; ++k) {
+      const int32_t b = list[(int64_t)k * A.ld];
+      double r2 = 0.0;
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) {
+        const double d = A.x[i][a] - A.x[i][b];
+        r2 = fma(d, d, r2);
+      }
+      H.partner(A.h[b]);
+      w = fma(A.m[b] * H.hD, value64(r2 * rsqrt64(r2) * H.hinv), w);
+    }
+    sum.add(sig * w);
+  } else {
+    for (int k = 0; k < cnt; ++k) {
+      const int32_t b = list[(int64_t)k * A.ld];
+      R d[3], w[3], hb, rhob, mb, vol;
+      o.pair(A, b, d, w, hb, rhob, mb, vol);
+      R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+      R r = r2 * rsqrt_or_zero(r2);
+      R hinv = pair_rcp(R(0.5) * ((R)o.h + hb));
+      sum.add(mb * kern_W(r * hinv, sig * hpow(hinv, dim)));
+    }
   }
   A.rho_out[a] = sum.value() * (MIXED ? A.U->rho : 1.0);
 }
@@ -365,12 +378,39 @@ __device__ __forceinline__ void correction_tensor(int dim, const R L[3][3], bool
 // eigenvectors).  Each rotation zeroes A[p][q] with t = tan of the angle,
 // t = sign(tau)/(|tau| + sqrt(1 + tau^2)), tau = (A_qq - A_pp)/(2 A_pq).
 template <class R>
+__device__ __forceinline__ void jacobi_angle(R app, R aqq, R apq, R &t, R &c) {
+  R tau = (aqq - app) / (R(2) * apq);
+  t = (tau >= R(0) ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
+  c = R(1) / sqrt(R(1) + t * t);
+}
+static __device__ __noinline__ double2 jacobi_angle_slow(double app, double aqq, double apq) {
+  double2 r;
+  jacobi_angle<double>(app, aqq, apq, r.x, r.y);
+  return r;
+}
+// FP64: the same tangent as a_pq / (e + sign(e) sqrt(e^2 + a_pq^2)), e = (a_qq
+// - a_pp) / 2, from the reciprocals of fp64fast.cuh (22 instead of 60 FP64
+// instructions for the angle); out of their range, the form above
+__device__ __forceinline__ void jacobi_angle(double app, double aqq, double apq, double &t, double &c) {
+  const double e = 0.5 * (aqq - app), m = fma(e, e, apq * apq);
+  if (!mid_range(m)) {
+    const double2 r = jacobi_angle_slow(app, aqq, apq);
+    t = r.x;
+    c = r.y;
+    return;
+  }
+  const double root = m * rsqrt64(m);
+  t = apq * rcp64((int64_t)dbits(e) < 0 ? e - root : e + root);
+  c = rsqrt64(fma(t, t, 1.0));
+}
+
+template <class R, bool VECS>
 __device__ __forceinline__ void jacobi_rotate(int p, int q, R A[3][3], R V[3][3], int dim) {
   R apq = A[p][q];
   if (apq == R(0)) return;
-  R tau = (A[q][q] - A[p][p]) / (R(2) * apq);
-  R t = (tau >= R(0) ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
-  R c = R(1) / sqrt(R(1) + t * t), s = t * c;
+  R t, c;
+  jacobi_angle(A[p][p], A[q][q], apq, t, c);
+  const R s = t * c;
   A[p][p] -= t * apq;
   A[q][q] += t * apq;
   A[p][q] = A[q][p] = R(0);
@@ -380,30 +420,85 @@ __device__ __forceinline__ void jacobi_rotate(int p, int q, R A[3][3], R V[3][3]
       A[r][p] = A[p][r] = c * arp - s * arq;
       A[r][q] = A[q][r] = s * arp + c * arq;
     }
-    R vrp = V[r][p], vrq = V[r][q];
-    V[r][p] = c * vrp - s * vrq;
-    V[r][q] = s * vrp + c * vrq;
+    if constexpr (VECS) {
+      R vrp = V[r][p], vrq = V[r][q];
+      V[r][p] = c * vrp - s * vrq;
+      V[r][q] = s * vrp + c * vrq;
+    }
   }
 }
 
-template <class R>
+// VECS: also the eigenvectors
+template <class R, bool VECS>
 __device__ __forceinline__ void sym_eigen(int dim, R A[3][3], R w[3], R V[3][3]) {
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) V[i][j] = i == j ? R(1) : R(0);
   if (dim == 2) {
-    jacobi_rotate(0, 1, A, V, 2);
+    jacobi_rotate<R, VECS>(0, 1, A, V, 2);
   } else {
     const R tiny = sizeof(R) == 4 ? R(1e-14) : R(1e-30);
     for (int sweep = 0; sweep < 12; ++sweep) {
       R off = A[0][1] * A[0][1] + A[0][2] * A[0][2] + A[1][2] * A[1][2];
       R dg = A[0][0] * A[0][0] + A[1][1] * A[1][1] + A[2][2] * A[2][2];
       if (!(off > tiny * dg)) break;
-      jacobi_rotate(0, 1, A, V, 3);
-      jacobi_rotate(0, 2, A, V, 3);
-      jacobi_rotate(1, 2, A, V, 3);
+      jacobi_rotate<R, VECS>(0, 1, A, V, 3);
+      jacobi_rotate<R, VECS>(0, 2, A, V, 3);
+      jacobi_rotate<R, VECS>(1, 2, A, V, 3);
     }
   }
   for (int i = 0; i < 3; ++i) w[i] = i < dim ? A[i][i] : R(0);
+}
+
+template <int DIM>
+__device__ __forceinline__ void pairs_A64(const RhsArgs &A, int64_t a, const int32_t *list, int cnt, bool xsph,
+                                          double L[3][3], double G[3][3], double xs[3]) {
+  double xa[DIM], va[DIM];
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
+    xa[i] = A.x[i][a];
+    va[i] = A.v[i][a];
+  }
+  const double rhoa = A.rho[a];
+  Support64<DIM> H;
+  H.start(A.h[a]);
+  for (int k = 0; k < cnt; ++k) {
+    const int32_t b = list[(int64_t)k * A.ld];
+    double d[DIM], w[DIM], gd[DIM], r2 = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      d[i] = xa[i] - A.x[i][b];
+      w[i] = va[i] - A.v[i][b];
+      r2 = fma(d[i], d[i], r2);
+    }
+    H.partner(A.h[b]);
+    const double rinv = rsqrt64(r2);
+    const double q = r2 * rinv * H.hinv;
+    const double f = slope64(q) * H.hD1 * rinv * A.pk.vol[b];  // V_b (dW/dr) / (6 sigma r)
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) gd[i] = f * d[i];
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) {
+        if (j <= i) L[i][j] = fma(-gd[i], d[j], L[i][j]);
+        G[i][j] = fma(-w[i], gd[j], G[i][j]);
+      }
+    if (xsph) {
+      const double c = A.m[b] * rcp64(rhoa + A.rho[b]) * (value64(q) * H.hD);
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) xs[i] = fma(-c, w[i], xs[i]);
+    }
+  }
+  const double sig = kernel_sigma<double>(DIM);
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
+    xs[i] *= 2.0 * sig;
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) {
+      L[i][j] *= 6.0 * sig;
+      G[i][j] *= 6.0 * sig;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -413,7 +508,12 @@ __device__ __forceinline__ void sym_eigen(int dim, R A[3][3], R w[3], R V[3][3])
 // rows of stride ld: 0 the continuity sum sum_b V_b (v_a - v_b).grad W (code
 // units 1/T), 1..6 the lower triangle of L (00, 10, 11, 20, 21, 22), 7..15 G
 // row by row (1/T).
-template <bool MIXED, int DIM, bool KEEP_SUMS = false>
+// AS = false: no artificial stress, the only user of the principal frame's
+// axes, so only the principal values are formed (for the damage strain).  The
+// mixed form is instantiated with AS alone, where the parameter decides: its
+// own instance without the axes was slower (0.487 against 0.446 ms per 1M
+// launch, at the same 72 registers).
+template <bool MIXED, bool AS, int DIM, bool KEEP_SUMS = false>
 __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
   using R = typename std::conditional<MIXED, float, double>::type;
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -431,42 +531,49 @@ __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
     for (int j = 0; j < 3; ++j) L[i][j] = G[i][j] = R(0);
   const int32_t *list;
   const int cnt = partner_list(A, a, list);
+  if constexpr (!MIXED) {
+    pairs_A64<DIM>(A, a, list, cnt, xsph, L, G, xs);
+    double tr = 0.0;  // sum_b V_b (v_a - v_b).grad W = -tr G
+    for (int i = 0; i < dim; ++i) tr += G[i][i];
+    drho.add(-tr);
+  } else {
 #if SPH_PASS_PREFETCH
-  PartnerCursor<MIXED, true> cur;
-  cur.start(A, o, list, cnt);
+    PartnerCursor<MIXED, true> cur;
+    cur.start(A, o, list, cnt);
 #endif
-  for (int k = 0; k < cnt; ++k) {
-    R d[3], w[3], hb, rhob, mb, vol;
+    for (int k = 0; k < cnt; ++k) {
+      R d[3], w[3], hb, rhob, mb, vol;
 #if SPH_PASS_PREFETCH
-    typename PartnerCursor<MIXED, true>::Raw raw;
-    cur.next(A, o, k, raw);
-    o.from(A, raw, d, w, hb, rhob, mb, vol);
+      typename PartnerCursor<MIXED, true>::Raw raw;
+      cur.next(A, o, k, raw);
+      o.from(A, raw, d, w, hb, rhob, mb, vol);
 #else
-    const int32_t b = list[(int64_t)k * A.ld];
-    o.pair(A, b, d, w, hb, rhob, mb, vol);
+      const int32_t b = list[(int64_t)k * A.ld];
+      o.pair(A, b, d, w, hb, rhob, mb, vol);
 #endif
-    const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    const R rinv = rsqrt_or_zero(r2);
-    const R r = r2 * rinv;
-    const R hinv = pair_rcp(R(0.5) * (ha + hb));
-    const R q = r * hinv;
-    const R hD = hpow(hinv, dim);
-    const R fr = kern_dW(q, R(6) * sig * hD * hinv) * rinv;
-    R g[3] = {fr * d[0], fr * d[1], fr * d[2]};
-    drho.add(vol * (w[0] * g[0] + w[1] * g[1] + w[2] * g[2]));
-    // L is symmetric (grad W is parallel to d): its lower triangle only
-    for (int i = 0; i < 3; ++i) {
-      if (i >= dim) break;
-      const R vd = vol * d[i], vw = vol * w[i];
-      for (int j = 0; j < 3; ++j) {
-        if (j >= dim) break;
-        if (j <= i) L[i][j] -= vd * g[j];
-        G[i][j] -= vw * g[j];
+      const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+      const R rinv = rsqrt_or_zero(r2);
+      const R r = r2 * rinv;
+      const R hinv = pair_rcp(R(0.5) * (ha + hb));
+      const R q = r * hinv;
+      const R hD = hpow(hinv, dim);
+      const R fr = kern_dW(q, R(6) * sig * hD * hinv) * rinv;
+      R g[3] = {fr * d[0], fr * d[1], fr * d[2]};
+      drho.add(vol * (w[0] * g[0] + w[1] * g[1] + w[2] * g[2]));
+      // L is symmetric (grad W is parallel to d): its lower triangle only
+      for (int i = 0; i < 3; ++i) {
+        if (i >= dim) break;
+        const R vd = vol * d[i], vw = vol * w[i];
+        for (int j = 0; j < 3; ++j) {
+          if (j >= dim) break;
+          if (j <= i) L[i][j] -= vd * g[j];
+          G[i][j] -= vw * g[j];
+        }
       }
-    }
-    if (xsph) {
-      const R c = pair_div(R(2) * mb, rhoa + rhob) * kern_W(q, sig * hD);
-      for (int i = 0; i < 3; ++i) xs[i] -= c * w[i];
+      if (xsph) {
+        const R c = pair_div(R(2) * mb, rhoa + rhob) * kern_W(q, sig * hD);
+        for (int i = 0; i < 3; ++i) xs[i] -= c * w[i];
+      }
     }
   }
   // ---- per-particle update ----
@@ -557,12 +664,13 @@ __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
     for (int j = 0; j < 3; ++j) sd[i][j] = (R(1) - dd) * S[i][j];
   // principal frame of the deviatoric part (sigma_d shares its axes)
   R lam[3] = {R(0), R(0), R(0)}, Q[3][3];
-  const bool need_eig = (damage || P.eps_s > 0.0);
+  const bool as = AS && P.eps_s > 0.0;
+  const bool need_eig = damage || as;
   if (need_eig) {
     R E[3][3];
     for (int i = 0; i < 3; ++i)
       for (int j = 0; j < 3; ++j) E[i][j] = sd[i][j];
-    sym_eigen<R>(dim, E, lam, Q);
+    sym_eigen<R, AS>(dim, E, lam, Q);
     for (int i = 0; i < dim; ++i) lam[i] -= phat;
   }
   int nact = 0;
@@ -594,7 +702,7 @@ __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) Z[i][j] = R(0);
   const R rr = rhoa * rhoa;
-  if (P.eps_s > 0.0) {
+  if (as) {
     R zl[3];
     for (int k = 0; k < 3; ++k) zl[k] = (k < dim && lam[k] > R(0)) ? -(R)P.eps_s * lam[k] / rr : R(0);
     for (int i = 0; i < dim; ++i)
@@ -621,14 +729,14 @@ __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
     }
     A.Tf[a] = make_float4(t[0], t[1], t[2], t[3]);
     A.Tf[A.ld + a] = make_float4(t[4], t[5], cs, 0.f);
-    if (P.eps_s > 0.0) {
+    if (as) {
       A.Zf[a] = make_float4(z[0], z[1], z[2], z[3]);
       A.Zf[A.ld + a] = make_float4(z[4], z[5], 0.f, 0.f);
     }
   } else {
     for (int k = 0; k < ns; ++k) {
       A.Td[(int64_t)k * A.ld + a] = T[k];
-      if (P.eps_s > 0.0) A.Zd[(int64_t)k * A.ld + a] = Zc[k];
+      if (as) A.Zd[(int64_t)k * A.ld + a] = Zc[k];
     }
     A.csd[a] = cs;
   }
@@ -727,6 +835,71 @@ __device__ __forceinline__ R ipow(R f, R n) {
   return pow(f, n);
 }
 
+// Momentum and energy sums in FP64 (see pairs_A64).  The bracket T_a + T_b -
+// Pi I is applied to d, and m_b (dW/dr)/r multiplies the result.
+template <bool AS, int DIM>
+__device__ __forceinline__ void pairs_B64(const RhsArgs &A, int64_t a, const int32_t *list, int cnt,
+                                          const double Ta[6], double csa, const double Za[6], KahanT<double> acc[3],
+                                          KahanT<double> &du) {
+  constexpr int NS = DIM == 3 ? 6 : 3;
+  const sph_params &P = A.prm;
+  double xa[DIM], va[DIM];
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
+    xa[i] = A.x[i][a];
+    va[i] = A.v[i][a];
+  }
+  const double rhoa = A.rho[a], alpha = P.alpha, beta2 = 2.0 * P.beta;
+  Support64<DIM> H;
+  H.start(A.h[a]);
+  for (int k = 0; k < cnt; ++k) {
+    const int32_t b = list[(int64_t)k * A.ld];
+    double d[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0}, r2 = 0.0, vx = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      d[i] = xa[i] - A.x[i][b];
+      w[i] = va[i] - A.v[i][b];
+      r2 = fma(d[i], d[i], r2);
+      vx = fma(w[i], d[i], vx);
+    }
+    H.partner(A.h[b]);
+    const double rinv = rsqrt64(r2);
+    const double q = r2 * rinv * H.hinv;
+    const double f = slope64(q) * H.hD1 * rinv * A.m[b];  // m_b (dW/dr) / (6 sigma r)
+    double t[6];
+#pragma unroll
+    for (int c = 0; c < NS; ++c) t[c] = Ta[c] + A.Td[(int64_t)c * A.ld + b];
+    if ((int64_t)dbits(vx) < 0) {  // approaching (or -0, when Pi is 0): artificial viscosity
+      const double nu = H.hab * vx * rcp64(fma(P.eps_v * H.hab, H.hab, r2));
+      const double Pi = nu * fma(beta2, nu, -alpha * (csa + A.csd[b])) * rcp64(rhoa + A.rho[b]);
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) t[i] -= Pi;
+    }
+    double s[3];
+    sym_mv(DIM, t, d, s);
+    double ws = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) ws = fma(w[i], s[i], ws);
+    du.s = fma(f, ws, du.s);
+    if (AS) {
+      double z[6], zs[3], Zb[6];
+      load_Z<false>(A, b, NS, Zb);
+      const double fn = ipow(value64(q) * rcp64(kern_W(P.dmpd * H.hinv, 1.0)), P.n_as);
+#pragma unroll
+      for (int c = 0; c < NS; ++c) z[c] = (Za[c] + Zb[c]) * fn;
+      sym_mv(DIM, z, d, zs);
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) s[i] += zs[i];
+    }
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) acc[i].s = fma(f, s[i], acc[i].s);
+  }
+  const double norm = 6.0 * kernel_sigma<double>(DIM);
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) acc[i].s *= norm;
+  du.s *= -0.5 * norm;
+}
+
 template <bool MIXED, bool AS, int DIM>
 __global__ void SPH_PASSB_BOUNDS k_passB(RhsArgs A) {
   using R = typename std::conditional<MIXED, float, double>::type;
@@ -747,57 +920,61 @@ __global__ void SPH_PASSB_BOUNDS k_passB(RhsArgs A) {
   KahanT<R> acc[3], du;
   const int32_t *list;
   const int cnt = partner_list(A, a, list);
+  if constexpr (!MIXED) {
+    pairs_B64<AS, DIM>(A, a, list, cnt, Ta, csa, Za, acc, du);
+  } else {
 #if SPH_PASS_PREFETCH
-  PartnerCursor<MIXED> cur;
-  cur.start(A, o, list, cnt);
+    PartnerCursor<MIXED> cur;
+    cur.start(A, o, list, cnt);
 #endif
-  for (int k = 0; k < cnt; ++k) {
-    R d[3], w[3], hb, rhob, mb, vol;
-    R Tb[6], csb;
+    for (int k = 0; k < cnt; ++k) {
+      R d[3], w[3], hb, rhob, mb, vol;
+      R Tb[6], csb;
 #if SPH_PASS_PREFETCH
-    typename Own<MIXED>::Raw raw;
-    const int32_t b = cur.next(A, o, k, raw);
-    o.from(A, raw, d, w, hb, rhob, mb, vol);
-    load_T<MIXED>(A, b, ns, Tb, csb);
+      typename Own<MIXED>::Raw raw;
+      const int32_t b = cur.next(A, o, k, raw);
+      o.from(A, raw, d, w, hb, rhob, mb, vol);
+      load_T<MIXED>(A, b, ns, Tb, csb);
 #else
-    const int32_t b = list[(int64_t)k * A.ld];
-    o.pair(A, b, d, w, hb, rhob, mb, vol);
-    load_T<MIXED>(A, b, ns, Tb, csb);
+      const int32_t b = list[(int64_t)k * A.ld];
+      o.pair(A, b, d, w, hb, rhob, mb, vol);
+      load_T<MIXED>(A, b, ns, Tb, csb);
 #endif
-    const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    const R rinv = rsqrt_or_zero(r2);
-    const R r = r2 * rinv;
-    const R hab = R(0.5) * (ha + hb);
-    const R hinv = pair_rcp(hab);
-    const R q = r * hinv;
-    const R hD = hpow(hinv, dim);
-    const R fr = kern_dW(q, R(6) * sig * hD * hinv) * rinv;
-    const R g[3] = {fr * d[0], fr * d[1], fr * d[2]};
-    // artificial viscosity for approaching pairs
-    const R vx = w[0] * d[0] + w[1] * d[1] + w[2] * d[2];
-    R Pi = R(0);
-    if (vx < R(0)) {
-      const R nu = pair_div(hab * vx, r2 + epsv * hab * hab);
-      Pi = pair_div(-alpha * R(0.5) * (csa + csb) * nu + beta * nu * nu, R(0.5) * (rhoa + rhob));
+      const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+      const R rinv = rsqrt_or_zero(r2);
+      const R r = r2 * rinv;
+      const R hab = R(0.5) * (ha + hb);
+      const R hinv = pair_rcp(hab);
+      const R q = r * hinv;
+      const R hD = hpow(hinv, dim);
+      const R fr = kern_dW(q, R(6) * sig * hD * hinv) * rinv;
+      const R g[3] = {fr * d[0], fr * d[1], fr * d[2]};
+      // artificial viscosity for approaching pairs
+      const R vx = w[0] * d[0] + w[1] * d[1] + w[2] * d[2];
+      R Pi = R(0);
+      if (vx < R(0)) {
+        const R nu = pair_div(hab * vx, r2 + epsv * hab * hab);
+        Pi = pair_div(-alpha * R(0.5) * (csa + csb) * nu + beta * nu * nu, R(0.5) * (rhoa + rhob));
+      }
+      R tsum[6];
+      for (int c = 0; c < 6; ++c) tsum[c] = Ta[c] + Tb[c];
+      R tg[3];
+      sym_mv(dim, tsum, g, tg);
+      R su[3] = {tg[0] - Pi * g[0], tg[1] - Pi * g[1], tg[2] - Pi * g[2]};
+      R sv[3] = {su[0], su[1], su[2]};
+      if (AS) {
+        R Zb[6];
+        load_Z<MIXED>(A, b, ns, Zb);
+        const R fn = ipow(kern_W(q, R(1)) / kern_W(dmpd * hinv, R(1)), nas);
+        R zs[6];
+        for (int c = 0; c < 6; ++c) zs[c] = (Za[c] + Zb[c]) * fn;
+        R zg[3];
+        sym_mv(dim, zs, g, zg);
+        for (int i = 0; i < 3; ++i) sv[i] += zg[i];
+      }
+      for (int i = 0; i < dim; ++i) acc[i].add(mb * sv[i]);
+      du.add(R(-0.5) * mb * (w[0] * su[0] + w[1] * su[1] + w[2] * su[2]));
     }
-    R tsum[6];
-    for (int c = 0; c < 6; ++c) tsum[c] = Ta[c] + Tb[c];
-    R tg[3];
-    sym_mv(dim, tsum, g, tg);
-    R su[3] = {tg[0] - Pi * g[0], tg[1] - Pi * g[1], tg[2] - Pi * g[2]};
-    R sv[3] = {su[0], su[1], su[2]};
-    if (AS) {
-      R Zb[6];
-      load_Z<MIXED>(A, b, ns, Zb);
-      const R fn = ipow(kern_W(q, R(1)) / kern_W(dmpd * hinv, R(1)), nas);
-      R zs[6];
-      for (int c = 0; c < 6; ++c) zs[c] = (Za[c] + Zb[c]) * fn;
-      R zg[3];
-      sym_mv(dim, zs, g, zg);
-      for (int i = 0; i < 3; ++i) sv[i] += zg[i];
-    }
-    for (int i = 0; i < dim; ++i) acc[i].add(mb * sv[i]);
-    du.add(R(-0.5) * mb * (w[0] * su[0] + w[1] * su[1] + w[2] * su[2]));
   }
   if constexpr (MIXED) {
     const double u_acc = A.U->acc, u_du = A.U->E * A.U->invT;
@@ -833,6 +1010,7 @@ __global__ void k_repack_rho(const double *__restrict__ rho, const double *__res
   w.w = __fdiv_rn(pk.pxl(i).w, rf);
   pk.pv(i) = v;
   pk.pvl(i) = w;
+  if (pk.vol) pk.vol[i] = m[i] / rho[i];
 }
 
 void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &p, const sph_derivs &out,
@@ -886,7 +1064,10 @@ void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &
   A.err = c->d_err;
   const bool mixed = p.precision == SPH_MIXED;
   A.sums = mixed ? sums : nullptr;
-  const int T = c->tune.pass_threads;
+  // FP64 passes are bound by each SM's FP64 unit, so what counts for a small n
+  // is that the warps spread evenly over the SMs: one-warp blocks while that
+  // leaves fewer than eight 128-thread blocks per SM.
+  const int T = !mixed && nblk(n, 128) < 8 * c->num_sms ? 32 : c->tune.pass_threads;
   int pr = -1;
   const bool d3 = s->dim == 3;
 #define SPH_LAUNCH(kern, ...)                                                     \
@@ -903,17 +1084,18 @@ void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &
     prof_end(c, st, pr);
   }
   pr = prof_begin(c, st, PH_PASSA);
-  if (mixed && A.sums) {
-    if (d3) k_passA<true, 3, true><<<nblk(n, T), T, 0, st>>>(A);
-    else k_passA<true, 2, true><<<nblk(n, T), T, 0, st>>>(A);
+  const bool as = p.eps_s > 0.0;
+  if (mixed && A.sums) {  // the adjoint's forward
+    if (d3) k_passA<true, true, 3, true><<<nblk(n, T), T, 0, st>>>(A);
+    else k_passA<true, true, 2, true><<<nblk(n, T), T, 0, st>>>(A);
     ++sph::g_launches;
   } else if (mixed) {
-    SPH_LAUNCH(k_passA, true);
+    SPH_LAUNCH(k_passA, true, true);
   } else {
-    SPH_LAUNCH(k_passA, false);
+    if (as) SPH_LAUNCH(k_passA, false, true);
+    else SPH_LAUNCH(k_passA, false, false);
   }
   prof_end(c, st, pr);
-  const bool as = p.eps_s > 0.0;
   pr = prof_begin(c, st, PH_PASSB);
   if (mixed) {
     if (as) SPH_LAUNCH(k_passB, true, true);

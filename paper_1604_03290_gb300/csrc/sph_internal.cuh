@@ -53,6 +53,7 @@ constexpr int kMaxShell = 24;
 // (more lines, i.e. L1 wavefronts, per gather instruction).
 struct PackedF32 {
   float4 *px_, *pxl_, *pv_, *pvl_;
+  double *vol;  // FP64 calls: m / rho, written with the views (NULL otherwise)
   __host__ __device__ float4 &px(int64_t i) const { return px_[i]; }    // (x_hi, y_hi, z_hi, h)
   __host__ __device__ float4 &pxl(int64_t i) const { return pxl_[i]; }  // (x_lo, y_lo, z_lo, m)
   __host__ __device__ float4 &pv(int64_t i) const { return pv_[i]; }    // (vx_hi, vy_hi, vz_hi, rho)
@@ -196,6 +197,7 @@ struct sph_ctx {
   int64_t *csr_total;   // device scalar for sph_neighbours
   int32_t *hflags;      // variable-h iteration: done, updates, off-target count per pass
   // pass A -> pass B per-particle data
+  double *vol;          // volumes m / rho of FP64 calls (pk.vol points here then)
   void *T;              // nsym * cap_n of double (FP64) or float (mixed)
   void *zeta;
   double *cs;

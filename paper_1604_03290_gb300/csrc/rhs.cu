@@ -59,6 +59,7 @@ struct RhsArgs {
   double *rho_out;          // density-sum output
   const Units *U;           // code units of the FP32 views (mixed mode)
   float *sums;              // mixed, KEEP_SUMS: pass A's pair sums (16 rows of stride ld)
+  int lane_shift;           // FP64: 2^lane_shift lanes share a particle's partner list
   MatTable mt;
   sph_params prm;
   int32_t *err;
@@ -79,6 +80,10 @@ __device__ __forceinline__ float rsqrt_or_zero(float r2) { return r2 > 0.f ? rsq
 #else
 #define SPH_PASSB_BOUNDS __launch_bounds__(128)
 #endif
+
+// FP64 passes: the warps per SM below which several lanes share a particle's
+// list (see rhs_passes).
+constexpr int kLaneWarps = 4;
 
 // 1 / x, correctly rounded: the same value as the division
 template <class R>
@@ -270,6 +275,63 @@ struct Support64 {
   }
 };
 
+// The lanes that share one particle's list: lane `sub` of n takes partners
+// sub, sub + n, ...  Sums are combined over the group in a fixed order.
+struct Lanes64 {
+  int sub, n;
+  unsigned mask;
+  __device__ __forceinline__ Lanes64(int shift) {
+    n = 1 << shift;
+    const int lane = threadIdx.x & 31;
+    sub = lane & (n - 1);
+    mask = (n == 32 ? ~0u : (1u << n) - 1u) << (lane - sub);
+  }
+  __device__ __forceinline__ double sum(double v) const {
+    for (int o = 1; o < n; o <<= 1) v += __shfl_xor_sync(mask, v, o);
+    return v;
+  }
+};
+
+// A partner's data (m: the array given, V_b or m_b), read one pair ahead, and
+// its index two ahead, as the mixed passes do
+template <int DIM>
+struct Partner64 {
+  double x[DIM], v[DIM], h, m;
+};
+template <int DIM>
+struct Cursor64 {
+  const int32_t *col;
+  int cnt, step;
+  int32_t b1, b2;
+  Partner64<DIM> p1;
+  __device__ __forceinline__ void fetch(const RhsArgs &A, const double *m, int32_t b) {
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      p1.x[i] = A.x[i][b];
+      p1.v[i] = A.v[i][b];
+    }
+    p1.h = A.h[b];
+    p1.m = m[b];
+  }
+  __device__ __forceinline__ void start(const RhsArgs &A, const double *m, const int32_t *list, int n,
+                                        const Lanes64 &ln) {
+    col = list;
+    cnt = n;
+    step = ln.n;
+    b1 = ln.sub < cnt ? col[(int64_t)ln.sub * A.ld] : 0;
+    b2 = ln.sub + step < cnt ? col[(int64_t)(ln.sub + step) * A.ld] : 0;
+    if (ln.sub < cnt) fetch(A, m, b1);
+  }
+  __device__ __forceinline__ int32_t next(const RhsArgs &A, const double *m, int k, Partner64<DIM> &p) {
+    const int32_t b = b1;
+    p = p1;
+    b1 = b2;
+    if (k + 2 * step < cnt) b2 = col[(int64_t)(k + 2 * step) * A.ld];
+    if (k + step < cnt) fetch(A, m, b1);
+    return b;
+  }
+};
+
 // q < 1/2 for q >= 0, from the bits
 __device__ __forceinline__ bool below_half(double q) { return __double2hiint(q) < 0x3fe00000; }
 
@@ -291,7 +353,7 @@ __device__ __forceinline__ double value64(double q) {
 template <bool MIXED, int DIM>
 __global__ void __launch_bounds__(128) k_density_sum(RhsArgs A) {
   using R = typename std::conditional<MIXED, float, double>::type;
-  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t a = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> (MIXED ? 0 : A.lane_shift);
   if (a >= A.n) return;
   Own<MIXED> o;
   o.load(A, a);
@@ -305,10 +367,11 @@ __global__ void __launch_bounds__(128) k_density_sum(RhsArgs A) {
   const int32_t *list;
   const int cnt = partner_list(A, a, list);
   if constexpr (!MIXED) {
+    const Lanes64 ln(A.lane_shift);
     Support64<DIM> H;
     H.start(o.h);
     double w = 0.0;
-    for (int k = 0; k < cnt; ++k) {
+    for (int k = ln.sub; k < cnt; k += ln.n) {
       const int32_t b = list[(int64_t)k * A.ld];
       double r2 = 0.0;
 #pragma unroll
@@ -319,7 +382,8 @@ __global__ void __launch_bounds__(128) k_density_sum(RhsArgs A) {
       H.partner(A.h[b]);
       w = fma(A.m[b] * H.hD, value64(r2 * rsqrt64(r2) * H.hinv), w);
     }
-    sum.add(sig * w);
+    sum.add(sig * ln.sum(w));
+    if (ln.sub) return;
   } else {
     for (int k = 0; k < cnt; ++k) {
       const int32_t b = list[(int64_t)k * A.ld];
@@ -450,8 +514,8 @@ __device__ __forceinline__ void sym_eigen(int dim, R A[3][3], R w[3], R V[3][3])
 }
 
 template <int DIM>
-__device__ __forceinline__ void pairs_A64(const RhsArgs &A, int64_t a, const int32_t *list, int cnt, bool xsph,
-                                          double L[3][3], double G[3][3], double xs[3]) {
+__device__ __forceinline__ void pairs_A64(const RhsArgs &A, int64_t a, const Lanes64 &ln, const int32_t *list, int cnt,
+                                          bool xsph, double L[3][3], double G[3][3], double xs[3]) {
   double xa[DIM], va[DIM];
 #pragma unroll
   for (int i = 0; i < DIM; ++i) {
@@ -461,19 +525,22 @@ __device__ __forceinline__ void pairs_A64(const RhsArgs &A, int64_t a, const int
   const double rhoa = A.rho[a];
   Support64<DIM> H;
   H.start(A.h[a]);
-  for (int k = 0; k < cnt; ++k) {
-    const int32_t b = list[(int64_t)k * A.ld];
+  Cursor64<DIM> cur;
+  cur.start(A, A.pk.vol, list, cnt, ln);
+  for (int k = ln.sub; k < cnt; k += ln.n) {
+    Partner64<DIM> B;
+    const int32_t b = cur.next(A, A.pk.vol, k, B);
     double d[DIM], w[DIM], gd[DIM], r2 = 0.0;
 #pragma unroll
     for (int i = 0; i < DIM; ++i) {
-      d[i] = xa[i] - A.x[i][b];
-      w[i] = va[i] - A.v[i][b];
+      d[i] = xa[i] - B.x[i];
+      w[i] = va[i] - B.v[i];
       r2 = fma(d[i], d[i], r2);
     }
-    H.partner(A.h[b]);
+    H.partner(B.h);
     const double rinv = rsqrt64(r2);
     const double q = r2 * rinv * H.hinv;
-    const double f = slope64(q) * H.hD1 * rinv * A.pk.vol[b];  // V_b (dW/dr) / (6 sigma r)
+    const double f = slope64(q) * H.hD1 * rinv * B.m;  // V_b (dW/dr) / (6 sigma r)
 #pragma unroll
     for (int i = 0; i < DIM; ++i) gd[i] = f * d[i];
 #pragma unroll
@@ -492,11 +559,11 @@ __device__ __forceinline__ void pairs_A64(const RhsArgs &A, int64_t a, const int
   const double sig = kernel_sigma<double>(DIM);
 #pragma unroll
   for (int i = 0; i < DIM; ++i) {
-    xs[i] *= 2.0 * sig;
+    if (xsph) xs[i] = 2.0 * sig * ln.sum(xs[i]);
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
-      L[i][j] *= 6.0 * sig;
-      G[i][j] *= 6.0 * sig;
+      if (j <= i) L[i][j] = 6.0 * sig * ln.sum(L[i][j]);
+      G[i][j] = 6.0 * sig * ln.sum(G[i][j]);
     }
   }
 }
@@ -516,7 +583,7 @@ __device__ __forceinline__ void pairs_A64(const RhsArgs &A, int64_t a, const int
 template <bool MIXED, bool AS, int DIM, bool KEEP_SUMS = false>
 __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
   using R = typename std::conditional<MIXED, float, double>::type;
-  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t a = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> (MIXED ? 0 : A.lane_shift);
   if (a >= A.n) return;
   constexpr int dim = DIM;
   const sph_params &P = A.prm;
@@ -532,7 +599,9 @@ __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
   const int32_t *list;
   const int cnt = partner_list(A, a, list);
   if constexpr (!MIXED) {
-    pairs_A64<DIM>(A, a, list, cnt, xsph, L, G, xs);
+    const Lanes64 ln(A.lane_shift);
+    pairs_A64<DIM>(A, a, ln, list, cnt, xsph, L, G, xs);
+    if (ln.sub) return;
     double tr = 0.0;  // sum_b V_b (v_a - v_b).grad W = -tr G
     for (int i = 0; i < dim; ++i) tr += G[i][i];
     drho.add(-tr);
@@ -838,7 +907,7 @@ __device__ __forceinline__ R ipow(R f, R n) {
 // Momentum and energy sums in FP64 (see pairs_A64).  The bracket T_a + T_b -
 // Pi I is applied to d, and m_b (dW/dr)/r multiplies the result.
 template <bool AS, int DIM>
-__device__ __forceinline__ void pairs_B64(const RhsArgs &A, int64_t a, const int32_t *list, int cnt,
+__device__ __forceinline__ void pairs_B64(const RhsArgs &A, int64_t a, const Lanes64 &ln, const int32_t *list, int cnt,
                                           const double Ta[6], double csa, const double Za[6], KahanT<double> acc[3],
                                           KahanT<double> &du) {
   constexpr int NS = DIM == 3 ? 6 : 3;
@@ -852,23 +921,26 @@ __device__ __forceinline__ void pairs_B64(const RhsArgs &A, int64_t a, const int
   const double rhoa = A.rho[a], alpha = P.alpha, beta2 = 2.0 * P.beta;
   Support64<DIM> H;
   H.start(A.h[a]);
-  for (int k = 0; k < cnt; ++k) {
-    const int32_t b = list[(int64_t)k * A.ld];
-    double d[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0}, r2 = 0.0, vx = 0.0;
-#pragma unroll
-    for (int i = 0; i < DIM; ++i) {
-      d[i] = xa[i] - A.x[i][b];
-      w[i] = va[i] - A.v[i][b];
-      r2 = fma(d[i], d[i], r2);
-      vx = fma(w[i], d[i], vx);
-    }
-    H.partner(A.h[b]);
-    const double rinv = rsqrt64(r2);
-    const double q = r2 * rinv * H.hinv;
-    const double f = slope64(q) * H.hD1 * rinv * A.m[b];  // m_b (dW/dr) / (6 sigma r)
+  Cursor64<DIM> cur;
+  cur.start(A, A.m, list, cnt, ln);
+  for (int k = ln.sub; k < cnt; k += ln.n) {
+    Partner64<DIM> B;
+    const int32_t b = cur.next(A, A.m, k, B);
     double t[6];
 #pragma unroll
     for (int c = 0; c < NS; ++c) t[c] = Ta[c] + A.Td[(int64_t)c * A.ld + b];
+    double d[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0}, r2 = 0.0, vx = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      d[i] = xa[i] - B.x[i];
+      w[i] = va[i] - B.v[i];
+      r2 = fma(d[i], d[i], r2);
+      vx = fma(w[i], d[i], vx);
+    }
+    H.partner(B.h);
+    const double rinv = rsqrt64(r2);
+    const double q = r2 * rinv * H.hinv;
+    const double f = slope64(q) * H.hD1 * rinv * B.m;  // m_b (dW/dr) / (6 sigma r)
     if ((int64_t)dbits(vx) < 0) {  // approaching (or -0, when Pi is 0): artificial viscosity
       const double nu = H.hab * vx * rcp64(fma(P.eps_v * H.hab, H.hab, r2));
       const double Pi = nu * fma(beta2, nu, -alpha * (csa + A.csd[b])) * rcp64(rhoa + A.rho[b]);
@@ -896,14 +968,14 @@ __device__ __forceinline__ void pairs_B64(const RhsArgs &A, int64_t a, const int
   }
   const double norm = 6.0 * kernel_sigma<double>(DIM);
 #pragma unroll
-  for (int i = 0; i < DIM; ++i) acc[i].s *= norm;
-  du.s *= -0.5 * norm;
+  for (int i = 0; i < DIM; ++i) acc[i].s = norm * ln.sum(acc[i].s);
+  du.s = -0.5 * norm * ln.sum(du.s);
 }
 
 template <bool MIXED, bool AS, int DIM>
 __global__ void SPH_PASSB_BOUNDS k_passB(RhsArgs A) {
   using R = typename std::conditional<MIXED, float, double>::type;
-  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t a = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> (MIXED ? 0 : A.lane_shift);
   if (a >= A.n) return;
   constexpr int dim = DIM;
   const int ns = nsym(dim);
@@ -921,7 +993,9 @@ __global__ void SPH_PASSB_BOUNDS k_passB(RhsArgs A) {
   const int32_t *list;
   const int cnt = partner_list(A, a, list);
   if constexpr (!MIXED) {
-    pairs_B64<AS, DIM>(A, a, list, cnt, Ta, csa, Za, acc, du);
+    const Lanes64 ln(A.lane_shift);
+    pairs_B64<AS, DIM>(A, a, ln, list, cnt, Ta, csa, Za, acc, du);
+    if (ln.sub) return;
   } else {
 #if SPH_PASS_PREFETCH
     PartnerCursor<MIXED> cur;
@@ -1068,12 +1142,20 @@ void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &
   // is that the warps spread evenly over the SMs: one-warp blocks while that
   // leaves fewer than eight 128-thread blocks per SM.
   const int T = !mixed && nblk(n, 128) < 8 * c->num_sms ? 32 : c->tune.pass_threads;
+  // With fewer than kLaneWarps warps per SM even that leaves the unit idle
+  // between dependent operations: 2, 4 or 8 lanes then share a particle's
+  // list, and the constitutive update is repeated on each.  Against one lane,
+  // at thresholds of 2, 4 and 8 warps: rings at 4.4k (ten steps) 6.90 -> 5.67,
+  // 5.79, 5.80 ms; a right-hand side at 8k 902 -> 815, 804, 920 us and at 27k
+  // 1078 -> 1080, 1078, 1125 us; RK3 at 14k 3.18 -> 3.18, 2.96, 3.25 ms.
+  while (!mixed && A.lane_shift < 3 && (n << A.lane_shift) < (int64_t)32 * kLaneWarps * c->num_sms) ++A.lane_shift;
+  const int64_t nt = n << A.lane_shift;  // threads of a pass
   int pr = -1;
   const bool d3 = s->dim == 3;
 #define SPH_LAUNCH(kern, ...)                                                     \
   do {                                                                            \
-    if (d3) kern<__VA_ARGS__, 3><<<nblk(n, T), T, 0, st>>>(A);                   \
-    else kern<__VA_ARGS__, 2><<<nblk(n, T), T, 0, st>>>(A);                      \
+    if (d3) kern<__VA_ARGS__, 3><<<nblk(nt, T), T, 0, st>>>(A);                  \
+    else kern<__VA_ARGS__, 2><<<nblk(nt, T), T, 0, st>>>(A);                     \
     ++sph::g_launches;                                                            \
   } while (0)
   if (p.density_sum) {

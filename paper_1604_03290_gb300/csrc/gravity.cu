@@ -23,8 +23,7 @@
 // acceptance test in FP32 with a relative band of 1e-4 around the threshold
 // inside which the FP64 expression decides, FP32 monopole terms summed with
 // Kahan compensation.
-#include <type_traits>
-
+#include "fp64fast.cuh"
 #include "morton.cuh"
 #include "sph_internal.cuh"
 
@@ -41,6 +40,8 @@ constexpr int kGrWarps = SPH_GRAV_WARPS;  // warps (particle groups) per block
 #ifndef SPH_GRAV_MIN_BLOCKS
 #define SPH_GRAV_MIN_BLOCKS 32
 #endif
+// FP64 walk: resident one-warp blocks per SM (80 registers, 8 KB of lists each)
+constexpr int kGrav64Blocks = 24;
 constexpr float kMacBand = 1e-4f;
 constexpr int kFlushTerms = 16;
 // A leaf summed directly by few lanes: rather than each of them looping over
@@ -80,27 +81,12 @@ struct GravSumF {
   }
 };
 
-struct GravSumD {
-  double sx = 0.0, sy = 0.0, sz = 0.0;
-  __device__ __forceinline__ void add(double fx, double fy, double fz) {
-    sx += fx;
-    sy += fy;
-    sz += fz;
-  }
-  __device__ __forceinline__ void value(double &x, double &y, double &z) {
-    x = sx;
-    y = sy;
-    z = sz;
-  }
-};
-
-// 1 / q^(3/2): from the reciprocal square root in FP32 (a few ulps, far below
-// the mixed form's tolerance), correctly rounded operations in FP64
+// 1 / q^(3/2) from the reciprocal square root in FP32 (a few ulps, far below
+// the mixed form's tolerance)
 __device__ __forceinline__ float inv_q32(float q) {
   const float r = rsqrtf(q);
   return r * r * r;
 }
-__device__ __forceinline__ double inv_q32(double q) { return 1.0 / (q * sqrt(q)); }
 
 struct GravArgs {
   Tree T;
@@ -111,6 +97,7 @@ struct GravArgs {
   double *out[3];
   const Units *U;
   int32_t *err;
+  int share;  // FP64: 2^share lanes per particle
   int reuse;  // the tree was built at earlier positions: locate each particle anew
   unsigned long long *ctr;  // NULL, or the interaction counters
 };
@@ -127,15 +114,14 @@ __device__ __forceinline__ double r2_fp64(const double xa[3], double cx, double 
   return r2;
 }
 
-// PACKED (mixed, Tree::packed_walk): a node's skip, level and leaf flag come
-// from the w word of its second COM view, so that a visit loads two float4
+// Mixed precision.  PACKED (Tree::packed_walk): a node's skip, level and leaf
+// flag come from the w word of its second COM view, so that a visit loads two float4
 // (the node's member range only when some lane sums it directly), and the
 // node edge s0 / 2^level is the instance's FP32 edge shifted by the level:
 // the same value k_node_finish stores otherwise.
-template <bool MIXED, int DIM, bool PACKED>
+template <int DIM, bool PACKED>
 __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(GravArgs A) {
-  static_assert(MIXED || !PACKED, "the packed word is read by the mixed walk");
-  using R = typename std::conditional<MIXED, float, double>::type;
+  using R = float;
   __shared__ float4 sh_hi[kGrWarps][kMaxLeaf];  // (x_hi, y_hi, z_hi, G m_b) of leaf members
   __shared__ float4 sh_lo[kGrWarps][kMaxLeaf];
   __shared__ int32_t sh_b[kGrWarps][kMaxLeaf];
@@ -151,7 +137,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
   const int L = T.leaf_size, B = T.max_depth;
   const int nnodes = T.iter_cap > 0 ? min(*T.nnodes, T.iter_cap) : *T.nnodes;
   const int64_t cap = T.cap_nodes;
-  const double Gs = MIXED ? A.G * A.U->M * A.U->T * A.U->T * A.U->invL * A.U->invL * A.U->invL : A.G;
+  const double Gs = A.G * A.U->M * A.U->T * A.U->T * A.U->invL * A.U->invL * A.U->invL;
   const R G = (R)Gs;
   for (int g = blockIdx.x * kGrWarps + w; g < ngroups; g += gridDim.x * kGrWarps) {
     const int32_t s0 = chunks ? g * 32 : T.grp_start[g];
@@ -168,7 +154,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
         !act ? 0ULL
              : (A.reuse ? morton_key(xa, dim, B, inst, T.inst_lo, T.inst_s0[inst], T.inst_rs0[inst]) : T.skey[slot]);
     const float4 Pa = A.pk.px(a), Qa = A.pk.pxl(a);
-    const double e = MIXED ? A.eps * (double)Pa.w : A.eps * A.h[a];
+    const double e = A.eps * (double)Pa.w;
     const R eps2 = (R)(e * e);
     const double s0r = T.inst_s0[inst];
     // the instance's root edge in FP32 code units (PACKED: shifted by the level per node)
@@ -180,7 +166,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
     // rounding of either test) the opening criterion already rejects it and
     // the containment test can be skipped: the accepted set is the same.
     const bool test_inside = (double)dim * th * th >= 0.99;
-    typename std::conditional<MIXED, GravSumF, GravSumD>::type acc;
+    GravSumF acc;
     int32_t skip_until = -1;
     const int32_t root = T.inst_root[inst];
     const int32_t stop = root >= 0 ? T.skip[root] : root;
@@ -213,38 +199,28 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
         float mpf = 0.f;
         R d[3] = {R(0), R(0), R(0)}, r2 = R(0);
         if (!inside) {
-          if constexpr (MIXED) {
-            if constexpr (!PACKED) {
-              ch = T.fcom_hi[nd];
-              cl = T.fcom_lo[nd];
-            }
-            d[0] = (Pa.x - ch.x) + (Qa.x - cl.x);
-            d[1] = (Pa.y - ch.y) + (Qa.y - cl.y);
-            d[2] = (Pa.z - ch.z) + (Qa.z - cl.z);
-            r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-            mpf = ch.w;
-            const float sf = PACKED ? __int_as_float(__float_as_int(s0f) - (lev << 23)) : cl.w;
-            const float lhs = sf * sf, rhs = th2f * r2;
-            if (lhs < rhs * (1.0f - kMacBand)) accept = true;
-            else if (lhs > rhs * (1.0f + kMacBand)) accept = false;
-            else {
-              // rare: the FP64 decision, from values reloaded here rather than kept live in the loop
-              const double xr[3] = {A.x[0][a], A.x[1][a], DIM == 3 ? A.x[2][a] : 0.0};
-              accept = ldexp(T.inst_s0[inst], -lev) <
-                       A.theta * sqrt(r2_fp64<DIM>(xr, T.com[nd], T.com[cap + nd], DIM == 3 ? T.com[2 * cap + nd] : 0.0));
-            }
-          } else {
-            const double s = ldexp(s0r, -lev);
-            const double cx = T.com[nd], cy = T.com[cap + nd], cz = DIM == 3 ? T.com[2 * cap + nd] : 0.0;
-            d[0] = xa[0] - cx;
-            d[1] = xa[1] - cy;
-            d[2] = DIM == 3 ? xa[2] - cz : 0.0;
-            r2 = r2_fp64<DIM>(xa, cx, cy, cz);
-            accept = s < th * sqrt(r2);
+          if constexpr (!PACKED) {
+            ch = T.fcom_hi[nd];
+            cl = T.fcom_lo[nd];
+          }
+          d[0] = (Pa.x - ch.x) + (Qa.x - cl.x);
+          d[1] = (Pa.y - ch.y) + (Qa.y - cl.y);
+          d[2] = (Pa.z - ch.z) + (Qa.z - cl.z);
+          r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+          mpf = ch.w;
+          const float sf = PACKED ? __int_as_float(__float_as_int(s0f) - (lev << 23)) : cl.w;
+          const float lhs = sf * sf, rhs = th2f * r2;
+          if (lhs < rhs * (1.0f - kMacBand)) accept = true;
+          else if (lhs > rhs * (1.0f + kMacBand)) accept = false;
+          else {
+            // rare: the FP64 decision, from values reloaded here rather than kept live in the loop
+            const double xr[3] = {A.x[0][a], A.x[1][a], DIM == 3 ? A.x[2][a] : 0.0};
+            accept = ldexp(T.inst_s0[inst], -lev) <
+                     A.theta * sqrt(r2_fp64<DIM>(xr, T.com[nd], T.com[cap + nd], DIM == 3 ? T.com[2 * cap + nd] : 0.0));
           }
         }
         if (accept) {
-          const R mp = MIXED ? (R)mpf : (R)T.mass[nd];
+          const R mp = mpf;
           const R gq = -G * mp * inv_q32(r2 + eps2);
           acc.add(gq * d[0], gq * d[1], dim == 3 ? gq * d[2] : R(0));
           skip_until = sk;
@@ -277,8 +253,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
             sh_b[w][lane] = bm;
           }
           __syncwarp();
-          bool transposed = false;
-          if constexpr (MIXED) transposed = __popc(dmask) * kTransposedCost < c * kSerialCost;
+          const bool transposed = __popc(dmask) * kTransposedCost < c * kSerialCost;
           if (transposed) {
             const float gmk = -(float)G * qb.w;
             unsigned mm = dmask;
@@ -322,16 +297,11 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
               const int32_t b = sh_b[w][k];
               if (b == a) continue;
               R d[3], gm;  // gm = -G m_b
-              if constexpr (MIXED) {
-                const float4 ph = sh_hi[w][k], pl = sh_lo[w][k];
-                d[0] = (Pa.x - ph.x) + (Qa.x - pl.x);
-                d[1] = (Pa.y - ph.y) + (Qa.y - pl.y);
-                d[2] = (Pa.z - ph.z) + (Qa.z - pl.z);
-                gm = ph.w;
-              } else {
-                for (int ax = 0; ax < 3; ++ax) d[ax] = ax < dim ? xa[ax] - A.x[ax][b] : 0.0;
-                gm = -G * A.m[b];
-              }
+              const float4 ph = sh_hi[w][k], pl = sh_lo[w][k];
+              d[0] = (Pa.x - ph.x) + (Qa.x - pl.x);
+              d[1] = (Pa.y - ph.y) + (Qa.y - pl.y);
+              d[2] = (Pa.z - ph.z) + (Qa.z - pl.z);
+              gm = ph.w;
               const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
               const R q = r2 + eps2;
               if (!(q > R(0))) continue;
@@ -354,10 +324,158 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
     if (act) {
       double gx, gy, gz;
       acc.value(gx, gy, gz);
-      const double osc = MIXED ? A.U->acc : 1.0;
+      const double osc = A.U->acc;
       A.out[0][a] = gx * osc;
       A.out[1][a] = gy * osc;
       if (DIM == 3) A.out[2][a] = gz * osc;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 walk.  Bound by the FP64 unit (a warp instruction every 16 cycles per
+// SM), so the walk itself spends none of it and the terms run on full warps:
+//  - acceptance as in the mixed walk, in FP32 with the FP64 expression inside
+//    a band of 1e-4 (far above the FP32 error): the same accepted set;
+//  - a lane appends what it accepts (nodes) and what it sums directly (leaf
+//    members) to its own list in shared memory; when a list may overflow the
+//    warp evaluates all lists in lockstep.  Evaluated where they are met, a
+//    term would occupy the unit for the 18 of 32 lanes that accept the node;
+//  - a term takes 17 FP64 instructions, with rsqrt64 in place of a square root
+//    and a division, and G applied to the sums.
+// A lane's terms are summed in the order of its own walk, whatever the warp.
+// 50k cloud, the whole call: 9.05 -> 3.14 ms (before: acceptance and terms in FP64
+// at the node, about 45 instructions each).
+// ---------------------------------------------------------------------------
+constexpr int kList64 = 64;  // entries per lane: a leaf's 32 members fit while 32 wait
+
+template <int DIM>
+__global__ void __launch_bounds__(32, kGrav64Blocks) k_gravity64(GravArgs A) {
+  __shared__ int32_t list[kList64][32];  // node id, or ~particle
+  const Tree &T = A.T;
+  const int lane = threadIdx.x & 31;
+  // lane `sub` of the 2^share lanes of a particle takes its terms sub, sub + 2^share, ...
+  const int share = A.share, sub = lane & ((1 << share) - 1), every = (1 << share) - 1;
+  const bool chunks = T.ninst <= 1;
+  const int per = 32 >> share;  // particles of a chunk
+  const int ngroups = chunks ? (int)((T.n + per - 1) / per) : *T.ngroups;
+  const int L = T.leaf_size, B = T.max_depth;
+  const int nnodes = T.iter_cap > 0 ? min(*T.nnodes, T.iter_cap) : *T.nnodes;
+  const int64_t cap = T.cap_nodes;
+  const double th = A.theta;
+  const float th2f = (float)(th * th);
+  const bool test_inside = (double)DIM * th * th >= 0.99;  // see k_gravity
+  for (int g = blockIdx.x; g < ngroups; g += gridDim.x) {
+    const int32_t s0 = chunks ? g * per : T.grp_start[g];
+    const int32_t s1 = chunks ? (int32_t)(((int64_t)s0 + per < T.n) ? (int64_t)s0 + per : T.n) : T.grp_end[g];
+    const int inst = chunks ? 0 : T.grp_inst[g];
+    const int32_t slot = s0 + (lane >> share);
+    const bool act = slot < s1;
+    const int32_t a = act ? (T.perm_identity ? slot : T.perm[slot]) : 0;
+    double xa[3] = {0.0, 0.0, 0.0}, acc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int ax = 0; ax < DIM; ++ax) xa[ax] = A.x[ax][a];
+    const unsigned long long ka =
+        !act || !test_inside
+            ? 0ULL
+            : (A.reuse ? morton_key(xa, DIM, B, inst, T.inst_lo, T.inst_s0[inst], T.inst_rs0[inst]) : T.skey[slot]);
+    const float4 Pa = A.pk.px(a), Qa = A.pk.pxl(a);
+    const double e = A.eps * A.h[a], eps2 = e * e;
+    const float s0f = to_f32_scaled(T.inst_s0[inst], pow2_exp(A.U->invL), A.U->invL);
+    const int32_t root = T.inst_root[inst];
+    const int32_t stop = root >= 0 ? T.skip[root] : root;
+    int32_t skip_until = -1;
+    int len = 0, iter = 0, met = 0;  // met: terms of this particle, on all its lanes
+    unsigned nacc = 0, nterm = 0;
+    auto evaluate = [&]() {
+      double p[DIM], m = 0.0;
+      int32_t ent = 0;
+      auto fetch = [&](int k) {
+        ent = list[k][lane];
+        const bool part = ent < 0;
+        const int64_t i = part ? ~ent : ent;
+#pragma unroll
+        for (int ax = 0; ax < DIM; ++ax) p[ax] = part ? A.x[ax][i] : T.com[ax * cap + i];
+        m = part ? A.m[i] : T.mass[i];
+      };
+      if (len > 0) fetch(0);
+      for (int k = 0; k < len; ++k) {
+        double d[DIM], q = eps2;
+        const double mk = m;
+#pragma unroll
+        for (int ax = 0; ax < DIM; ++ax) {
+          d[ax] = xa[ax] - p[ax];
+          q = fma(d[ax], d[ax], q);
+        }
+        nterm += (unsigned)(ent < 0 && (int64_t)dbits(q) > 0);
+        if (k + 1 < len) fetch(k + 1);
+        const double y = rsqrt64(q);  // 0 where q = 0
+        const double f = mk * y * (y * y);
+#pragma unroll
+        for (int ax = 0; ax < DIM; ++ax) acc[ax] = fma(f, d[ax], acc[ax]);
+      }
+      len = 0;
+      __syncwarp();
+    };
+    for (int32_t nd = root; nd < stop && iter <= nnodes; ++iter) {
+      const int4 rec = __ldg(&T.nrec[nd]);  // (first, end, skip, level)
+      const float4 ch = __ldg(&T.fcom_hi[nd]), cl = __ldg(&T.fcom_lo[nd]);
+      const bool leaf = rec.y - rec.x <= L || rec.w == B;
+      bool open = false, direct = false;
+      if (act && nd >= skip_until) {
+        bool accept = false;
+        if (!(test_inside && (ka >> (DIM * (B - rec.w))) == T.cell[nd])) {
+          const float dx = (Pa.x - ch.x) + (Qa.x - cl.x), dy = (Pa.y - ch.y) + (Qa.y - cl.y),
+                      dz = (Pa.z - ch.z) + (Qa.z - cl.z);
+          const float sf = __int_as_float(__float_as_int(s0f) - (rec.w << 23));
+          const float lhs = sf * sf, rhs = th2f * (dx * dx + dy * dy + dz * dz);
+          if (lhs < rhs * (1.0f - kMacBand) && rhs < 1e37f && lhs > 1e-30f) accept = true;
+          else if (lhs > rhs * (1.0f + kMacBand) && lhs < 1e37f && lhs > 1e-30f) accept = false;
+          else  // rare: the FP64 decision
+            accept = ldexp(T.inst_s0[inst], -rec.w) <
+                     th * sqrt(r2_fp64<DIM>(xa, T.com[nd], T.com[cap + nd], DIM == 3 ? T.com[2 * cap + nd] : 0.0));
+        }
+        if (accept) {
+          if ((met++ & every) == sub) {
+            list[len++][lane] = nd;
+            ++nacc;
+          }
+          skip_until = rec.z;
+        } else if (leaf) {
+          direct = true;
+          skip_until = rec.z;
+        } else {
+          open = true;
+        }
+      }
+      const bool any_open = __any_sync(0xffffffffu, open);
+      if (__any_sync(0xffffffffu, direct)) {
+        for (int32_t base = rec.x; base < rec.y; base += kMaxLeaf) {
+          const int c = min(rec.y - base, kMaxLeaf);
+          if (__any_sync(0xffffffffu, len > kList64 - kMaxLeaf)) evaluate();
+          const int32_t bm = lane < c ? (T.perm_identity ? base + lane : T.perm[base + lane]) : -1;
+          for (int k = 0; k < c; ++k) {
+            const int32_t b = __shfl_sync(0xffffffffu, bm, k);
+            if (direct && b != a && (met++ & every) == sub) list[len++][lane] = ~b;
+          }
+        }
+      }
+      if (__any_sync(0xffffffffu, len == kList64)) evaluate();
+      nd = any_open ? nd + 1 : rec.z;
+    }
+    evaluate();
+    if (iter > nnodes) raise_err(A.err, ERR_TIMEOUT);
+    if (A.ctr) {
+      warp_count(A.ctr + CTR_GRAV_NODES, nacc);
+      warp_count(A.ctr + CTR_GRAV_TERMS, nterm);
+      if (lane == 0) atomicAdd(A.ctr + CTR_GRAV_VISITS, (unsigned long long)iter);
+    }
+    for (int o = 1; o <= every; o <<= 1)
+#pragma unroll
+      for (int ax = 0; ax < DIM; ++ax) acc[ax] += __shfl_xor_sync(0xffffffffu, acc[ax], o);
+    if (act && sub == 0) {
+#pragma unroll
+      for (int ax = 0; ax < DIM; ++ax) A.out[ax][a] = -A.G * acc[ax];
     }
   }
 }
@@ -385,16 +503,26 @@ void gravity_walk(sph_ctx *c, const sph_state *s, const sph_params &p, double *a
   A.ctr = counters(c);
   int blocks = c->num_sms * SPH_GRAV_MIN_BLOCKS;  // persistent: the resident blocks, looping over groups
   const bool mixed = p.precision == SPH_MIXED;
+  // FP64, one instance: two lanes share a particle (a warp then walks for 16
+  // particles, whose lists fill evenly), four or eight where those still fit
+  // one wave of resident warps.  One, two, four, eight lanes: 10k cloud -,
+  // 1.58, 1.36, 1.38 ms; 50k 3.9, 3.14, 3.42, 4.28; 200k 14.4, 11.6, 10.8,
+  // 14.1; 1M 64, 55.6, 58.5, 85.4 ms.
+  A.share = !mixed && c->tree.ninst <= 1 ? 1 : 0;
+  while (A.share > 0 && A.share < 3 && (s->n << (A.share + 1)) <= (int64_t)32 * 32 * c->num_sms) ++A.share;
   const bool packed = mixed && c->tree.packed_walk;
+  // one block per chunk where their number is known (see the grid of the mixed walk)
+  const int blocks64 = c->tree.ninst <= 1 ? nblk(s->n << A.share, 32) : c->num_sms * kGrav64Blocks;
   if (s->dim == 3) {
-    if (packed) { k_gravity<true, 3, true><<<blocks, kGrWarps * 32, 0, st>>>(A); ++sph::g_launches; }
-    else if (mixed) { k_gravity<true, 3, false><<<blocks, kGrWarps * 32, 0, st>>>(A); ++sph::g_launches; }
-    else { k_gravity<false, 3, false><<<blocks, kGrWarps * 32, 0, st>>>(A); ++sph::g_launches; }
+    if (packed) k_gravity<3, true><<<blocks, kGrWarps * 32, 0, st>>>(A);
+    else if (mixed) k_gravity<3, false><<<blocks, kGrWarps * 32, 0, st>>>(A);
+    else k_gravity64<3><<<blocks64, 32, 0, st>>>(A);
   } else {
-    if (packed) { k_gravity<true, 2, true><<<blocks, kGrWarps * 32, 0, st>>>(A); ++sph::g_launches; }
-    else if (mixed) { k_gravity<true, 2, false><<<blocks, kGrWarps * 32, 0, st>>>(A); ++sph::g_launches; }
-    else { k_gravity<false, 2, false><<<blocks, kGrWarps * 32, 0, st>>>(A); ++sph::g_launches; }
+    if (packed) k_gravity<2, true><<<blocks, kGrWarps * 32, 0, st>>>(A);
+    else if (mixed) k_gravity<2, false><<<blocks, kGrWarps * 32, 0, st>>>(A);
+    else k_gravity64<2><<<blocks64, 32, 0, st>>>(A);
   }
+  ++sph::g_launches;
 }
 
 }  // namespace sph

@@ -501,7 +501,12 @@ void gravity_walk(sph_ctx *c, const sph_state *s, const sph_params &p, double *a
   A.err = c->d_err;
   A.reuse = reuse ? 1 : 0;
   A.ctr = counters(c);
-  int blocks = c->num_sms * SPH_GRAV_MIN_BLOCKS;  // persistent: the resident blocks, looping over groups
+  // One instance: a block per chunk, so that the hardware hands chunks out as
+  // warps finish (a persistent grid gave each block every 4864th chunk: at 400k
+  // two or three of them, and a last wave a sixth full; 2M cloud step 39.7 ->
+  // 36.9 ms, 400k pair window 21.3 -> 19.9 ms).  Several: the number of groups
+  // is only known on the device, and the resident blocks loop over them.
+  const int blocks = c->tree.ninst <= 1 ? nblk(s->n, 32 * kGrWarps) : c->num_sms * SPH_GRAV_MIN_BLOCKS;
   const bool mixed = p.precision == SPH_MIXED;
   // FP64, one instance: two lanes share a particle (a warp then walks for 16
   // particles, whose lists fill evenly), four or eight where those still fit
@@ -511,7 +516,6 @@ void gravity_walk(sph_ctx *c, const sph_state *s, const sph_params &p, double *a
   A.share = !mixed && c->tree.ninst <= 1 ? 1 : 0;
   while (A.share > 0 && A.share < 3 && (s->n << (A.share + 1)) <= (int64_t)32 * 32 * c->num_sms) ++A.share;
   const bool packed = mixed && c->tree.packed_walk;
-  // one block per chunk where their number is known (see the grid of the mixed walk)
   const int blocks64 = c->tree.ninst <= 1 ? nblk(s->n << A.share, 32) : c->num_sms * kGrav64Blocks;
   if (s->dim == 3) {
     if (packed) k_gravity<3, true><<<blocks, kGrWarps * 32, 0, st>>>(A);

@@ -151,6 +151,7 @@ sph_status sph_create(sph_ctx **out, int32_t dim, int64_t max_particles, int32_t
   c->sh_cnt = ctx_alloc<int32_t>(c, N, ok);
   c->sh_in = ctx_alloc<int32_t>(c, N, ok);
   c->need_walk = ctx_alloc<int32_t>(c, 1, ok);
+  c->tick = ctx_alloc<int32_t>(c, 2, ok);
   c->csr_total = ctx_alloc<int64_t>(c, 1, ok);
   c->hflags = ctx_alloc<int32_t>(c, kMaxHIter + 3, ok);
   c->vol = ctx_alloc<double>(c, N, ok);
@@ -216,6 +217,7 @@ sph_status sph_create(sph_ctx **out, int32_t dim, int64_t max_particles, int32_t
   F.ck_sum = ctx_alloc<double>(c, F.cap_chunks, ok);
   F.g_ck = ctx_alloc<int32_t>(c, F.cap_groups + 1, ok);
   if (ok) ok = cudaMemset(c->d_err, 0, sizeof(int32_t)) == cudaSuccess;
+  if (ok) ok = cudaMemset(c->tick, 0, 2 * sizeof(int32_t)) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     sph_destroy(c);

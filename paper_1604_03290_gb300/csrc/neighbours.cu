@@ -17,6 +17,9 @@
 // relative band of 6e-5 around h_ab^2 - far wider than the FP32 error of
 // about 2e-6 - are decided by the FP64 expression.  The result is therefore
 // bit-identical to the FP64 definition.
+#include <algorithm>
+#include <climits>
+
 #include "fpbits.cuh"
 #include "sph_internal.cuh"
 
@@ -28,10 +31,11 @@ namespace sph {
 #define SPH_WALK_WARPS 4
 #endif
 constexpr int kNbWarps = SPH_WALK_WARPS;
-// resident blocks per SM the walk is compiled for: 8 (64 registers) was the
-// fastest of 4..12 on GB300, the walk being latency- and issue-bound
+// resident blocks per SM the walk is compiled for: at 8 (64 registers) it
+// spills, 5 and 6 are equally fast at 1M and 5 is faster at small n (a 14k RK3
+// call 2.84 against 2.89 ms)
 #ifndef SPH_WALK_MIN_BLOCKS
-#define SPH_WALK_MIN_BLOCKS 8
+#define SPH_WALK_MIN_BLOCKS 5
 #endif
 #define SPH_WALK_BOUNDS __launch_bounds__(kNbWarps * 32, SPH_WALK_MIN_BLOCKS)
 constexpr float kBand = 6e-5f;
@@ -73,12 +77,89 @@ constexpr float kSkinF = (float)kSkin;
 constexpr float kShell2 = (1.0f + kSkinF) * (1.0f + kSkinF) * (1.0f + kBand);
 constexpr float kInner2 = (1.0f - kSkinF) * (1.0f - kSkinF) * (1.0f - kBand);
 
+// ---------------------------------------------------------------------------
+// The walk.  A warp takes one group (<= 32 particles of sibling cells) and
+//  1. finds the nodes where the walk stops (flagged in their box word) whose
+//     box comes within reach of the group's: a stack of nodes in shared
+//     memory, up to 32 popped and tested at once, one per lane, their children
+//     pushed together.  The ranges found are then sorted by their first slot,
+//     so that partners come out ascending whatever the order of the tests;
+//  2. streams the ranges' particles as one sequence, 32 at a time across range
+//     ends, and keeps those within reach of the group's box;
+//  3. tests the kept candidates, 33 to 64 at a time, against every lane's own
+//     particle.
+// Visiting the nodes one after the other, as a single particle would, cost
+// 146 dependent visits per group on the 1M impact, each a round trip to the
+// L1 or L2, and a separate round of loads and a separate test loop for every
+// range: 1.11 ms there (now 0.80), 0.40 ms with shells at 263k (now 0.26, half
+// of the difference by the tickets), 84 us for the 600 groups of a 14k body
+// (now 70).  Issue-bound at 1M (0.62G warp instructions).  Tried and left out:
+// two or four lanes per particle at small n (1 % of an RK3 call).
+// More ranges or nodes than the shared buffers hold: the ranges of that group
+// come from a one-by-one walk in slot order instead, consumed as the buffer
+// fills.
+// ---------------------------------------------------------------------------
+constexpr int kWalkStack = 384;   // nodes
+constexpr int kWalkRanges = 128;  // ranges of one group
+constexpr int kWalkCand = 64;     // kept candidates (tested when more than 32 wait)
+struct WalkScratch {
+  union {
+    int32_t stack[kWalkStack];
+    struct {
+      float4 c[kWalkCand];  // position relative to the group's reference, half its support radius
+      int32_t b[kWalkCand];
+    } cand;
+  };
+  int32_t first[kWalkRanges], count[kWalkRanges];    // as found
+  int32_t sfirst[kWalkRanges], soff[kWalkRanges];    // sorted: first slot, and number of particles before
+};
+
+// Ranges of a group, sorted by first slot, with the running particle count;
+// returns the total.
+__device__ __forceinline__ int32_t sort_ranges(WalkScratch &W, int nr, int lane) {
+  int32_t f[kWalkRanges / 32], r[kWalkRanges / 32];
+#pragma unroll
+  for (int j = 0; j < kWalkRanges / 32; ++j) {
+    f[j] = 32 * j + lane < nr ? W.first[32 * j + lane] : INT_MAX;
+    r[j] = 0;
+  }
+  for (int t = 0; t < nr; ++t) {
+    const int32_t k = W.first[t];
+#pragma unroll
+    for (int j = 0; j < kWalkRanges / 32; ++j)
+      if (32 * j < nr) r[j] += k < f[j];
+  }
+#pragma unroll
+  for (int j = 0; j < kWalkRanges / 32; ++j)
+    if (32 * j + lane < nr) {
+      W.sfirst[r[j]] = f[j];
+      W.soff[r[j]] = W.count[32 * j + lane];
+    }
+  __syncwarp();
+  int32_t total = 0;
+  for (int j = 0; j < nr; j += 32) {
+    const int32_t v = j + lane < nr ? W.soff[j + lane] : 0;
+    int32_t incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (j + lane < nr) W.soff[j + lane] = total + incl - v;
+    total += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  __syncwarp();
+  return total;
+}
+
 // OWN_H = false: interaction partners (h_ab), lists and counts, skipped when
 // the flag `done` is given and is 0 (it is then a run-if flag).  OWN_H = true:
 // only the number of particles within each particle's own h (the current h of
 // the state, not the packed one), plus the count of particles whose number
 // lies farther than tol from n_des (*unconverged); the walk is skipped once
 // *done is set.
+// Warps draw their groups from a ticket counter (tick[0]): a fixed stride left
+// half the warps a second group and the others none at 263k particles.  The
+// last warp to find no group left (tick[1] counts them) sets both back to 0.
 template <bool OWN_H, bool SHELL>
 __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *__restrict__ x,
                                            const double *__restrict__ y, const double *__restrict__ z,
@@ -88,7 +169,7 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
                                            const Units *__restrict__ U, const int32_t *__restrict__ done,
                                            int32_t *__restrict__ unconverged, double n_des, int tol,
                                            int32_t *__restrict__ sh_idx, int32_t *__restrict__ sh_cnt,
-                                           int32_t *__restrict__ sh_in, unsigned long long *ctr) {
+                                           int32_t *__restrict__ sh_in, int32_t *tick, unsigned long long *ctr) {
   static_assert(!(OWN_H && SHELL), "shells are partner candidates");
   if constexpr (OWN_H) {
     if (*done) return;
@@ -97,9 +178,10 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
   }
   // the shell widens every test by the factor (1 + kSkin) of its radius
   const float wide = SHELL ? 1.0f + kSkinF : 1.0f;
-  __shared__ float4 sc[kNbWarps][kMaxLeaf];
-  __shared__ int32_t sb[kNbWarps][kMaxLeaf];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ WalkScratch scratch[kNbWarps];
+  WalkScratch &W = scratch[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const unsigned lt_mask = (1u << lane) - 1u;
   const int ngroups = *T.ngroups;
   // The walk stops at nodes flagged in their box word (at most
   // max(leaf_size, walk_leaf) particles, or depth B; set by the tree build)
@@ -110,7 +192,11 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
   // group's box by that much keeps every node that may hold a partner.
   float gw = 0.f;
   if (grow) gw = to_f32_dir_scaled(bitsd(*grow), pow2_exp(U->invL), true, U->invL);
-  for (int g = blockIdx.x * kNbWarps + w; g < ngroups; g += gridDim.x * kNbWarps) {
+  for (;;) {
+    int g = 0;
+    if (lane == 0) g = atomicAdd(&tick[0], 1);
+    g = __shfl_sync(0xffffffffu, g, 0);
+    if (g >= ngroups) break;
     const int32_t s0 = T.grp_start[g], s1 = T.grp_end[g], inst = T.grp_inst[g];
     const int32_t slot = s0 + lane;
     const bool act = slot < s1;
@@ -151,95 +237,224 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
     }
     // relative coordinates carry an error of a few 1e-7 of the group's extent + h
     const float rslack = 1e-5f * (fmaxf(fmaxf(rh[0] - rl[0], rh[1] - rl[1]), rh[2] - rl[2]) + hg);
-    const unsigned lt_mask = (1u << lane) - 1u;
     const int32_t root = T.inst_root[inst];
-    const int32_t stop = root >= 0 ? T.skip[root] : root;
     int cnt = 0, scnt = 0;
     uint32_t sin = 0;  // shell entries that are partners (bit per entry)
-    int iter = 0;
     unsigned ntest = 0;  // candidates this lane tested (counters)
-    // Stackless pre-order walk over the node box words: (lo, +-hmax) and
-    // (hi, skip), the sign of hmax marking the nodes where the walk stops.
-    for (int32_t nd = root; nd < stop && iter <= nnodes; ++iter) {
-      const float4 bl = __ldg(&T.fbox_lo[nd]), bh = __ldg(&T.fbox_hi[nd]);
+    int32_t *out = nb_idx + a, *sout = SHELL ? sh_idx + a : nullptr;  // a = -1 writes nothing
+
+    // a node's box words: is it within reach, and where does the walk go on
+    auto reached = [&](const float4 &bl, const float4 &bh) {
       const float hw = fabsf(bl.w);
       float gx = fmaxf(0.f, fmaxf(bl.x - gh[0], gl[0] - bh.x));
       float gy = fmaxf(0.f, fmaxf(bl.y - gh[1], gl[1] - bh.y));
       float gz = fmaxf(0.f, fmaxf(bl.z - gh[2], gl[2] - bh.z));
       float d2 = gx * gx + gy * gy + gz * gz;
       float thr = (OWN_H ? hg : 0.5f * (hg + hw)) * (1.0f + 1e-5f) * wide;
-      bool enter = false;
-      if (d2 <= thr * thr) {
-        if (__float_as_uint(bl.w) >> 31) {  // the walk stops here: cull its particles
-          const int4 nr = __ldg(&T.nrec[nd]);
-          const int32_t f = nr.x, e = nr.y;
-          for (int32_t base = f; base < e; base += kMaxLeaf) {  // leaves at full depth may exceed 32
-            // stage the candidates that come within reach of the group's box
-            bool keep = false;
-            float4 cand = make_float4(0.f, 0.f, 0.f, 0.f);
-            int32_t b = -1;
-            if (base + lane < e) {
-              b = T.perm_identity ? base + lane : __ldg(&T.perm[base + lane]);
-              float4 Pb = __ldg(&pk.px(b)), Qb = __ldg(&pk.pxl(b));
-              cand = make_float4((Pb.x - cx) + (Qb.x - lx), (Pb.y - cy) + (Qb.y - ly), (Pb.z - cz) + (Qb.z - lz),
-                                 0.5f * Pb.w);  // half support radius: h_ab = h_a / 2 + h_b / 2
-              float qx = fmaxf(0.f, fmaxf(rl[0] - cand.x, cand.x - rh[0]));
-              float qy = fmaxf(0.f, fmaxf(rl[1] - cand.y, cand.y - rh[1]));
-              float qz = fmaxf(0.f, fmaxf(rl[2] - cand.z, cand.z - rh[2]));
-              float reach = (OWN_H ? hg : 0.5f * hg + cand.w) * (1.0f + 1e-5f) * wide + rslack;
-              keep = qx * qx + qy * qy + qz * qz <= reach * reach;
+      return d2 <= thr * thr;
+    };
+    // 3. the kept candidates against every lane's particle, four at a time
+    // (one round of shared loads, four independent distances); the buffer is
+    // padded with candidates out of everyone's reach
+    auto test = [&](int nc) {
+      const int np = (nc + 3) & ~3;
+      if (lane < np - nc) {
+        W.cand.c[nc + lane] = make_float4(3e38f, 3e38f, 3e38f, 0.f);
+        W.cand.b[nc + lane] = -2;
+      }
+      __syncwarp();
+      if (act) {
+        ntest += nc;
+        for (int k = 0; k < np; k += 4) {
+          const int4 b4 = *reinterpret_cast<const int4 *>(&W.cand.b[k]);
+          const int32_t bs[4] = {b4.x, b4.y, b4.z, b4.w};
+          float r2[4], h2[4];
+          bool in[4];
+          unsigned unsure = 0;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const float4 cb = W.cand.c[k + u];
+            float dx = rax - cb.x, dy = ray - cb.y, dz = raz - cb.z;
+            r2[u] = dx * dx + dy * dy + dz * dz;
+            float hab = OWN_H ? hown : hha + cb.w;
+            h2[u] = hab * hab;
+            in[u] = r2[u] < h2[u] * (1.0f - kBand);
+            if (!in[u] && !(r2[u] > h2[u] * (1.0f + kBand))) unsure |= 1u << u;
+          }
+          if (unsure) {  // rare: the FP64 predicate
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if ((unsure >> u) & 1u)
+                in[u] = OWN_H ? exact_within_own_h(x, y, z, h, dim, a, bs[u]) : exact_partner(x, y, z, h, dim, a, bs[u]);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const bool other = bs[u] != a;
+            if (in[u] && other) {
+              if constexpr (!OWN_H) {
+                if (cnt < kmax) *out = bs[u];
+                out += ld;
+              }
+              ++cnt;
             }
-            const unsigned km = __ballot_sync(0xffffffffu, keep);
-            const int c = __popc(km);
-            if (keep) {
-              const int pos = __popc(km & lt_mask);
-              sc[w][pos] = cand;
-              sb[w][pos] = b;
-            }
-            __syncwarp();
-            if (act) {
-              ntest += c;
-              for (int k = 0; k < c; ++k) {
-                const float4 cb = sc[w][k];
-                const int32_t b = sb[w][k];
-                float dx = rax - cb.x, dy = ray - cb.y, dz = raz - cb.z;
-                float r2 = dx * dx + dy * dy + dz * dz;
-                float hab = OWN_H ? hown : hha + cb.w;
-                float h2 = hab * hab;
-                bool in;
-                if (r2 < h2 * (1.0f - kBand)) in = true;
-                else if (r2 > h2 * (1.0f + kBand)) in = false;
-                else in = OWN_H ? exact_within_own_h(x, y, z, h, dim, a, b) : exact_partner(x, y, z, h, dim, a, b);
-                if (in && b != a) {
-                  if constexpr (!OWN_H)
-                    if (cnt < kmax) nb_idx[(int64_t)cnt * ld + a] = b;
-                  ++cnt;
-                  if constexpr (SHELL) {
-                    if (r2 >= h2 * kInner2) {  // a partner near the support radius
-                      if (scnt < kMaxShell) {
-                        sh_idx[(int64_t)scnt * ld + a] = b;
-                        sin |= 1u << scnt;
-                      }
-                      ++scnt;
-                    }
-                  }
-                } else if constexpr (SHELL) {
-                  if (b != a && r2 <= h2 * kShell2) {
-                    if (scnt < kMaxShell) sh_idx[(int64_t)scnt * ld + a] = b;
-                    ++scnt;
-                  }
+            if constexpr (SHELL) {
+              // near the support radius on either side
+              if (other && r2[u] >= h2[u] * kInner2 && r2[u] <= h2[u] * kShell2) {
+                if (scnt < kMaxShell) {
+                  *sout = bs[u];
+                  sin |= (uint32_t)in[u] << scnt;
                 }
+                sout += ld;
+                ++scnt;
               }
             }
-            __syncwarp();
           }
-        } else {
-          enter = true;
         }
       }
-      nd = enter ? nd + 1 : __float_as_int(bh.w);
+      __syncwarp();
+    };
+    // 2. the particles of nr ranges (sorted), culled against the group's box
+    auto consume = [&](int nr, int32_t total) {
+      int i = 0, kept = 0;  // i: this lane's range
+      int32_t b = -1;
+      float4 Pb, Qb;
+      auto load = [&](int32_t flat) {
+        b = -1;
+        if (flat < total) {
+          while (i + 1 < nr && W.soff[i + 1] <= flat) ++i;
+          const int32_t sl = W.sfirst[i] + (flat - W.soff[i]);
+          b = T.perm_identity ? sl : __ldg(&T.perm[sl]);
+          Pb = __ldg(&pk.px(b));
+          Qb = __ldg(&pk.pxl(b));
+        }
+      };
+      load(lane);
+      for (int32_t base = 0; base < total; base += 32) {
+        bool keep = false;
+        const int32_t bk = b;
+        float4 cand = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (bk >= 0) {
+          cand = make_float4((Pb.x - cx) + (Qb.x - lx), (Pb.y - cy) + (Qb.y - ly), (Pb.z - cz) + (Qb.z - lz),
+                             0.5f * Pb.w);  // half support radius: h_ab = h_a / 2 + h_b / 2
+          float qx = fmaxf(0.f, fmaxf(rl[0] - cand.x, cand.x - rh[0]));
+          float qy = fmaxf(0.f, fmaxf(rl[1] - cand.y, cand.y - rh[1]));
+          float qz = fmaxf(0.f, fmaxf(rl[2] - cand.z, cand.z - rh[2]));
+          float reach = (OWN_H ? hg : 0.5f * hg + cand.w) * (1.0f + 1e-5f) * wide + rslack;
+          keep = qx * qx + qy * qy + qz * qz <= reach * reach;
+        }
+        load(base + 32 + lane);  // the next 32, in flight during the tests
+        const unsigned km = __ballot_sync(0xffffffffu, keep);
+        if (keep) {
+          const int pos = kept + __popc(km & lt_mask);
+          W.cand.c[pos] = cand;
+          W.cand.b[pos] = bk;
+        }
+        kept += __popc(km);
+        if (kept > kWalkCand - 32) {
+          test(kept);
+          kept = 0;
+        }
+      }
+      if (kept) test(kept);
+    };
+
+    // 1. the ranges within reach
+    int nr = 0, visited = 0;
+    bool fits = true;
+    if (root >= 0) {
+      int sp = 1;
+      if (lane == 0) W.stack[0] = root;
+      __syncwarp();
+      while (sp > 0 && visited <= nnodes) {
+        const int m = min(sp, 32);
+        const int32_t nd = lane < m ? W.stack[sp - m + lane] : -1;
+        sp -= m;
+        visited += m;
+        __syncwarp();
+        bool hit = false;
+        int nc = 0;
+        int4 rec = make_int4(0, 0, 0, 0);
+        if (nd >= 0) {
+          const float4 bl = __ldg(&T.fbox_lo[nd]), bh = __ldg(&T.fbox_hi[nd]);
+          if (reached(bl, bh)) {
+            hit = (__float_as_uint(bl.w) >> 31) != 0u;  // the walk stops here
+            if (hit) rec = __ldg(&T.nrec[nd]);
+            else nc = min(T.nchild[nd], 8);
+          }
+        }
+        const unsigned hm = __ballot_sync(0xffffffffu, hit);
+        const int pos = nr + __popc(hm & lt_mask);
+        if (hit && pos < kWalkRanges) {
+          W.first[pos] = rec.x;
+          W.count[pos] = rec.y - rec.x;
+        }
+        nr += __popc(hm);
+        int incl = nc;  // children pushed by the lanes up to this one
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += u;
+        }
+        const int push = __shfl_sync(0xffffffffu, incl, 31);
+        if (nr > kWalkRanges || sp + push > kWalkStack) {
+          fits = false;
+          break;
+        }
+        const int4 *ch = reinterpret_cast<const int4 *>(T.child) + 2 * (int64_t)nd;
+        const int at = sp + incl - nc;
+        if (nc > 0) {
+          const int4 c0 = ch[0];
+          const int32_t k[4] = {c0.x, c0.y, c0.z, c0.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (j < nc) W.stack[at + j] = k[j];
+        }
+        if (nc > 4) {
+          const int4 c1 = ch[1];
+          const int32_t k[4] = {c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (4 + j < nc) W.stack[at + 4 + j] = k[j];
+        }
+        sp += push;
+        __syncwarp();
+      }
     }
-    if (iter > nnodes) raise_err(err, ERR_TIMEOUT);
+    if (fits) {
+      const int32_t total = sort_ranges(W, nr, lane);
+      consume(nr, total);
+    } else {
+      // one by one in slot order: enter a node (nd + 1) or jump its subtree
+      visited = 0;
+      nr = 0;
+      __syncwarp();
+      const int32_t stop = T.skip[root];
+      for (int32_t nd = root; nd < stop && visited <= nnodes; ++visited) {
+        const float4 bl = __ldg(&T.fbox_lo[nd]), bh = __ldg(&T.fbox_hi[nd]);
+        bool enter = false;
+        if (reached(bl, bh)) {
+          if (__float_as_uint(bl.w) >> 31) {
+            const int4 rec = __ldg(&T.nrec[nd]);
+            if (lane == 0) {
+              W.first[nr] = rec.x;
+              W.count[nr] = rec.y - rec.x;
+            }
+            if (++nr == kWalkRanges) {
+              __syncwarp();
+              const int32_t total = sort_ranges(W, nr, lane);
+              consume(nr, total);
+              nr = 0;
+            }
+          } else {
+            enter = true;
+          }
+        }
+        nd = enter ? nd + 1 : __float_as_int(bh.w);
+      }
+      __syncwarp();
+      const int32_t total = sort_ranges(W, nr, lane);
+      consume(nr, total);
+    }
+    if (visited > nnodes) raise_err(err, ERR_TIMEOUT);
     if (ctr) {
       warp_count(ctr + CTR_WALK_TESTS, ntest);
       warp_count(ctr + CTR_WALK_PARTNERS, act && !OWN_H ? (unsigned)cnt : 0u);
@@ -257,6 +472,10 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
         sh_in[a] = (int32_t)sin;
       }
     }
+  }
+  if (lane == 0 && atomicAdd(&tick[1], 1) == (int)(gridDim.x * kNbWarps) - 1) {
+    tick[0] = 0;
+    tick[1] = 0;
   }
 }
 
@@ -361,17 +580,23 @@ __global__ void __launch_bounds__(kRefineThreads)
   if (cnt > kmax) raise_err(err, ERR_NB_OVERFLOW);
 }
 
+// Blocks of a walk: the resident ones, or at small n about as many warps as
+// there are groups (16 particles a warp; idle warps still draw a ticket).
+static int walk_grid(const sph_ctx *c, int64_t n) {
+  return std::min(c->num_sms * c->tune.walk_blocks_per_sm * (4 / kNbWarps), nblk(n, 16 * kNbWarps));
+}
+
 static void walk(sph_ctx *c, const sph_state *s, cudaStream_t st, const unsigned long long *grow, int32_t *idx,
                  int32_t *cnt, bool shell, const int32_t *run_if) {
-  const int blocks = c->num_sms * c->tune.walk_blocks_per_sm * (4 / kNbWarps);
+  const int blocks = walk_grid(c, s->n);
   if (shell)
     k_partners<false, true><<<blocks, kNbWarps * 32, 0, st>>>(
         c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h, s->dim, c->kmax, idx, cnt, c->cap_n, c->d_err, grow,
-        c->units, run_if, nullptr, 0.0, 0, c->sh_idx, c->sh_cnt, c->sh_in, counters(c));
+        c->units, run_if, nullptr, 0.0, 0, c->sh_idx, c->sh_cnt, c->sh_in, c->tick, counters(c));
   else
     k_partners<false, false><<<blocks, kNbWarps * 32, 0, st>>>(
         c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h, s->dim, c->kmax, idx, cnt, c->cap_n, c->d_err, grow,
-        c->units, run_if, nullptr, 0.0, 0, nullptr, nullptr, nullptr, counters(c));
+        c->units, run_if, nullptr, 0.0, 0, nullptr, nullptr, nullptr, c->tick, counters(c));
   ++sph::g_launches;
 }
 
@@ -423,12 +648,12 @@ void adapt_h(sph_ctx *c, sph_state *s, double n_des, int tol, int max_iter, int3
   const int64_t n = s->n;
   cudaMemsetAsync(flags, 0, sizeof(int32_t) * (max_iter + 3), st);
   if (n == 0) return;
-  const int blocks = c->num_sms * c->tune.walk_blocks_per_sm * (4 / kNbWarps);
+  const int blocks = walk_grid(c, n);
   for (int i = 0; i <= max_iter; ++i) {
     { k_partners<true, false><<<blocks, kNbWarps * 32, 0, st>>>(c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h,
                                                                s->dim, c->kmax, c->nb_idx, c->nb_cnt, c->cap_n,
                                                                c->d_err, nullptr, c->units, flags, flags + 2 + i,
-                                                               n_des, tol, nullptr, nullptr, nullptr, nullptr); ++sph::g_launches; }
+                                                               n_des, tol, nullptr, nullptr, nullptr, c->tick, nullptr); ++sph::g_launches; }
     if (i == max_iter) break;
     { k_h_update<<<nblk(n, 256), 256, 0, st>>>(s->h, c->nb_cnt, n, s->dim, n_des, flags + 2 + i, flags,
                                              flags + 1); ++sph::g_launches; }

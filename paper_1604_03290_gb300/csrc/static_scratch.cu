@@ -55,6 +55,7 @@ struct Carve {
 void layout(sph_ctx *c, Carve &k, int64_t n, int ninst, int leaf_size, int kmax) {
   const int64_t N = std::max<int64_t>(n, 1);
   c->d_err = k.take<int32_t>(1);
+  c->tick = k.take<int32_t>(2);
   c->units = k.take<Units>(1);
   Tree &T = c->tree;
   for (int i = 0; i < 2; ++i) {
@@ -178,8 +179,10 @@ extern "C" sph_status sph_neighbours_static(const sph_state *s, int32_t leaf_siz
   if (c.num_sms < 1) c.num_sms = 1;
 
   cudaStream_t st = (cudaStream_t)stream;
-  // the scratch keeps the previous call's contents: clear the error word
+  // the scratch keeps the previous call's contents: clear the error word and
+  // the walk's tickets
   cudaMemsetAsync(c.d_err, 0, sizeof(int32_t), st);
+  cudaMemsetAsync(c.tick, 0, 2 * sizeof(int32_t), st);
   tree_build(&c, s, leaf_size, max_depth, st);
   find_partners(&c, s, st);
   partners_to_csr(&c, s, nb_offset, nb_index, nb_capacity, st);

@@ -98,12 +98,10 @@ sph_status sph_create(sph_ctx **out, int32_t dim, int64_t max_particles, int32_t
     T.keys[k] = ctx_alloc<unsigned long long>(c, N, ok);
     T.vals[k] = ctx_alloc<int32_t>(c, N, ok);
   }
-  T.hist_cap = (int64_t)256 * ((N + 4095) / 4096 + 1);
-  T.hist = ctx_alloc<uint32_t>(c, T.hist_cap, ok);
   T.ncount = ctx_alloc<int32_t>(c, N + 1, ok);
   T.nstart = ctx_alloc<int32_t>(c, N + 1, ok);
   T.cap_nodes = std::max<int64_t>(4096, leaf_size <= 2 ? 4 * N : 2 * N);
-  T.scan_tmp = ctx_alloc<int32_t>(c, (std::max(N, T.cap_nodes) + 1) / 4096 + 2, ok);
+  T.look = ctx_alloc<uint32_t>(c, look_words(N, T.cap_nodes), ok);
   const int64_t cn = T.cap_nodes;
   T.nnodes = ctx_alloc<int32_t>(c, 1, ok);
   T.nleaf = ctx_alloc<int32_t>(c, 1, ok);
@@ -132,8 +130,6 @@ sph_status sph_create(sph_ctx **out, int32_t dim, int64_t max_particles, int32_t
   T.inst_s0 = ctx_alloc<double>(c, ci, ok);
   T.inst_rs0 = ctx_alloc<double>(c, ci, ok);
   T.inst_root = ctx_alloc<int32_t>(c, ci, ok);
-  T.gcnt = ctx_alloc<int32_t>(c, cn + 1, ok);
-  T.gstart = ctx_alloc<int32_t>(c, cn + 1, ok);
   T.cap_groups = N + ci + 1;
   T.grp_start = ctx_alloc<int32_t>(c, T.cap_groups, ok);
   T.grp_end = ctx_alloc<int32_t>(c, T.cap_groups, ok);
@@ -348,9 +344,9 @@ static sph_status finish(sph_ctx *c, const sph_params *p, cudaStream_t st, const
 }
 
 // One full right-hand side on state s into out (tree + partners + passes).
-static void timed_tree(sph_ctx *c, const sph_state *s, const sph_params &p, cudaStream_t st) {
+static void timed_tree(sph_ctx *c, const sph_state *s, const sph_params &p, cudaStream_t st, bool pack = true) {
   int pr = prof_begin(c, st, PH_TREE);
-  tree_build(c, s, p.leaf_size, p.max_depth, st);
+  tree_build(c, s, p.leaf_size, p.max_depth, st, pack);
   prof_end(c, st, pr);
 }
 
@@ -402,7 +398,7 @@ sph_status sph_build_tree(sph_ctx *c, sph_state *s, int32_t leaf_size, int32_t m
   if ((r = check_tree_args(c, s, leaf_size, max_depth)) != SPH_OK) return r;
   cudaStream_t st = (cudaStream_t)stream;
   set_materials(c, nullptr);
-  tree_build(c, s, leaf_size, max_depth, st);
+  tree_build(c, s, leaf_size, max_depth, st, !reorder);
   if (perm && s->n > 0)
     cudaMemcpyAsync(perm, c->tree.perm, sizeof(int32_t) * s->n, cudaMemcpyDeviceToDevice, st);
   if (reorder) tree_reorder_state(c, s, st);
@@ -666,7 +662,7 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
     int pr;
     if (build) {
       // order the state along the tree once per build (coalesced partner gathers)
-      timed_tree(c, s, *p, st);
+      timed_tree(c, s, *p, st, false);  // the reorder packs
       pr = prof_begin(c, st, PH_REORDER);
       tree_reorder_state(c, s, st);
       prof_end(c, st, pr);
@@ -784,7 +780,7 @@ sph_status sph_step_rk3(sph_ctx *c, sph_state *s, const sph_material *mats, int3
       adapt_h(c, s, p->n_des, p->h_tol, p->h_iter, c->hflags, st);
       prof_end(c, st, pa);
     }
-    timed_tree(c, s, *p, st);
+    timed_tree(c, s, *p, st, false);  // the reorder packs
     int pr = prof_begin(c, st, PH_REORDER);
     tree_reorder_state(c, s, st);
     prof_end(c, st, pr);

@@ -67,16 +67,14 @@ struct Tree {
   // sort
   unsigned long long *keys[2];
   int32_t *vals[2];
-  uint32_t *hist;
-  int64_t hist_cap;
+  uint32_t *look;      // tickets, digit histograms and look-back states of a build's sort and scans (tree.cu)
   int32_t *perm;       // sorted slot -> state index (points into vals[*])
   unsigned long long *skey;  // sorted keys (points into keys[*])
-  // per-slot node emission counts and their exclusive scan; after the scan
-  // ncount holds the list of leaf ids (nleaf of them, in no fixed order)
+  // the list of leaf ids (nleaf of them, in no fixed order; scratch of n + 1
+  // counts outside a build), and the scan of the nodes that start at each slot
   int32_t *ncount;
   int32_t *nleaf;      // device scalar
   int32_t *nstart;
-  int32_t *scan_tmp;
   // nodes (pre-order)
   int64_t cap_nodes;
   int packed_walk;     // fcom_lo.w holds the packed node word (cap_nodes <= kPackedSkip + 1)
@@ -102,7 +100,6 @@ struct Tree {
   double *inst_rs0;    // 1 / s0, correctly rounded
   int32_t *inst_root;
   // walk groups: up to 32 consecutive slots inside one tree cell
-  int32_t *gcnt, *gstart;  // per node: groups it starts, and their exclusive scan (cap_nodes + 1)
   int32_t *grp_start, *grp_end, *grp_inst;
   int32_t *ngroups;    // device scalar
   int64_t cap_groups;
@@ -344,7 +341,10 @@ __device__ __forceinline__ void warp_count(unsigned long long *ctr, unsigned lon
 int prof_begin(sph_ctx *c, cudaStream_t st, int phase);
 void prof_end(sph_ctx *c, cudaStream_t st, int idx);
 // tree.cu
-void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cudaStream_t st);
+// pack: also the FP32 views of s (not needed where a reorder follows, which
+// writes those of the state in its new order)
+void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cudaStream_t st, bool pack = true);
+int64_t look_words(int64_t max_particles, int64_t cap_nodes);
 void tree_reorder_state(sph_ctx *c, sph_state *s, cudaStream_t st);
 void pack_f32(sph_ctx *c, const sph_state *s, cudaStream_t st);
 // neighbours.cu

@@ -62,13 +62,11 @@ void layout(sph_ctx *c, Carve &k, int64_t n, int ninst, int leaf_size, int kmax)
     T.keys[i] = k.take<unsigned long long>(N);
     T.vals[i] = k.take<int32_t>(N);
   }
-  T.hist_cap = (int64_t)256 * ((N + 4095) / 4096 + 1);
-  T.hist = k.take<uint32_t>(T.hist_cap);
   T.ncount = k.take<int32_t>(N + 1);
   T.nstart = k.take<int32_t>(N + 1);
   T.cap_nodes = std::max<int64_t>(4096, leaf_size <= 2 ? 4 * N : 2 * N);
   const int64_t cn = T.cap_nodes;
-  T.scan_tmp = k.take<int32_t>((std::max(N, cn) + 1) / 4096 + 2);
+  T.look = k.take<uint32_t>(look_words(N, cn));
   T.nnodes = k.take<int32_t>(1);
   T.nleaf = k.take<int32_t>(1);
   T.first = k.take<int32_t>(cn);
@@ -95,8 +93,6 @@ void layout(sph_ctx *c, Carve &k, int64_t n, int ninst, int leaf_size, int kmax)
   T.inst_s0 = k.take<double>(ninst);
   T.inst_rs0 = k.take<double>(ninst);
   T.inst_root = k.take<int32_t>(ninst);
-  T.gcnt = k.take<int32_t>(cn + 1);
-  T.gstart = k.take<int32_t>(cn + 1);
   T.cap_groups = N + ninst + 1;
   T.grp_start = k.take<int32_t>(T.cap_groups);
   T.grp_end = k.take<int32_t>(T.cap_groups);

@@ -26,14 +26,24 @@ namespace sph {
 // ---------------------------------------------------------------------------
 // Bounding boxes and validity
 // ---------------------------------------------------------------------------
-__global__ void k_bbox_init(unsigned long long *bb, int ninst) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < ninst) {
+// Words of Tree::look: counters and tickets, the digit histograms of the
+// sort, then the look-back states of the sort's tiles and of the two scans.
+enum { LK_BBOX = 0, LK_NODES, LK_GROUPS, LK_SORT = 8, LK_HIST = 64 };
+constexpr int kLookFixed = LK_HIST + 8 * 256;
+
+// Everything a build starts from, in one launch: the words of Tree::look it
+// will use, the bounding boxes, no roots, no leaves.
+__global__ void k_tree_init(Tree T, int64_t words, int ninst) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = t; i < words; i += step) T.look[i] = 0;
+  for (int64_t i = t; i < ninst; i += step) {
     for (int ax = 0; ax < 3; ++ax) {
-      bb[6 * i + ax] = dbl_to_ord(__longlong_as_double(0x7ff0000000000000LL));       // +inf
-      bb[6 * i + 3 + ax] = dbl_to_ord(__longlong_as_double((long long)0xfff0000000000000ULL));  // -inf
+      T.inst_bb[6 * i + ax] = dbl_to_ord(__longlong_as_double(0x7ff0000000000000LL));  // +inf
+      T.inst_bb[6 * i + 3 + ax] = dbl_to_ord(__longlong_as_double((long long)0xfff0000000000000ULL));  // -inf
     }
+    T.inst_root[i] = -1;
   }
+  if (t == 0) *T.nleaf = 0;
 }
 
 // min / max of order-preserving encodings (integer pipe)
@@ -52,75 +62,14 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
   return v;
 }
 
-// One block per instance when several instances are given; otherwise a
-// grid-stride pass.  Also flags non-finite positions/velocities and h, rho
-// that are not positive.
-__global__ void k_bbox(const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
-                       const double *__restrict__ vx, const double *__restrict__ vy, const double *__restrict__ vz,
-                       const double *__restrict__ h, const double *__restrict__ rho, int64_t n, int dim,
-                       const int64_t *__restrict__ inst_off, int ninst, unsigned long long *bb, int32_t *err) {
-  // extrema as order-preserving integers: comparisons stay off the FP64 unit
-  unsigned long long lo[3] = {~0ULL, ~0ULL, ~0ULL}, hi[3] = {0ULL, 0ULL, 0ULL};
-  int64_t i0, i1, stride;
-  int inst;
-  if (ninst > 1 && inst_off) {
-    inst = blockIdx.x;
-    i0 = inst_off[inst] + threadIdx.x;
-    i1 = inst_off[inst + 1];
-    stride = blockDim.x;
-  } else {
-    inst = 0;
-    i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    i1 = n;
-    stride = (int64_t)gridDim.x * blockDim.x;
-  }
-  bool bad = false;
-  for (int64_t i = i0; i < i1; i += stride) {
-    const double p[3] = {x[i], y[i], dim == 3 ? z[i] : 0.0};
-    bad |= !finite_bits(p[0]) || !finite_bits(p[1]) || !finite_bits(p[2]) || !finite_bits(vx[i]) ||
-           !finite_bits(vy[i]) || (dim == 3 && !finite_bits(vz[i])) || !positive_finite_bits(h[i]) ||
-           !positive_finite_bits(rho[i]);
-    for (int ax = 0; ax < 3; ++ax) {
-      const unsigned long long o = ord_of(p[ax]);
-      lo[ax] = o < lo[ax] ? o : lo[ax];
-      hi[ax] = o > hi[ax] ? o : hi[ax];
-    }
-  }
-  if (bad) raise_err(err, ERR_NONFINITE);
-  __shared__ unsigned long long s[6][32];
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int ax = 0; ax < 3; ++ax) {
-    unsigned long long a = warp_min_u64(lo[ax]), b = warp_max_u64(hi[ax]);
-    if (lane == 0) {
-      s[ax][w] = a;
-      s[3 + ax][w] = b;
-    }
-  }
-  __syncthreads();
-  if (w == 0) {
-    for (int ax = 0; ax < 3; ++ax) {
-      unsigned long long a = lane < nw ? s[ax][lane] : ~0ULL;
-      unsigned long long b = lane < nw ? s[3 + ax][lane] : 0ULL;
-      a = warp_min_u64(a);
-      b = warp_max_u64(b);
-      if (lane == 0) {
-        atomicMin(&bb[6 * inst + ax], a);
-        atomicMax(&bb[6 * inst + 3 + ax], b);
-      }
-    }
-  }
-}
-
 // Root cube per instance (Sect. 3.5.1): corner = per-axis minimum, edge
 // s0 = max over axes of the extent, enlarged by 2^-20 so that the particle
 // at the maximum falls inside; a zero extent (one particle) gives s0 = 1.
-__global__ void k_root(const unsigned long long *bb, int ninst, int dim, double *lo_out, double *s0_out,
-                       double *rs0_out) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ninst) return;
+__device__ void make_root(const unsigned long long *bb, int i, int dim, double *lo_out, double *s0_out,
+                          double *rs0_out) {
   double ext = 0.0;
   for (int ax = 0; ax < 3; ++ax) {
-    double lo = ord_to_dbl(bb[6 * i + ax]), hi = ord_to_dbl(bb[6 * i + 3 + ax]);
+    double lo = ord_to_dbl(__ldcg(&bb[6 * i + ax])), hi = ord_to_dbl(__ldcg(&bb[6 * i + 3 + ax]));
     if (ax >= dim || !(hi >= lo)) {  // unused axis or empty instance
       lo = 0.0;
       hi = 0.0;
@@ -134,33 +83,11 @@ __global__ void k_root(const unsigned long long *bb, int ninst, int dim, double 
   rs0_out[i] = __drcp_rn(s0);
 }
 
-__global__ void k_keys(const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
-                       int64_t n, int dim, int B, const int64_t *__restrict__ inst_off, int ninst,
-                       const double *__restrict__ ilo, const double *__restrict__ is0,
-                       const double *__restrict__ irs0, unsigned long long *keys, int32_t *vals) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int inst = inst_of(inst_off, ninst, i);
-  const double s0 = is0[inst], rs0 = irs0[inst];
-  unsigned long long kx = cell_index_fast(x[i], ilo[3 * inst + 0], s0, rs0, B);
-  unsigned long long ky = cell_index_fast(y[i], ilo[3 * inst + 1], s0, rs0, B);
-  unsigned long long key;
-  if (dim == 3) {
-    unsigned long long kz = cell_index_fast(z[i], ilo[3 * inst + 2], s0, rs0, B);
-    key = spread3(kx) | (spread3(ky) << 1) | (spread3(kz) << 2);
-  } else {
-    key = spread2(kx) | (spread2(ky) << 1);
-  }
-  key |= (unsigned long long)inst << (dim * B);
-  keys[i] = key;
-  vals[i] = (int32_t)i;
-}
-
 // Code units from particle 0 (see Units).
 __device__ __forceinline__ double pow2_floor(double v) { return (v > 0.0 && isfinite(v)) ? ldexp(1.0, ilogb(v)) : 1.0; }
 
-__global__ void k_units(const double *__restrict__ h, const double *__restrict__ m, int64_t n, int dim,
-                        double vscale, MatTable mt, Units *U) {
+__device__ void make_units(const double *__restrict__ h, const double *__restrict__ m, int64_t n, int dim,
+                           double vscale, const MatTable &mt, Units *U) {
   // every lane forms the (power-of-two) base units; lane i converts material i
   const double L = pow2_floor(n > 0 ? h[0] : 1.0), M = pow2_floor(n > 0 ? m[0] : 1.0);
   const double T = pow2_floor(L / (vscale > 0.0 ? vscale : 1.0));
@@ -223,6 +150,109 @@ __global__ void k_units(const double *__restrict__ h, const double *__restrict__
   }
 }
 
+// Bounding boxes: block (inst, j) takes chunks j, j + gridDim.y - 1, ... of
+// its instance (one block per instance took 0.49 ms for 64 instances of up to
+// 50k particles, now 0.04).  Also flags non-finite positions/velocities and h, rho that are
+// not positive.  The block after the last column forms the code units
+// meanwhile, and the last block to finish the root cubes.
+struct BboxArgs {
+  const double *x[3], *v[3], *h, *m, *rho;
+  int64_t n;
+  int dim, ninst;
+  const int64_t *inst_off;
+  double vscale;
+  MatTable mt;
+  Units *U;
+  int32_t *err;
+};
+__global__ void __launch_bounds__(256) k_bbox(BboxArgs A, Tree T) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (blockIdx.y == gridDim.y - 1) {
+    if (blockIdx.x == 0 && w == 0) make_units(A.h, A.m, A.n, A.dim, A.vscale, A.mt, A.U);
+    return;
+  }
+  const int cols = gridDim.y - 1, inst = blockIdx.x, dim = A.dim;
+  // extrema as order-preserving integers: comparisons stay off the FP64 unit
+  unsigned long long lo[3] = {~0ULL, ~0ULL, ~0ULL}, hi[3] = {0ULL, 0ULL, 0ULL};
+  const bool many = A.ninst > 1 && A.inst_off;
+  const int64_t i0 = (many ? A.inst_off[inst] : 0) + (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
+  const int64_t i1 = many ? A.inst_off[inst + 1] : A.n, stride = (int64_t)cols * blockDim.x;
+  bool bad = false;
+  for (int64_t i = i0; i < i1; i += stride) {
+    const double p[3] = {A.x[0][i], A.x[1][i], dim == 3 ? A.x[2][i] : 0.0};
+    bad |= !finite_bits(p[0]) || !finite_bits(p[1]) || !finite_bits(p[2]) || !finite_bits(A.v[0][i]) ||
+           !finite_bits(A.v[1][i]) || (dim == 3 && !finite_bits(A.v[2][i])) || !positive_finite_bits(A.h[i]) ||
+           !positive_finite_bits(A.rho[i]);
+    for (int ax = 0; ax < 3; ++ax) {
+      const unsigned long long o = ord_of(p[ax]);
+      lo[ax] = o < lo[ax] ? o : lo[ax];
+      hi[ax] = o > hi[ax] ? o : hi[ax];
+    }
+  }
+  if (bad) raise_err(A.err, ERR_NONFINITE);
+  __shared__ unsigned long long s[6][32];
+  __shared__ bool last;
+  for (int ax = 0; ax < 3; ++ax) {
+    unsigned long long a = warp_min_u64(lo[ax]), b = warp_max_u64(hi[ax]);
+    if (lane == 0) {
+      s[ax][w] = a;
+      s[3 + ax][w] = b;
+    }
+  }
+  __syncthreads();
+  if (w == 0) {
+    for (int ax = 0; ax < 3; ++ax) {
+      unsigned long long a = lane < nw ? s[ax][lane] : ~0ULL;
+      unsigned long long b = lane < nw ? s[3 + ax][lane] : 0ULL;
+      a = warp_min_u64(a);
+      b = warp_max_u64(b);
+      if (lane == 0) {
+        atomicMin(&T.inst_bb[6 * inst + ax], a);
+        atomicMax(&T.inst_bb[6 * inst + 3 + ax], b);
+      }
+    }
+    if (lane == 0) {
+      __threadfence();
+      last = atomicAdd(&T.look[LK_BBOX], 1u) == (uint32_t)cols * gridDim.x - 1u;
+    }
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = threadIdx.x; i < A.ninst; i += blockDim.x)
+    make_root(T.inst_bb, i, dim, T.inst_lo, T.inst_s0, T.inst_rs0);
+}
+
+// Morton keys, the histograms of all the digits the sort will use (a key's
+// digits are the same in every pass) and, with `pack`, the FP32 views.  Both
+// value buffers start as valid indices.
+__global__ void __launch_bounds__(256) k_keys(const double *__restrict__ x, const double *__restrict__ y,
+                                              const double *__restrict__ z, const double *__restrict__ vx,
+                                              const double *__restrict__ vy, const double *__restrict__ vz,
+                                              const double *__restrict__ h, const double *__restrict__ m,
+                                              const double *__restrict__ rho, int64_t n, int dim, int B,
+                                              const int64_t *__restrict__ inst_off, int ninst, int passes, bool pack,
+                                              PackedF32 pk, const Units *__restrict__ U, Tree T) {
+  __shared__ uint32_t hs[8][256];
+  for (int p = 0; p < passes; ++p) hs[p][threadIdx.x] = 0;
+  __syncthreads();
+  const double *__restrict__ ilo = T.inst_lo;
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+    const int inst = inst_of(inst_off, ninst, i);
+    const double xa[3] = {x[i], y[i], dim == 3 ? z[i] : 0.0};
+    const unsigned long long key = morton_key(xa, dim, B, inst, ilo, T.inst_s0[inst], T.inst_rs0[inst]);
+    T.keys[0][i] = key;
+    T.vals[0][i] = T.vals[1][i] = (int32_t)i;
+    for (int p = 0; p < passes; ++p) atomicAdd(&hs[p][(key >> (8 * p)) & 255], 1u);
+    if (pack)
+      pack_particle(pk, i, dim, xa[0], xa[1], xa[2], vx[i], vy[i], dim == 3 ? vz[i] : 0.0, h[i], m[i], rho[i],
+                    ilo + 3 * inst, U);
+  }
+  __syncthreads();
+  for (int p = 0; p < passes; ++p)
+    if (const uint32_t c = hs[p][threadIdx.x]) atomicAdd(&T.look[LK_HIST + 256 * p + threadIdx.x], c);
+}
+
 // FP32 views of the state (see PackedF32), in code units.
 __global__ void k_pack(const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
                        const double *__restrict__ vx, const double *__restrict__ vy, const double *__restrict__ vz,
@@ -237,108 +267,45 @@ __global__ void k_pack(const double *__restrict__ x, const double *__restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// LSD radix sort of (u64 key, i32 value), 8-bit digits, stable.
+// Decoupled look-back (Merrill and Garland, "Single-pass parallel prefix scan
+// with decoupled look-back"): a tile publishes its own count, adds up the
+// counts of the tiles before it until it meets one that already knows its
+// inclusive sum, and publishes its own.  Tiles are numbered by a ticket in
+// the order their blocks start, so a tile only ever waits for blocks that
+// are running.  Every wait is bounded; one that runs out raises the timeout
+// bit and goes on with the sum so far, which every later access tolerates.
+// State word: count in the low 30 bits, then 1 = the tile's own count, 2 =
+// inclusive.
 // ---------------------------------------------------------------------------
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;
-constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr uint32_t kLookOwn = 1u << 30, kLookIncl = 2u << 30, kLookVal = kLookOwn - 1u;
+constexpr int kLookPolls = 1 << 22;
 
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const unsigned long long *__restrict__ keys, int64_t n,
-                                                             int shift, uint32_t *hist, int nblocks) {
-  __shared__ uint32_t hs[256];
-  hs[threadIdx.x] = 0;
-  __syncthreads();
-  int64_t base = (int64_t)blockIdx.x * kSortTile;
-#pragma unroll 4
-  for (int it = 0; it < kSortItems; ++it) {
-    int64_t i = base + it * kSortThreads + threadIdx.x;
-    if (i < n) atomicAdd(&hs[(keys[i] >> shift) & 255], 1u);
-  }
-  __syncthreads();
-  hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = hs[threadIdx.x];
-}
+__device__ __forceinline__ uint32_t look_load(const uint32_t *p) { return *(const volatile uint32_t *)p; }
 
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const unsigned long long *__restrict__ kin,
-                                                                const int32_t *__restrict__ vin,
-                                                                unsigned long long *__restrict__ kout,
-                                                                int32_t *__restrict__ vout, int64_t n, int shift,
-                                                                const uint32_t *__restrict__ hist, int nblocks) {
-  __shared__ uint32_t off[256];
-  __shared__ uint32_t wc[kSortThreads / 32][256];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  off[threadIdx.x] = hist[(int64_t)threadIdx.x * nblocks + blockIdx.x];
-  const unsigned lt = (1u << lane) - 1u;
-  int64_t base = (int64_t)blockIdx.x * kSortTile;
-  for (int it = 0; it < kSortItems; ++it) {
-    int64_t i = base + it * kSortThreads + threadIdx.x;
-    bool valid = i < n;
-    unsigned long long key = valid ? kin[i] : 0ULL;
-    int32_t val = valid ? vin[i] : 0;
-    int d = valid ? (int)((key >> shift) & 255) : 256;
-#pragma unroll
-    for (int ww = 0; ww < kSortThreads / 32; ++ww) wc[ww][threadIdx.x] = 0;
-    __syncthreads();
-    unsigned peers = __match_any_sync(0xffffffffu, d);
-    int rank = __popc(peers & lt);
-    if (valid && rank == 0) wc[w][d] = __popc(peers);
-    __syncthreads();
-    uint32_t tot = 0;
-    {
-      int dd = threadIdx.x;
-#pragma unroll
-      for (int ww = 0; ww < kSortThreads / 32; ++ww) {
-        uint32_t t = wc[ww][dd];
-        wc[ww][dd] = tot;
-        tot += t;
-      }
+// Sum of the tiles before `tile` for one counter; called by a whole warp,
+// lane i reading the i-th tile back.  Publishes the inclusive sum.
+__device__ __forceinline__ uint32_t look_back_warp(uint32_t *state, int tile, uint32_t own, int32_t *err) {
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) *(volatile uint32_t *)&state[tile] = own | (tile == 0 ? kLookIncl : kLookOwn);
+  uint32_t before = 0;
+  for (int t = tile - 1; t >= 0; t -= 32) {
+    const int mine = t - lane;
+    uint32_t v = kLookIncl;  // before the first tile: nothing, known
+    if (mine >= 0) {
+      int polls = 0;
+      while (((v = look_load(&state[mine])) >> 30) == 0u && ++polls < kLookPolls) __nanosleep(20);
+      if (polls >= kLookPolls) raise_err(err, ERR_TIMEOUT);
     }
-    __syncthreads();
-    if (valid) {
-      uint32_t pos = off[d] + wc[w][d] + rank;
-      kout[pos] = key;
-      vout[pos] = val;
-    }
-    __syncthreads();
-    off[threadIdx.x] += tot;
-    __syncthreads();
+    const unsigned incl = __ballot_sync(0xffffffffu, (v >> 30) != 1u);
+    const int last = incl ? __ffs(incl) - 1 : 31;
+    uint32_t sum = lane <= last ? v & kLookVal : 0u;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    before += sum;
+    if (incl) break;
   }
+  if (lane == 0 && tile > 0) *(volatile uint32_t *)&state[tile] = (before + own) | kLookIncl;
+  return before;
 }
-
-static void scan_excl_i32(const int32_t *in, int32_t *out, int64_t m, int32_t *tmp, cudaStream_t st);
-
-static void radix_sort(sph_ctx *c, int64_t n, int bits, cudaStream_t st) {
-  Tree &T = c->tree;
-  int nblocks = nblk(n, kSortTile);
-  int passes = (bits + 7) / 8;
-  int src = 0;
-  for (int p = 0; p < passes; ++p) {
-    int shift = 8 * p;
-    { k_radix_hist<<<nblocks, kSortThreads, 0, st>>>(T.keys[src], n, shift, T.hist, nblocks); ++sph::g_launches; }
-    scan_excl_i32((const int32_t *)T.hist, (int32_t *)T.hist, (int64_t)256 * nblocks, T.scan_tmp, st);
-    { k_radix_scatter<<<nblocks, kSortThreads, 0, st>>>(T.keys[src], T.vals[src], T.keys[src ^ 1], T.vals[src ^ 1], n,
-                                                     shift, T.hist, nblocks); ++sph::g_launches; }
-    src ^= 1;
-  }
-  T.skey = T.keys[src];
-  T.perm = T.vals[src];
-}
-
-// Sorts (keys[0], vals[0]) of the tree's sort buffers; the result is left
-// in (skey, perm).  Used outside the tree build by the flaw generator and the
-// fragment finder, which do not need the tree afterwards.
-void sort_pairs(sph_ctx *c, int64_t n, int bits, cudaStream_t st) {
-  if (n > 0) {
-    radix_sort(c, n, bits, st);
-  } else {
-    c->tree.skey = c->tree.keys[0];
-    c->tree.perm = c->tree.vals[0];
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Exclusive scan of int32 counts (length m), three phases.
-// ---------------------------------------------------------------------------
-constexpr int kScanThreads = 256, kScanItems = 16, kScanTile = kScanThreads * kScanItems;
 
 __device__ __forceinline__ int32_t block_excl_scan(int32_t v, int32_t *total) {
   __shared__ int32_t ws[32];
@@ -365,54 +332,204 @@ __device__ __forceinline__ int32_t block_excl_scan(int32_t v, int32_t *total) {
   return res;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const int32_t *__restrict__ in, int32_t *__restrict__ out,
-                                                             int64_t m, int32_t *tile_sums) {
-  int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
+// ---------------------------------------------------------------------------
+// LSD radix sort of (u64 key, i32 value), 8-bit digits, stable: one launch per
+// digit, each reading and writing its pairs once ("onesweep", Adinets and
+// Merrill).  The digit totals come from one histogram pass over the keys.  A
+// tile ranks its pairs by warp matching, looks back per digit (a thread per
+// digit, eight tiles at a time) and scatters.  The histogram, three scan
+// kernels and scatter per digit that this replaces took 311 us of a 1M build
+// and 163 of a 4.4k one, nearly all of the latter latency; now 212 and 48 us.
+// ---------------------------------------------------------------------------
+constexpr int kSortThreads = 256;
+constexpr int kSortItems = 8;
+constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kSortWarps = kSortThreads / 32;
+
+__global__ void __launch_bounds__(kSortThreads) k_sort_hist(const unsigned long long *__restrict__ keys, int64_t n,
+                                                            int passes, uint32_t *hist) {
+  __shared__ uint32_t hs[8][256];
+  for (int p = 0; p < passes; ++p) hs[p][threadIdx.x] = 0;
+  __syncthreads();
+  for (int64_t i = (int64_t)blockIdx.x * kSortThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSortThreads) {
+    const unsigned long long k = keys[i];
+    for (int p = 0; p < passes; ++p) atomicAdd(&hs[p][(k >> (8 * p)) & 255], 1u);
+  }
+  __syncthreads();
+  for (int p = 0; p < passes; ++p)
+    if (const uint32_t c = hs[p][threadIdx.x]) atomicAdd(&hist[256 * p + threadIdx.x], c);
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_sort_pass(const unsigned long long *__restrict__ kin,
+                                                            const int32_t *__restrict__ vin,
+                                                            unsigned long long *__restrict__ kout,
+                                                            int32_t *__restrict__ vout, int64_t n, int shift,
+                                                            const uint32_t *__restrict__ hist, uint32_t *state,
+                                                            uint32_t *ticket, int32_t *err) {
+  __shared__ uint32_t wc[kSortWarps][256];
+  __shared__ uint32_t base[256];
+  __shared__ int tile_s;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = threadIdx.x;
+  const unsigned lt = (1u << lane) - 1u;
+  if (t == 0) tile_s = (int)atomicAdd(ticket, 1u);
+#pragma unroll
+  for (int ww = 0; ww < kSortWarps; ++ww) wc[ww][t] = 0;
+  __syncthreads();
+  const int tile = tile_s;
+  // a warp's pairs are consecutive, so that rank order is input order
+  const int64_t first = (int64_t)tile * kSortTile + w * (32 * kSortItems) + lane;
+  unsigned long long key[kSortItems];
+  int32_t val[kSortItems];
+  uint32_t rank[kSortItems];
+#pragma unroll
+  for (int j = 0; j < kSortItems; ++j) {
+    const int64_t i = first + 32 * j;
+    key[j] = i < n ? kin[i] : 0ULL;
+    val[j] = i < n ? vin[i] : 0;
+  }
+#pragma unroll
+  for (int j = 0; j < kSortItems; ++j) {
+    const bool valid = first + 32 * j < n;
+    const int d = valid ? (int)((key[j] >> shift) & 255) : 256;
+    const unsigned peers = __match_any_sync(0xffffffffu, d);
+    const int leader = __ffs(peers) - 1;
+    uint32_t before = 0;
+    if (valid && lane == leader) {
+      before = wc[w][d];
+      wc[w][d] = before + __popc(peers);
+    }
+    rank[j] = __shfl_sync(0xffffffffu, before, leader) + __popc(peers & lt);
+    __syncwarp();
+  }
+  __syncthreads();
+  // thread t: digit t
+  uint32_t own = 0;
+#pragma unroll
+  for (int ww = 0; ww < kSortWarps; ++ww) {
+    const uint32_t c = wc[ww][t];
+    wc[ww][t] = own;
+    own += c;
+  }
+  volatile uint32_t *mine = state + (int64_t)tile * 256 + t;
+  *mine = own | (tile == 0 ? kLookIncl : kLookOwn);
+  uint32_t before = 0;
+  bool known = tile == 0;
+  for (int q = tile - 1; q >= 0 && !known; q -= 8) {
+    uint32_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = q - u >= 0 ? look_load(&state[(int64_t)(q - u) * 256 + t]) : kLookIncl;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (known) continue;
+      int polls = 0;
+      while ((v[u] >> 30) == 0u && ++polls < kLookPolls) {
+        __nanosleep(20);
+        v[u] = look_load(&state[(int64_t)(q - u) * 256 + t]);
+      }
+      if (polls >= kLookPolls) raise_err(err, ERR_TIMEOUT);
+      before += v[u] & kLookVal;
+      known = (v[u] >> 30) != 1u;
+    }
+  }
+  if (tile > 0) *mine = (before + own) | kLookIncl;
+  int32_t total;
+  base[t] = (uint32_t)block_excl_scan((int32_t)hist[t], &total) + before;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kSortItems; ++j) {
+    if (first + 32 * j >= n) continue;
+    const int d = (int)((key[j] >> shift) & 255);
+    const int64_t pos = (int64_t)base[d] + wc[w][d] + rank[j];
+    if (pos < n) {
+      kout[pos] = key[j];
+      vout[pos] = val[j];
+    }
+  }
+}
+
+static int sort_passes(int bits) { return (bits + 7) / 8; }
+
+// The passes; Tree::look zeroed, its histograms filled
+static void sort_run(sph_ctx *c, int64_t n, int bits, cudaStream_t st) {
+  Tree &T = c->tree;
+  const int tiles = nblk(n, kSortTile), passes = sort_passes(bits);
+  int src = 0;
+  for (int p = 0; p < passes; ++p) {
+    k_sort_pass<<<tiles, kSortThreads, 0, st>>>(T.keys[src], T.vals[src], T.keys[src ^ 1], T.vals[src ^ 1], n, 8 * p,
+                                                T.look + LK_HIST + 256 * p,
+                                                T.look + kLookFixed + (int64_t)p * tiles * 256, T.look + LK_SORT + p,
+                                                c->d_err);
+    ++sph::g_launches;
+    src ^= 1;
+  }
+  T.skey = T.keys[src];
+  T.perm = T.vals[src];
+}
+
+// Sorts (keys[0], vals[0]) of the tree's sort buffers; the result is left
+// in (skey, perm).  Used outside the tree build by the flaw generator and the
+// fragment finder, which do not need the tree afterwards.
+void sort_pairs(sph_ctx *c, int64_t n, int bits, cudaStream_t st) {
+  Tree &T = c->tree;
+  if (n <= 0) {
+    T.skey = T.keys[0];
+    T.perm = T.vals[0];
+    return;
+  }
+  const int passes = sort_passes(bits);
+  cudaMemsetAsync(T.look, 0, sizeof(uint32_t) * (kLookFixed + (int64_t)passes * nblk(n, kSortTile) * 256), st);
+  k_sort_hist<<<std::min(nblk(n, kSortThreads), 2 * c->num_sms), kSortThreads, 0, st>>>(T.keys[0], n, passes,
+                                                                                       T.look + LK_HIST);
+  ++sph::g_launches;
+  sort_run(c, n, bits, st);
+}
+
+// ---------------------------------------------------------------------------
+// Exclusive scan of int32 counts (length m), one pass
+// ---------------------------------------------------------------------------
+constexpr int kScanThreads = 256, kScanItems = 16, kScanTile = kScanThreads * kScanItems;
+
+__global__ void __launch_bounds__(kScanThreads) k_scan(const int32_t *in, int32_t *out,  // may be the same
+                                                       int64_t m, uint32_t *ticket, uint32_t *state, int32_t *err) {
+  __shared__ int tile_s;
+  __shared__ uint32_t before_s;
+  if (threadIdx.x == 0) tile_s = (int)atomicAdd(ticket, 1u);
+  __syncthreads();
+  const int64_t at = (int64_t)tile_s * kScanTile + (int64_t)threadIdx.x * kScanItems;
   int32_t v[kScanItems];
   int32_t s = 0;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
-    v[k] = (base + k < m) ? in[base + k] : 0;
+    v[k] = (at + k < m) ? in[at + k] : 0;
     s += v[k];
   }
   int32_t tot;
   int32_t off = block_excl_scan(s, &tot);
+  if (threadIdx.x < 32) {
+    const uint32_t b = look_back_warp(state, tile_s, (uint32_t)tot, err);
+    if (threadIdx.x == 0) before_s = b;
+  }
+  __syncthreads();
+  off += (int32_t)before_s;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
-    if (base + k < m) out[base + k] = off;
+    if (at + k < m) out[at + k] = off;
     off += v[k];
   }
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = tot;
-}
-
-__global__ void __launch_bounds__(1024) k_scan_tops(int32_t *t, int m) {
-  int chunk = (m + 1023) / 1024;
-  int b = threadIdx.x * chunk, e = min(m, b + chunk);
-  int32_t s = 0;
-  for (int i = b; i < e; ++i) s += t[i];
-  int32_t tot;
-  int32_t off = block_excl_scan(s, &tot);
-  for (int i = b; i < e; ++i) {
-    int32_t x = t[i];
-    t[i] = off;
-    off += x;
-  }
-}
-
-__global__ void k_scan_add(int32_t *out, int64_t m, const int32_t *tile_sums) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) out[i] += tile_sums[i / kScanTile];
-}
-
-static void scan_excl_i32(const int32_t *in, int32_t *out, int64_t m, int32_t *tmp, cudaStream_t st) {
-  int tiles = nblk(m, kScanTile);
-  { k_scan_tiles<<<tiles, kScanThreads, 0, st>>>(in, out, m, tmp); ++sph::g_launches; }
-  { k_scan_tops<<<1, 1024, 0, st>>>(tmp, tiles); ++sph::g_launches; }
-  { k_scan_add<<<nblk(m, 256), 256, 0, st>>>(out, m, tmp); ++sph::g_launches; }
 }
 
 void scan_counts(sph_ctx *c, const int32_t *in, int32_t *out, int64_t m, cudaStream_t st) {
-  scan_excl_i32(in, out, m, c->tree.scan_tmp, st);
+  Tree &T = c->tree;
+  const int tiles = nblk(m, kScanTile);
+  cudaMemsetAsync(T.look, 0, sizeof(uint32_t) * (kLookFixed + tiles), st);
+  k_scan<<<tiles, kScanThreads, 0, st>>>(in, out, m, T.look, T.look + kLookFixed, c->d_err);
+  ++sph::g_launches;
+}
+
+// Words of Tree::look a context for N particles and `cap` nodes needs: a
+// build's sort and its two scans (or any other sort or scan alone).
+int64_t look_words(int64_t N, int64_t cap) {
+  return kLookFixed + (int64_t)8 * 256 * ((N + kSortTile - 1) / kSortTile) + (N + 256) / 256 + (cap + 255) / 256 + 8;
 }
 
 // ---------------------------------------------------------------------------
@@ -476,40 +593,53 @@ __device__ __forceinline__ int first_node_level(const KeyLevels &K, int64_t i, i
   return l0;
 }
 
-__global__ void k_node_count(KeyLevels K, int64_t n, int L, const int64_t *__restrict__ inst_off, int ninst,
-                             int32_t *cnt) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Nodes that start at each slot, and their scan (nstart[n] = their number); a
+// slot's nodes also get their child and arrival counts cleared.
+__global__ void __launch_bounds__(256) k_node_scan(KeyLevels K, int64_t n, int L, const int64_t *__restrict__ inst_off,
+                                                   int ninst, Tree T, uint32_t *state, int32_t *err) {
+  __shared__ int tile_s;
+  __shared__ uint32_t before_s;
+  if (threadIdx.x == 0) tile_s = (int)atomicAdd(&T.look[LK_NODES], 1u);
+  __syncthreads();
+  const int64_t i = (int64_t)tile_s * 256 + threadIdx.x;
+  int k = 0;
+  if (i < n) {
+    int64_t seg_lo, seg_hi;
+    slot_segment(inst_off, ninst, n, i, seg_lo, seg_hi);
+    const int l0 = first_node_level(K, i, seg_lo, seg_hi, L);
+    int64_t e = seg_hi;
+    for (int l = l0; l <= K.B; ++l) {
+      int64_t end = K.upper(K.prefix(i, l), l, i + 1, e);
+      ++k;
+      if (end - i <= L || l == K.B) break;
+      e = end;
+    }
+  }
+  int32_t tot;
+  int32_t off = block_excl_scan(k, &tot);
+  if (threadIdx.x < 32) {
+    const uint32_t b = look_back_warp(state, tile_s, (uint32_t)tot, err);
+    if (threadIdx.x == 0) before_s = b;
+  }
+  __syncthreads();
+  off += (int32_t)before_s;
   if (i > n) return;
+  T.nstart[i] = off;
   if (i == n) {
-    cnt[n] = 0;
+    *T.nnodes = off <= T.cap_nodes ? off : (int32_t)T.cap_nodes;
+    if (off > T.cap_nodes) raise_err(err, ERR_NODE_OVERFLOW);
     return;
   }
-  int64_t seg_lo, seg_hi;
-  slot_segment(inst_off, ninst, n, i, seg_lo, seg_hi);
-  int l0 = first_node_level(K, i, seg_lo, seg_hi, L);
-  int k = 0;
-  int64_t e = seg_hi;
-  for (int l = l0; l <= K.B; ++l) {
-    int64_t end = K.upper(K.prefix(i, l), l, i + 1, e);
-    ++k;
-    if (end - i <= L || l == K.B) break;
-    e = end;
-  }
-  cnt[i] = k;
+  for (int64_t id = off; id < off + k && id < T.cap_nodes; ++id) T.nchild[id] = T.arrived[id] = 0;
 }
 
 __global__ void k_node_emit(KeyLevels K, int64_t n, int L, const int64_t *__restrict__ inst_off, int ninst,
-                            const int32_t *__restrict__ nstart, Tree T, int32_t *err) {
+                            const int32_t *__restrict__ nstart, Tree T) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i > n) return;
-  if (i == n) {
-    *T.nnodes = nstart[n] <= T.cap_nodes ? nstart[n] : (int32_t)T.cap_nodes;
-    if (nstart[n] > T.cap_nodes) raise_err(err, ERR_NODE_OVERFLOW);
-    return;
-  }
-  if (nstart[i + 1] == nstart[i]) return;
+  if (i >= n || nstart[i + 1] == nstart[i]) return;
   int64_t seg_lo, seg_hi;
   slot_segment(inst_off, ninst, n, i, seg_lo, seg_hi);
+  if (i == seg_lo) T.inst_root[inst_of(inst_off, ninst, i)] = nstart[i];
   int l0 = first_node_level(K, i, seg_lo, seg_hi, L);
   int32_t parent = -1;
   if (l0 > 0) {
@@ -531,7 +661,7 @@ __global__ void k_node_emit(KeyLevels K, int64_t n, int L, const int64_t *__rest
       T.skip[id] = min((int64_t)nstart[end], T.cap_nodes);
       T.nrec[id] = make_int4((int32_t)i, (int32_t)end, T.skip[id], l);
       T.parent[id] = parent;
-      if (parent >= 0) {
+      if (parent >= 0 && parent < id) {  // a parent always comes first
         const int r = atomicAdd(&T.nchild[parent], 1);
         if (r < 8) T.child[8 * (int64_t)parent + r] = id;
       }
@@ -549,18 +679,6 @@ __global__ void k_node_emit(KeyLevels K, int64_t n, int L, const int64_t *__rest
     base = __shfl_sync(mask, base, leader);
     T.ncount[base + __popc(mask & ((1u << lane) - 1u))] = id;
   }
-}
-
-__global__ void k_inst_roots(const int64_t *__restrict__ inst_off, int ninst, int64_t n, const int32_t *nstart,
-                             Tree T) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ninst) return;
-  int64_t lo = 0, hi = n;
-  if (ninst > 1 && inst_off) {
-    lo = inst_off[i];
-    hi = inst_off[i + 1];
-  }
-  T.inst_root[i] = (hi > lo) ? nstart[lo] : -1;
 }
 
 // Walk groups: runs of consecutive sibling cells that each hold at most 32
@@ -633,20 +751,33 @@ __device__ int group_runs(const Tree &T, int32_t id, int32_t g0, int inst) {
   return g;
 }
 
-__global__ void k_group_count(Tree T, int32_t *gcnt) {
-  const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id > T.cap_nodes) return;
-  const int nn = *T.nnodes;
-  gcnt[id] = id < nn ? group_runs<false>(T, (int32_t)id, 0, 0) : 0;
-}
-
-__global__ void k_group_emit(Tree T, const int32_t *__restrict__ gstart, const int64_t *__restrict__ inst_off,
-                             int ninst) {
-  const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int nn = *T.nnodes;
-  if (id == 0) *T.ngroups = min(gstart[nn], (int32_t)T.cap_groups);
-  if (id >= nn || gstart[id + 1] == gstart[id]) return;
-  group_runs<true>(T, (int32_t)id, gstart[id], inst_of(inst_off, ninst, T.first[id]));
+// Counts a node's groups, scans the counts and writes the groups, in tiles of
+// 256 nodes (the number of nodes is only known on the device: the resident
+// blocks draw tiles until there are none).
+__global__ void __launch_bounds__(256) k_groups(Tree T, const int64_t *__restrict__ inst_off, int ninst,
+                                                uint32_t *state, int32_t *err) {
+  __shared__ int tile_s;
+  __shared__ uint32_t before_s;
+  const int nn = *T.nnodes, tiles = max(1, (nn + 255) / 256);
+  for (;;) {
+    if (threadIdx.x == 0) tile_s = (int)atomicAdd(&T.look[LK_GROUPS], 1u);
+    __syncthreads();
+    const int tile = tile_s;
+    if (tile >= tiles) return;
+    const int64_t id = (int64_t)tile * 256 + threadIdx.x;
+    const int k = id < nn ? group_runs<false>(T, (int32_t)id, 0, 0) : 0;
+    int32_t tot;
+    int32_t off = block_excl_scan(k, &tot);
+    if (threadIdx.x < 32) {
+      const uint32_t b = look_back_warp(state, tile, (uint32_t)tot, err);
+      if (threadIdx.x == 0) before_s = b;
+    }
+    __syncthreads();
+    off += (int32_t)before_s;
+    if (k > 0) group_runs<true>(T, (int32_t)id, off, inst_of(inst_off, ninst, T.first[id]));
+    if (tile == tiles - 1 && threadIdx.x == 255) *T.ngroups = min(off + k, (int32_t)T.cap_groups);
+    __syncthreads();
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -801,7 +932,7 @@ void pack_f32(sph_ctx *c, const sph_state *s, cudaStream_t st) {
                                        s->dim, s->inst_off, s->ninst, c->tree.inst_lo, c->units, c->pk); ++sph::g_launches; }
 }
 
-void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cudaStream_t st) {
+void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cudaStream_t st, bool pack) {
   Tree &T = c->tree;
   const int64_t n = s->n;
   const int ninst = s->ninst > 0 ? s->ninst : 1;
@@ -813,55 +944,58 @@ void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cu
   T.dim = dim;
   T.ninst = ninst;
   T.n = n;
-  { k_bbox_init<<<nblk(ninst, 128), 128, 0, st>>>(T.inst_bb, ninst); ++sph::g_launches; }
-  if (n > 0) {
-    if (ninst > 1)
-      { k_bbox<<<ninst, 256, 0, st>>>(s->x[0], s->x[1], s->x[2], s->v[0], s->v[1], s->v[2], s->h, s->rho, n, dim,
-                                   s->inst_off, ninst, T.inst_bb, c->d_err); ++sph::g_launches; }
-    else
-      { k_bbox<<<min(nblk(n, 256), 152 * 8), 256, 0, st>>>(s->x[0], s->x[1], s->x[2], s->v[0], s->v[1], s->v[2], s->h,
-                                                        s->rho, n, dim, nullptr, 1, T.inst_bb, c->d_err); ++sph::g_launches; }
+  int ibits = 0;
+  while ((1 << ibits) < ninst) ++ibits;
+  const int bits = dim * max_depth + ibits, passes = sort_passes(bits);
+  const int node_tiles = nblk(n + 1, 256), group_tiles = nblk(T.cap_nodes, 256);
+  uint32_t *node_state = T.look + kLookFixed + (int64_t)passes * nblk(n, kSortTile) * 256;
+  uint32_t *group_state = node_state + node_tiles;
+  const int64_t words = group_state + group_tiles - T.look;
+  { k_tree_init<<<std::min(nblk(std::max<int64_t>(words, ninst), 256), 4 * c->num_sms), 256, 0, st>>>(T, words, ninst); ++sph::g_launches; }
+  {
+    BboxArgs A;
+    memset(&A, 0, sizeof(A));
+    for (int k = 0; k < 3; ++k) {
+      A.x[k] = s->x[k];
+      A.v[k] = s->v[k];
+    }
+    A.h = s->h;
+    A.m = s->m;
+    A.rho = s->rho;
+    A.n = n;
+    A.dim = dim;
+    A.ninst = ninst;
+    A.inst_off = s->inst_off;
+    A.vscale = c->vscale;
+    A.mt = c->mt;
+    A.U = c->units;
+    A.err = c->d_err;
+    const int cols = (int)std::max<int64_t>(1, std::min<int64_t>(nblk(n / ninst + 1, 512), 8 * c->num_sms));
+    { k_bbox<<<dim3(ninst, cols + 1), 256, 0, st>>>(A, T); ++sph::g_launches; }
   }
-  { k_root<<<nblk(ninst, 128), 128, 0, st>>>(T.inst_bb, ninst, dim, T.inst_lo, T.inst_s0, T.inst_rs0); ++sph::g_launches; }
-  { k_units<<<1, 32, 0, st>>>(s->h, s->m, n, dim, c->vscale, c->mt, c->units); ++sph::g_launches; }
   if (n > 0) {
-    { k_keys<<<nblk(n, 256), 256, 0, st>>>(s->x[0], s->x[1], s->x[2], n, dim, max_depth, s->inst_off, ninst,
-                                         T.inst_lo, T.inst_s0, T.inst_rs0, T.keys[0], T.vals[0]); ++sph::g_launches; }
-    int ibits = 0;
-    while ((1 << ibits) < ninst) ++ibits;
-    radix_sort(c, n, dim * max_depth + ibits, st);
+    { k_keys<<<std::min(nblk(n, 256), 8 * c->num_sms), 256, 0, st>>>(
+          s->x[0], s->x[1], s->x[2], s->v[0], s->v[1], s->v[2], s->h, s->m, s->rho, n, dim, max_depth, s->inst_off,
+          ninst, passes, pack, c->pk, c->units, T); ++sph::g_launches; }
+    sort_run(c, n, bits, st);
   } else {
     T.skey = T.keys[0];
     T.perm = T.vals[0];
   }
-  pack_f32(c, s, st);
   KeyLevels K{T.skey, dim, max_depth};
-  { k_node_count<<<nblk(n + 1, 256), 256, 0, st>>>(K, n, leaf_size, s->inst_off, ninst, T.ncount); ++sph::g_launches; }
-  scan_excl_i32(T.ncount, T.nstart, n + 1, T.scan_tmp, st);
-  cudaMemsetAsync(T.nchild, 0, sizeof(int32_t) * T.cap_nodes, st);
-  cudaMemsetAsync(T.arrived, 0, sizeof(int32_t) * T.cap_nodes, st);
-  cudaMemsetAsync(T.nleaf, 0, sizeof(int32_t), st);
-  { k_node_emit<<<nblk(n + 1, 256), 256, 0, st>>>(K, n, leaf_size, s->inst_off, ninst, T.nstart, T, c->d_err); ++sph::g_launches; }
+  { k_node_scan<<<node_tiles, 256, 0, st>>>(K, n, leaf_size, s->inst_off, ninst, T, node_state, c->d_err); ++sph::g_launches; }
+  { k_node_emit<<<nblk(std::max<int64_t>(n, 1), 256), 256, 0, st>>>(K, n, leaf_size, s->inst_off, ninst, T.nstart, T); ++sph::g_launches; }
   { k_moments<<<nblk(std::max<int64_t>(n, 1), 256), 256, 0, st>>>(T, s->x[0], s->x[1], s->x[2], s->m, s->h,
                                                                    dim); ++sph::g_launches; }
   { k_node_finish<<<nblk(T.cap_nodes, 256), 256, 0, st>>>(T, dim, leaf_size, s->inst_off, ninst, c->units,
                                                         c->tune.walk_leaf); ++sph::g_launches; }
-  { k_inst_roots<<<nblk(ninst, 128), 128, 0, st>>>(s->inst_off, ninst, n, T.nstart, T); ++sph::g_launches; }
-  { k_group_count<<<nblk(T.cap_nodes + 1, 256), 256, 0, st>>>(T, T.gcnt); ++sph::g_launches; }
-  scan_excl_i32(T.gcnt, T.gstart, T.cap_nodes + 1, T.scan_tmp, st);
-  { k_group_emit<<<nblk(T.cap_nodes, 256), 256, 0, st>>>(T, T.gstart, s->inst_off, ninst); ++sph::g_launches; }
+  { k_groups<<<std::min(group_tiles, 4 * c->num_sms), 256, 0, st>>>(T, s->inst_off, ninst, group_state, c->d_err); ++sph::g_launches; }
 }
 
 // ---------------------------------------------------------------------------
 // In-place reorder of the caller's state along the tree
 // ---------------------------------------------------------------------------
-__global__ void k_iota(int32_t *p, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) p[i] = (int32_t)i;
-}
-
-// All fields at once: dst_f[i] = src_f[perm[i]] (gather) or dst_f[i] = src_f[i]
-// (copy back), doubles then ints.
+// All fields at once, doubles then ints: dst_f[i] = src_f[perm[i]].
 constexpr int kMaxFields = 20;
 struct FieldSet {
   const double *dsrc[kMaxFields];
@@ -874,10 +1008,25 @@ struct FieldSet {
 __global__ void k_gather_fields(FieldSet F, const int32_t *__restrict__ perm, int64_t n) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int64_t j = perm ? perm[i] : i;
+  const int64_t j = perm[i];
 #pragma unroll 4
   for (int f = 0; f < F.nd; ++f) F.ddst[f][i] = F.dsrc[f][j];
   for (int f = 0; f < F.ni; ++f) F.idst[f][i] = F.isrc[f][j];
+}
+
+// Back into the state's arrays, perm[i] = i, and the FP32 views of the state
+// in its new order
+__global__ void k_copy_back(FieldSet F, int32_t *__restrict__ perm, int64_t n, int dim, const sph_state s,
+                            const double *__restrict__ ilo, const Units *__restrict__ U, PackedF32 pk) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+#pragma unroll 4
+  for (int f = 0; f < F.nd; ++f) F.ddst[f][i] = F.dsrc[f][i];
+  for (int f = 0; f < F.ni; ++f) F.idst[f][i] = F.isrc[f][i];
+  perm[i] = (int32_t)i;
+  const int inst = inst_of(s.inst_off, s.ninst, i);
+  pack_particle(pk, i, dim, s.x[0][i], s.x[1][i], dim == 3 ? s.x[2][i] : 0.0, s.v[0][i], s.v[1][i],
+                dim == 3 ? s.v[2][i] : 0.0, s.h[i], s.m[i], s.rho[i], ilo + 3 * inst, U);
 }
 
 void tree_reorder_state(sph_ctx *c, sph_state *s, cudaStream_t st) {
@@ -928,10 +1077,8 @@ void tree_reorder_state(sph_ctx *c, sph_state *s, cudaStream_t st) {
     R.idst[f] = const_cast<int32_t *>(G.isrc[f]);
   }
   { k_gather_fields<<<nblk(n, 256), 256, 0, st>>>(G, c->tree.perm, n); ++sph::g_launches; }
-  { k_gather_fields<<<nblk(n, 256), 256, 0, st>>>(R, nullptr, n); ++sph::g_launches; }
-  { k_iota<<<nblk(n, 256), 256, 0, st>>>(c->tree.perm, n); ++sph::g_launches; }
+  { k_copy_back<<<nblk(n, 256), 256, 0, st>>>(R, c->tree.perm, n, s->dim, *s, c->tree.inst_lo, c->units, c->pk); ++sph::g_launches; }
   c->tree.perm_identity = 1;
-  pack_f32(c, s, st);
 }
 
 // ---------------------------------------------------------------------------

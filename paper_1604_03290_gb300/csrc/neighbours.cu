@@ -669,27 +669,69 @@ __global__ void k_cnt_copy(const int32_t *cnt, int32_t *out, int64_t n) {
   if (i == n) out[n] = 0;
 }
 
-__global__ void k_csr_fill(const int32_t *__restrict__ nb_idx, const int32_t *__restrict__ nb_cnt, int64_t ld,
-                           const int32_t *__restrict__ start, int64_t n, int64_t *off, int32_t *idx, int64_t cap,
-                           int32_t *err) {
-  int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per particle, eight neighbouring particles per block (their column
+// entries share sectors).  The lists are ascending in tree slots; in state
+// indices they are where the state is in tree order, and elsewhere each entry
+// goes to its rank, the number of smaller entries, counted against the list
+// in shared memory (up to kCsrShort entries; longer lists are read again from
+// memory).  An insertion sort into global memory, a thread per particle, took
+// 0.91 ms at 263k particles in lattice order, now 0.16.
+constexpr int kCsrShort = 128;
+constexpr int kCsrWarps = 8;
+__global__ void __launch_bounds__(32 * kCsrWarps) k_csr_fill(const int32_t *__restrict__ nb_idx,
+                                                            const int32_t *__restrict__ nb_cnt, int64_t ld,
+                                                            const int32_t *__restrict__ start, int64_t n, int64_t *off,
+                                                            int32_t *idx, int64_t cap, int32_t *err) {
+  __shared__ __align__(16) int32_t lists[kCsrWarps][kCsrShort];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t a = (int64_t)blockIdx.x * kCsrWarps + w;
   if (a > n) return;
-  off[a] = start[a];
+  const int64_t o = start[a];
+  if (lane == 0) off[a] = o;
   if (a == n) {
-    if ((int64_t)start[n] > cap) raise_err(err, ERR_CSR_OVERFLOW);
+    if (lane == 0 && o > cap) raise_err(err, ERR_CSR_OVERFLOW);
     return;
   }
-  int64_t o = start[a];
-  int k = nb_cnt[a];
+  const int k = nb_cnt[a];
   if (o + k > cap) return;
-  for (int i = 0; i < k; ++i) {  // insertion sort while copying
-    int32_t v = nb_idx[(int64_t)i * ld + a];
-    int j = i;
-    while (j > 0 && idx[o + j - 1] > v) {
-      idx[o + j] = idx[o + j - 1];
-      --j;
+  const int32_t *col = nb_idx + a;
+  if (k <= kCsrShort) {
+    constexpr int M = kCsrShort / 32;
+    int32_t *list = lists[w];
+    int32_t v[M], r[M];
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      v[j] = 32 * j + lane < k ? col[(int64_t)(32 * j + lane) * ld] : INT_MAX;
+      list[32 * j + lane] = v[j];
+      r[j] = 0;
     }
-    idx[o + j] = v;
+    __syncwarp();
+    bool sorted = true;
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+      if (32 * j + lane + 1 < k) sorted &= v[j] < list[32 * j + lane + 1];
+    if (__all_sync(0xffffffffu, sorted)) {
+#pragma unroll
+      for (int j = 0; j < M; ++j)
+        if (32 * j + lane < k) idx[o + 32 * j + lane] = v[j];
+      return;
+    }
+    for (int i = 0; i < k; i += 4) {  // entries beyond k are larger than any
+      const int4 e = *reinterpret_cast<const int4 *>(list + i);
+#pragma unroll
+      for (int j = 0; j < M; ++j)
+        if (32 * j < k) r[j] += (e.x < v[j]) + (e.y < v[j]) + (e.z < v[j]) + (e.w < v[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+      if (32 * j + lane < k) idx[o + r[j]] = v[j];
+    return;
+  }
+  for (int j = lane; j < k; j += 32) {
+    const int32_t v = col[(int64_t)j * ld];
+    int r = 0;
+    for (int i = 0; i < k; ++i) r += col[(int64_t)i * ld] < v;
+    idx[o + r] = v;
   }
 }
 
@@ -699,7 +741,7 @@ void partners_to_csr(sph_ctx *c, const sph_state *s, int64_t *off, int32_t *idx,
   int64_t n = s->n;
   { k_cnt_copy<<<nblk(n + 1, 256), 256, 0, st>>>(c->nb_cnt, c->tree.ncount, n); ++sph::g_launches; }
   scan_counts(c, c->tree.ncount, c->tree.nstart, n + 1, st);
-  { k_csr_fill<<<nblk(n + 1, 128), 128, 0, st>>>(c->nb_idx, c->nb_cnt, c->cap_n, c->tree.nstart, n, off, idx, cap,
+  { k_csr_fill<<<nblk(n + 1, kCsrWarps), 32 * kCsrWarps, 0, st>>>(c->nb_idx, c->nb_cnt, c->cap_n, c->tree.nstart, n, off, idx, cap,
                                                c->d_err); ++sph::g_launches; }
 }
 

@@ -47,3 +47,21 @@ def test_small_instances():
         roff, ridx = oracle.neighbours(ps.x[:, s0:s1], ps.h[s0:s1], 3)
         np.testing.assert_array_equal(off[s0:s1 + 1] - off[s0], roff)
         np.testing.assert_array_equal(idx[off[s0]:off[s1]] - s0, ridx)
+
+
+@pytest.mark.parametrize("h", [0.05, 0.3])
+def test_lists_of_a_state_in_tree_order(h):
+    """Lists already ascending (short) or longer than the shared-memory form."""
+    import oracle
+    from paper_1604_03290_gb300 import sph
+    rng = np.random.default_rng(7)
+    ps = wl.lattice_block(nx=3000, ny=1, nz=1)
+    ps.x, ps.h = rng.uniform(0.0, 1.0, (3, 3000)), np.full(3000, h)
+    ctx = sph.Context(3, 3000, max_neighbours=600)
+    ds = sph.DeviceState(ps)
+    sph.build_tree(ctx, ds, reorder=True)
+    off, idx = sph.neighbours(ctx, ds)
+    roff, ridx = oracle.neighbours(ds.x.cpu().numpy(), ps.h, 3)
+    assert (np.diff(roff).max() > 128) == (h > 0.1)
+    np.testing.assert_array_equal(off.cpu().numpy(), roff)
+    np.testing.assert_array_equal(idx.cpu().numpy(), ridx)

@@ -22,6 +22,7 @@
 // gravity.  Branch switches (viscosity on/off, yield on/off, EOS branches,
 // C = I fallback) are held at the forward evaluation's side.
 #include "eos.cuh"
+#include "pairs64.cuh"
 #include "sph_internal.cuh"
 
 namespace sph {
@@ -47,6 +48,7 @@ struct AdjArgs {
   float4 *Apk;                        // cotangents of the pass-A sums in code units (6 * ld)
   const Units *U;
   const float *sums;  // mixed: the forward pass A's pair sums (16 rows of stride ld)
+  int lane_shift;     // FP64: 2^lane_shift lanes share a particle's partner list
 };
 
 __device__ __forceinline__ int sidx(int dim, int i, int j) { return symk(dim, i, j); }
@@ -90,7 +92,6 @@ template <class R>
 struct KPair {
   R phi, dphi_r, W, dWdr;
 };
-using KernelPair = KPair<double>;
 
 template <class R>
 __device__ __forceinline__ KPair<R> kernel_pair(int dim, R r, R hab) {
@@ -139,7 +140,6 @@ template <class R>
 struct VPair {
   R vx, Pi, dPi_dnu, dnu_dvx, dnu_dr2, dPi_dc, dPi_drb;
 };
-using ViscPair = VPair<double>;
 
 template <class R>
 __device__ __forceinline__ VPair<R> visc_pair(int dim, const R d[3], const R w[3], R r2, R hab,
@@ -233,71 +233,112 @@ __device__ __forceinline__ void load_T64(const AdjArgs &A, int64_t a, double t[6
   for (int k = 0; k < 6; ++k) t[k] = k < ns ? A.T[(int64_t)k * A.ld + a] : 0.0;
 }
 
-// The kernels are instantiated per dimension, so that every small-matrix loop
-// has a compile-time bound and the matrices stay in registers.
+// FP64, per dimension (every small-matrix loop has a compile-time bound and the
+// matrices stay in registers).  Both terms of a pair are one bilinear form in
+// d and w: with y = m_e vb_c - m_c vb_e - (m_e ub_c + m_c ub_e) w / 2 the sum of
+// the two is phi y.(B d), so that one product B d, one B y and one outer
+// product give every cotangent of the pair.  Bound by the FP64 unit; about 150
+// FP64 instructions a pair where evaluating the two terms one after the other,
+// with their divisions, took 490 (33k particles: 1.40 -> 0.50 ms).
 template <int DIM>
 __global__ void k_adj_passB(AdjArgs A) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> A.lane_shift;
   if (c >= A.n) return;
-  constexpr int dim = DIM;
-  const int ns = nsym(dim);
-  double xc[3] = {0, 0, 0}, vc[3] = {0, 0, 0}, vbc[3] = {0, 0, 0};
-  for (int i = 0; i < dim; ++i) {
+  const Lanes64 ln(A.lane_shift);
+  constexpr int NS = DIM == 3 ? 6 : 3;
+  const sph_params &P = A.prm;
+  double xc[DIM], vc[DIM], vbc[DIM], Tc[6];
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
     xc[i] = A.x[i][c];
     vc[i] = A.v[i][c];
     vbc[i] = A.bdv[i] ? A.bdv[i][c] : 0.0;
   }
   const double ubc = A.bdu ? A.bdu[c] : 0.0;
-  double Tc[6];
   load_T64(A, c, Tc);
-  const double hc = A.h[c], rc = A.rho[c], csc = A.cs[c], mc = A.m[c];
-  double gx[3] = {0, 0, 0}, gv[3] = {0, 0, 0}, Tb_acc[6] = {0, 0, 0, 0, 0, 0};
-  double csbar = 0.0, rhobar = 0.0;
+  const double rc = A.rho[c], csc = A.cs[c], mc = A.m[c];
+  Support64<DIM> H;
+  H.start(A.h[c]);
+  double gx[DIM], gv[DIM], Tb[6], csbar = 0.0, rhobar = 0.0;
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) gx[i] = gv[i] = 0.0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) Tb[k] = 0.0;
   const int cnt = A.nb_cnt[c];
-  for (int k = 0; k < cnt; ++k) {
+  for (int k = ln.sub; k < cnt; k += ln.n) {
     const int32_t e = A.nb_idx[(int64_t)k * A.ld + c];
-    double d[3] = {0, 0, 0}, w[3] = {0, 0, 0}, vbe[3] = {0, 0, 0};
-    for (int i = 0; i < dim; ++i) {
+    const double me = A.m[e];
+    const double U = 0.5 * fma(me, ubc, A.bdu ? mc * A.bdu[e] : 0.0);
+    double d[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0}, y[3] = {0.0, 0.0, 0.0}, B[6];
+    double r2 = 0.0, vx = 0.0, yd = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
       d[i] = xc[i] - A.x[i][e];
       w[i] = vc[i] - A.v[i][e];
-      vbe[i] = A.bdv[i] ? A.bdv[i][e] : 0.0;
+      y[i] = fma(-U, w[i], fma(me, vbc[i], A.bdv[i] ? -mc * A.bdv[i][e] : 0.0));
+      r2 = fma(d[i], d[i], r2);
+      vx = fma(w[i], d[i], vx);
+      yd = fma(y[i], d[i], yd);
     }
-    const double ube = A.bdu ? A.bdu[e] : 0.0;
-    double Te[6];
-    load_T64(A, e, Te);
-    const double he = A.h[e], re = A.rho[e], cse = A.cs[e], me = A.m[e];
-    const double hab = 0.5 * (hc + he);
-    double r2 = 0.0;
-    for (int i = 0; i < dim; ++i) r2 += d[i] * d[i];
-    const KernelPair K = kernel_pair(dim, sqrt(r2), hab);
-    const ViscPair Vs = visc_pair(dim, d, w, r2, hab, rc, re, csc, cse, A.prm);
-    double db[3], wb[3], Bs[6], csh, rh;
-    // c's own term with partner e
-    pairB_adj(dim, d, w, K, Vs, Tc, Te, me, vbc, ubc, db, wb, Bs, csh, rh);
-    for (int i = 0; i < dim; ++i) {
-      gx[i] += db[i];
-      gv[i] += wb[i];
+#pragma unroll
+    for (int q = 0; q < NS; ++q) B[q] = Tc[q] + A.T[(int64_t)q * A.ld + e];
+    H.partner(A.h[e]);
+    double phi, dphi, qq;
+    radial64(H, r2, phi, dphi, qq);
+    double vxb = 0.0, r2b = 0.0;  // cotangents of v.r and (twice) r^2 through the viscosity
+    if ((int64_t)dbits(vx) < 0) {
+      const double iQ = rcp64(fma(P.eps_v * H.hab, H.hab, r2)), irb = rcp64(rc + A.rho[e]);
+      const double nu = H.hab * vx * iQ, cb = P.alpha * (csc + A.cs[e]), b2 = 2.0 * P.beta * nu;
+      const double Pi = nu * (b2 - cb) * irb;  // = (-alpha c nu + beta nu^2) / rho, c and rho means
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) B[i] -= Pi;
+      const double pib = -phi * yd;  // cotangent of Pi
+      const double nub = pib * (2.0 * b2 - cb) * irb;
+      vxb = nub * H.hab * iQ;
+      r2b = -2.0 * nub * nu * iQ;
+      csbar = fma(-pib * P.alpha, nu * irb, csbar);
+      rhobar = fma(-pib, Pi * irb, rhobar);
     }
-    for (int q = 0; q < ns; ++q) Tb_acc[q] += Bs[q];
-    csbar += csh;
-    rhobar += rh;
-    // e's term with partner c, differentiated with respect to c
-    double dn[3] = {-d[0], -d[1], -d[2]}, wn[3] = {-w[0], -w[1], -w[2]};
-    pairB_adj(dim, dn, wn, K, Vs, Te, Tc, mc, vbe, ube, db, wb, Bs, csh, rh);
-    for (int i = 0; i < dim; ++i) {
-      gx[i] -= db[i];
-      gv[i] -= wb[i];
+    double s[3], t[3];
+    sym_mv(DIM, B, d, s);
+    sym_mv(DIM, B, y, t);
+    double Fs = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) Fs = fma(y[i], s[i], Fs);
+    const double cd = fma(dphi, Fs, r2b), cw = -U * phi;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      gx[i] += fma(phi, t[i], fma(cd, d[i], vxb * w[i]));
+      gv[i] += fma(cw, s[i], vxb * d[i]);
+      y[i] *= phi;
     }
-    for (int q = 0; q < ns; ++q) Tb_acc[q] += Bs[q];
-    csbar += csh;
-    rhobar += rh;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+#pragma unroll
+      for (int j = i; j < DIM; ++j) {
+        const int q = symk(DIM, i, j);
+        Tb[q] = fma(y[i], d[j], Tb[q]);
+        if (j > i) Tb[q] = fma(y[j], d[i], Tb[q]);
+      }
   }
-  for (int i = 0; i < dim; ++i) {
+  const double norm = 6.0 * kernel_sigma<double>(DIM);
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
+    gx[i] = norm * ln.sum(gx[i]);
+    gv[i] = norm * ln.sum(gv[i]);
+  }
+#pragma unroll
+  for (int q = 0; q < NS; ++q) Tb[q] = (q < DIM ? 1.0 : 0.5) * norm * ln.sum(Tb[q]);
+  csbar = norm * ln.sum(csbar);
+  rhobar = norm * ln.sum(rhobar);
+  if (ln.sub) return;
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
     A.gx[i][c] += gx[i];
     A.gv[i][c] += gv[i];
   }
   A.grho[c] += rhobar;
-  for (int q = 0; q < 6; ++q) A.Tbar[(int64_t)q * A.ld + c] = q < ns ? Tb_acc[q] : 0.0;
+  for (int q = 0; q < 6; ++q) A.Tbar[(int64_t)q * A.ld + c] = q < NS ? Tb[q] : 0.0;
   A.csbar[c] = csbar;
 }
 
@@ -353,8 +394,8 @@ __device__ void eos_scaled(const sph_material &M0, double s, double rho, double 
 // reverse is linear in the cotangents it is given (of T, c_s and dS/dt), so
 // each particle's are scaled by a power of two to order one first and its
 // results scaled back exactly: FP32's exponent range then limits only the
-// state, whose SI values it holds.  FP64: the sums are recomputed here, and
-// the reverse is FP64 throughout (F = double, no scaling).
+// state, whose SI values it holds.  FP64: the sums of the FP64 pass A, and the
+// reverse is FP64 throughout (F = double, no scaling).
 template <bool MIXED, int DIM>
 __global__ void k_adj_update(AdjArgs A) {
   using F = typename std::conditional<MIXED, float, double>::type;
@@ -371,42 +412,19 @@ __global__ void k_adj_update(AdjArgs A) {
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) L[i][j] = G[i][j] = F(0);
   const int cnt = A.nb_cnt[c];
-  if constexpr (MIXED) {
-    // k_passA's KEEP_SUMS layout; the continuity sum and G are rates (code
-    // unit 1/T, a power of two: the conversion is exact), L is a number
-    const float *sm = A.sums;
-    const float it = (float)A.U->invT;
-    srho = (double)sm[c] * A.U->invT;
+  {
+    // k_passA's KEEP_SUMS layout; the continuity sum and G are rates (mixed:
+    // code unit 1/T, a power of two, so that the conversion is exact), L is a
+    // number.  FP64: the rows this kernel overwrites at its end.
+    const F *sm;
+    if constexpr (MIXED) sm = A.sums;
+    else sm = A.inter;
+    const F it = MIXED ? (F)A.U->invT : F(1);
+    srho = MIXED ? (double)sm[c] * A.U->invT : (double)sm[c];
     for (int i = 0; i < dim; ++i)
       for (int j = 0; j <= i; ++j) L[i][j] = L[j][i] = sm[(int64_t)(1 + i * (i + 1) / 2 + j) * ld + c];
     for (int i = 0; i < dim; ++i)
       for (int j = 0; j < dim; ++j) G[i][j] = sm[(int64_t)(7 + 3 * i + j) * ld + c] * it;
-  } else {
-    double xc[3] = {0, 0, 0}, vc[3] = {0, 0, 0};
-    for (int i = 0; i < dim; ++i) {
-      xc[i] = A.x[i][c];
-      vc[i] = A.v[i][c];
-    }
-    const double hc = A.h[c];
-    for (int k = 0; k < cnt; ++k) {
-      const int32_t e = A.nb_idx[(int64_t)k * A.ld + c];
-      double d[3] = {0, 0, 0}, w[3] = {0, 0, 0}, r2 = 0.0;
-      for (int i = 0; i < dim; ++i) {
-        d[i] = xc[i] - A.x[i][e];
-        w[i] = vc[i] - A.v[i][e];
-        r2 += d[i] * d[i];
-      }
-      const KernelPair K = kernel_pair(dim, sqrt(r2), 0.5 * (hc + A.h[e]));
-      const double vol = A.m[e] / A.rho[e];
-      double wg = 0.0;
-      for (int i = 0; i < dim; ++i) wg += w[i] * K.phi * d[i];
-      srho += vol * wg;
-      for (int i = 0; i < dim; ++i)
-        for (int j = 0; j < dim; ++j) {
-          L[i][j] -= vol * d[i] * K.phi * d[j];
-          G[i][j] -= vol * w[i] * K.phi * d[j];
-        }
-    }
   }
   F C[3][3];
   const bool corr = P.consistency && cnt >= dim + 1 && invert_L<F>(dim, L, C);
@@ -655,12 +673,22 @@ __global__ void k_adj_update(AdjArgs A) {
     if (A.bdx[i]) A.gv[i][c] += A.bdx[i][c];
   double *I = A.inter;
   I[c] = rc * bdr;
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      I[(1 + 3 * i + j) * ld + c] = (double)Lbar[i][j] * isc;
-      I[(10 + 3 * i + j) * ld + c] = (double)Gbar[i][j] * isc;
-    }
-  for (int i = 0; i < 3; ++i) I[(19 + i) * ld + c] = (i < dim && A.bdx[i]) ? P.xsph * A.bdx[i][c] : 0.0;
+  if constexpr (MIXED) {
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j) {
+        I[(1 + 3 * i + j) * ld + c] = (double)Lbar[i][j] * isc;
+        I[(10 + 3 * i + j) * ld + c] = (double)Gbar[i][j] * isc;
+      }
+    for (int i = 0; i < 3; ++i) I[(19 + i) * ld + c] = (i < dim && A.bdx[i]) ? P.xsph * A.bdx[i][c] : 0.0;
+  } else {
+    // the layout of k_adj_passA: L's cotangent enters through d^T Lbar d only
+    for (int i = 0; i < dim; ++i)
+      for (int j = i; j < dim; ++j)
+        I[(1 + sidx(dim, i, j)) * ld + c] = i == j ? (double)Lbar[i][i] : (double)(Lbar[i][j] + Lbar[j][i]);
+    for (int i = 0; i < dim; ++i)
+      for (int j = 0; j < dim; ++j) I[(7 + 3 * i + j) * ld + c] = Gbar[i][j];
+    for (int i = 0; i < dim; ++i) I[(16 + i) * ld + c] = A.bdx[i] ? P.xsph * A.bdx[i][c] : 0.0;
+  }
   A.pbar[c] = strength ? (double)mubar * isc : 0.0;
   A.pbar[ld + c] = (double)Y0bar * isc;
   A.pbar[2 * ld + c] = (double)Kbar * isc;
@@ -676,19 +704,6 @@ template <class R>
 struct ACot {
   R sr, Lb[3][3], Gb[3][3], xb[3];
 };
-
-__device__ __forceinline__ ACot<double> load_acot64(const double *I, int64_t ld, int64_t a) {
-  ACot<double> c;
-  c.sr = I[a];
-  for (int i = 0; i < 3; ++i) {
-    for (int j = 0; j < 3; ++j) {
-      c.Lb[i][j] = I[(1 + 3 * i + j) * ld + a];
-      c.Gb[i][j] = I[(10 + 3 * i + j) * ld + a];
-    }
-    c.xb[i] = I[(19 + i) * ld + a];
-  }
-  return c;
-}
 
 // K: the kernel factors of the pair, r = |d|; Ct: the cotangents of the sums
 // of the particle whose term this is.
@@ -746,50 +761,117 @@ __device__ void pairA_adj(int dim, const R d[3], const R w[3], R r, const KPair<
   rho_b_bar += -volbar * vol / rho_b;
 }
 
+// FP64.  As in pass B both terms of a pair are one form in d and w,
+//   phi (alpha w.d - d^T Lam d - w^T Gam d) - W w.xi,
+// with alpha = V_e sr_c + V_c sr_e, Lam and Gam the same combinations of the
+// cotangents of L (symmetric part) and G, xi = 2 (m_e xb_c - m_c xb_e) / (rho_c +
+// rho_e); only the derivative of V_c in rho_c needs e's term by itself.  About
+// 180 FP64 instructions a pair instead of 430 (33k particles: 1.23 -> 0.64
+// ms).
 template <int DIM>
 __global__ void k_adj_passA(AdjArgs A) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> A.lane_shift;
   if (c >= A.n) return;
-  constexpr int dim = DIM;
-  double xc[3] = {0, 0, 0}, vc[3] = {0, 0, 0};
-  for (int i = 0; i < dim; ++i) {
+  const Lanes64 ln(A.lane_shift);
+  constexpr int NS = DIM == 3 ? 6 : 3;
+  const int64_t ld = A.ld;
+  const double *I = A.inter;
+  const bool xsph = A.prm.xsph != 0.0;
+  double xc[DIM], vc[DIM], Lc[NS], Gc[DIM][DIM], xb[DIM];
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
     xc[i] = A.x[i][c];
     vc[i] = A.v[i][c];
+    xb[i] = I[(16 + i) * ld + c];
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) Gc[i][j] = I[(7 + 3 * i + j) * ld + c];
   }
-  const double hc = A.h[c], rc = A.rho[c], mc = A.m[c];
-  const ACot<double> Cc = load_acot64(A.inter, A.ld, c);
-  double gx[3] = {0, 0, 0}, gv[3] = {0, 0, 0}, grho = 0.0;
+#pragma unroll
+  for (int q = 0; q < NS; ++q) Lc[q] = I[(1 + q) * ld + c];
+  const double src = I[c], rc = A.rho[c], mc = A.m[c], Vc = A.pk.vol[c];
+  Support64<DIM> H;
+  H.start(A.h[c]);
+  double gx[DIM], gv[DIM], gvol = 0.0, gxs = 0.0;
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) gx[i] = gv[i] = 0.0;
   const int cnt = A.nb_cnt[c];
-  for (int k = 0; k < cnt; ++k) {
-    const int32_t e = A.nb_idx[(int64_t)k * A.ld + c];
-    double d[3] = {0, 0, 0}, w[3] = {0, 0, 0};
-    for (int i = 0; i < dim; ++i) {
+  for (int k = ln.sub; k < cnt; k += ln.n) {
+    const int32_t e = A.nb_idx[(int64_t)k * ld + c];
+    const double Ve = A.pk.vol[e];
+    double d[DIM], w[DIM], r2 = 0.0, wd = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
       d[i] = xc[i] - A.x[i][e];
       w[i] = vc[i] - A.v[i][e];
+      r2 = fma(d[i], d[i], r2);
+      wd = fma(w[i], d[i], wd);
     }
-    const double he = A.h[e], re = A.rho[e], me = A.m[e];
-    const double hab = 0.5 * (hc + he);
-    double r2 = 0.0;
-    for (int i = 0; i < dim; ++i) r2 += d[i] * d[i];
-    const double r = sqrt(r2);
-    const KernelPair K = kernel_pair(dim, r, hab);
-    double db[3], wb[3], ra, rb;
-    pairA_adj(dim, d, w, r, K, me, rc, re, Cc, db, wb, ra, rb);  // c's own term
-    for (int i = 0; i < dim; ++i) {
-      gx[i] += db[i];
-      gv[i] += wb[i];
+    H.partner(A.h[e]);
+    double phi, dphi, q;
+    radial64(H, r2, phi, dphi, q);
+    // e's term per unit volume, and the combined coefficients applied to d and w
+    const double sre = I[e], al = fma(Ve, src, Vc * sre);
+    double te = sre * wd, qd = al * wd;
+    double lam[DIM], gam[DIM], gat[DIM];  // (Lam + Lam^T) d, Gam d, Gam^T w
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) lam[i] = gam[i] = gat[i] = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+#pragma unroll
+      for (int j = i; j < DIM; ++j) {  // row symk: the sum of both off-diagonal entries
+        const int s = symk(DIM, i, j);
+        const double le = I[(1 + s) * ld + e], l = fma(Ve, Lc[s], Vc * le), dd = d[i] * d[j];
+        te = fma(-le, dd, te);
+        qd = fma(-l, dd, qd);
+        if (i == j) {
+          lam[i] = fma(2.0 * l, d[i], lam[i]);
+        } else {
+          lam[i] = fma(l, d[j], lam[i]);
+          lam[j] = fma(l, d[i], lam[j]);
+        }
+      }
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) {
+        const double ge = I[(7 + 3 * i + j) * ld + e], g = fma(Ve, Gc[i][j], Vc * ge);
+        te = fma(-ge, w[i] * d[j], te);
+        gam[i] = fma(g, d[j], gam[i]);
+        gat[j] = fma(g, w[i], gat[j]);
+      }
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) qd = fma(-w[i], gam[i], qd);
+    double cd = dphi * qd;
+    if (xsph) {
+      const double me = A.m[e], ir = rcp64(rc + A.rho[e]), W = value64(q) * H.hD * (1.0 / 6.0);
+      double wx = 0.0;
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) {
+        const double xi = 2.0 * ir * fma(me, xb[i], -mc * I[(16 + i) * ld + e]);
+        wx = fma(w[i], xi, wx);
+        gv[i] = fma(-W, xi, gv[i]);
+      }
+      cd = fma(-phi, wx, cd);
+      gxs = fma(W * ir, wx, gxs);
     }
-    grho += ra;
-    double dn[3] = {-d[0], -d[1], -d[2]}, wn[3] = {-w[0], -w[1], -w[2]};
-    const ACot<double> Ce = load_acot64(A.inter, A.ld, e);
-    pairA_adj(dim, dn, wn, r, K, mc, re, rc, Ce, db, wb, ra, rb);  // e's term, w.r.t. c
-    for (int i = 0; i < dim; ++i) {
-      gx[i] -= db[i];
-      gv[i] -= wb[i];
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      gx[i] = fma(phi, fma(al, w[i], -lam[i] - gat[i]), fma(cd, d[i], gx[i]));
+      gv[i] = fma(phi, fma(al, d[i], -gam[i]), gv[i]);
     }
-    grho += rb;
+    gvol = fma(phi, te, gvol);
   }
-  for (int i = 0; i < dim; ++i) {
+  const double norm = 6.0 * kernel_sigma<double>(DIM);
+  // dV_c / drho_c = -V_c / rho_c
+  const double grho = norm * ln.sum(gxs - gvol * (Vc / rc));
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
+    gx[i] = norm * ln.sum(gx[i]);
+    gv[i] = norm * ln.sum(gv[i]);
+  }
+  if (ln.sub) return;
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
     A.gx[i][c] += gx[i];
     A.gv[i][c] += gv[i];
   }
@@ -1122,14 +1204,20 @@ void rhs_adjoint(sph_ctx *c, const sph_state *s, const MatTable &mt, const sph_p
     { k_adj_pack_acot32<<<nblk(n, 256), 256, 0, st>>>(A); ++sph::g_launches; }
     if (s->dim == 3) { k_adj_passA32<3><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
     else { k_adj_passA32<2><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
-  } else if (s->dim == 3) {
-    { k_adj_passB<3><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
-    { k_adj_update<false, 3><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
-    { k_adj_passA<3><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
   } else {
-    { k_adj_passB<2><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
-    { k_adj_update<false, 2><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
-    { k_adj_passA<2><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
+    A.pk = c->pk;
+    A.lane_shift = lanes64_shift(n, c->num_sms);
+    const int T64 = threads64(n, c->num_sms, T), g = nblk(n << A.lane_shift, T64), gu = nblk(n, T64);
+    if (s->dim == 3) {
+      k_adj_passB<3><<<g, T64, 0, st>>>(A);
+      k_adj_update<false, 3><<<gu, T64, 0, st>>>(A);
+      k_adj_passA<3><<<g, T64, 0, st>>>(A);
+    } else {
+      k_adj_passB<2><<<g, T64, 0, st>>>(A);
+      k_adj_update<false, 2><<<gu, T64, 0, st>>>(A);
+      k_adj_passA<2><<<g, T64, 0, st>>>(A);
+    }
+    sph::g_launches += 3;
   }
   const int ninst = s->ninst > 0 ? s->ninst : 1;
   if (param_bar) adj_params_sum(c, s->mat, s->inst_off, ninst, n, mt.nmat, param_bar, st);

@@ -833,7 +833,7 @@ sph_status sph_rhs_adjoint(sph_ctx *c, sph_state *s, const sph_material *mats, i
   fwd.n_act = B.d_nact[0];
   tree_build(c, s, q.leaf_size, q.max_depth, st);
   find_partners(c, s, st);
-  rhs_passes(c, s, mt, q, fwd, st, q.precision == SPH_MIXED ? c->adj_sums : nullptr);
+  rhs_passes(c, s, mt, q, fwd, st, true);
   rhs_adjoint(c, s, mt, q, *dbar, sbar, param_bar, st);
   return finish(c, p, st, "sph_rhs_adjoint");
 }

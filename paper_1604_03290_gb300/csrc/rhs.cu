@@ -32,8 +32,8 @@
 #include <type_traits>
 
 #include "eos.cuh"
-#include "fp64fast.cuh"
 #include "fpbits.cuh"
+#include "pairs64.cuh"
 #include "sph_internal.cuh"
 
 namespace sph {
@@ -58,7 +58,8 @@ struct RhsArgs {
   const double *ag;         // gravity (3 * ld) or NULL
   double *rho_out;          // density-sum output
   const Units *U;           // code units of the FP32 views (mixed mode)
-  float *sums;              // mixed, KEEP_SUMS: pass A's pair sums (16 rows of stride ld)
+  float *sums;              // KEEP_SUMS: pass A's pair sums (16 rows of stride ld), mixed
+  double *sums64;           // or FP64
   int lane_shift;           // FP64: 2^lane_shift lanes share a particle's partner list
   MatTable mt;
   sph_params prm;
@@ -80,10 +81,6 @@ __device__ __forceinline__ float rsqrt_or_zero(float r2) { return r2 > 0.f ? rsq
 #else
 #define SPH_PASSB_BOUNDS __launch_bounds__(128)
 #endif
-
-// FP64 passes: the warps per SM below which several lanes share a particle's
-// list (see rhs_passes).
-constexpr int kLaneWarps = 4;
 
 // 1 / x, correctly rounded: the same value as the division
 template <class R>
@@ -246,52 +243,6 @@ struct PartnerCursor {
   }
 };
 
-// ---------------------------------------------------------------------------
-// FP64 pair sums.  Bound by the FP64 unit, so each pair is written in as few
-// FP64 instructions as its terms need: reciprocals from fp64fast.cuh, V_b read
-// from an array (one gather instead of a division), powers of 1/h_ab kept
-// while h_b stays the same from partner to partner (a bit test), the kernel
-// slope as one product of two linear factors whose coefficients are selected
-// by the branch, and the kernel norm applied to the sums.
-// ---------------------------------------------------------------------------
-template <int DIM>
-struct Support64 {
-  double ha, hab, hinv, hD, hD1;  // h_a, h_ab, 1/h_ab, its powers D and D + 1
-  uint64_t last;                  // bits of the h_b these belong to
-  __device__ __forceinline__ void set(double hb) {
-    last = dbits(hb);
-    hab = 0.5 * (ha + hb);
-    hinv = rcp64(hab);
-    const double i2 = hinv * hinv;
-    hD = DIM == 3 ? i2 * hinv : i2;
-    hD1 = hD * hinv;
-  }
-  __device__ __forceinline__ void start(double h) {
-    ha = h;
-    set(h);
-  }
-  __device__ __forceinline__ void partner(double hb) {
-    if (dbits(hb) != last) set(hb);
-  }
-};
-
-// The lanes that share one particle's list: lane `sub` of n takes partners
-// sub, sub + n, ...  Sums are combined over the group in a fixed order.
-struct Lanes64 {
-  int sub, n;
-  unsigned mask;
-  __device__ __forceinline__ Lanes64(int shift) {
-    n = 1 << shift;
-    const int lane = threadIdx.x & 31;
-    sub = lane & (n - 1);
-    mask = (n == 32 ? ~0u : (1u << n) - 1u) << (lane - sub);
-  }
-  __device__ __forceinline__ double sum(double v) const {
-    for (int o = 1; o < n; o <<= 1) v += __shfl_xor_sync(mask, v, o);
-    return v;
-  }
-};
-
 // A partner's data (m: the array given, V_b or m_b), read one pair ahead, and
 // its index two ahead, as the mixed passes do
 template <int DIM>
@@ -331,21 +282,6 @@ struct Cursor64 {
     return b;
   }
 };
-
-// q < 1/2 for q >= 0, from the bits
-__device__ __forceinline__ bool below_half(double q) { return __double2hiint(q) < 0x3fe00000; }
-
-// (h^(D+1) / 6 sigma) dW/dr at q = r/h: q (3q - 2), or -(1 - q)^2 from q = 1/2
-__device__ __forceinline__ double slope64(double q) {
-  const bool in = below_half(q);
-  const double a1 = in ? 1.0 : -1.0, b1 = in ? 0.0 : 1.0, c1 = in ? 3.0 : 1.0, d1 = in ? -2.0 : -1.0;
-  return fma(a1, q, b1) * fma(c1, q, d1);
-}
-// (h^D / sigma) W: 1 + 6 q^2 (q - 1), or 2 (1 - q)^3
-__device__ __forceinline__ double value64(double q) {
-  const double t = below_half(q) ? q : 1.0 - q, t2 = t * t;
-  return below_half(q) ? fma(6.0 * t2, t - 1.0, 1.0) : 2.0 * t2 * t;
-}
 
 // ---------------------------------------------------------------------------
 // Density by kernel sum (Eq. density_by_kernel_sum) including m_a W(0; h_a).
@@ -571,10 +507,10 @@ __device__ __forceinline__ void pairs_A64(const RhsArgs &A, int64_t a, const Lan
 // ---------------------------------------------------------------------------
 // Pass A + per-particle update
 // ---------------------------------------------------------------------------
-// KEEP_SUMS (mixed, for the adjoint): also store the pair sums in A.sums,
-// rows of stride ld: 0 the continuity sum sum_b V_b (v_a - v_b).grad W (code
-// units 1/T), 1..6 the lower triangle of L (00, 10, 11, 20, 21, 22), 7..15 G
-// row by row (1/T).
+// KEEP_SUMS (for the adjoint): also store the pair sums in A.sums (mixed, code
+// units) or A.sums64, rows of stride ld: 0 the continuity sum sum_b V_b (v_a -
+// v_b).grad W (1/T), 1..6 the lower triangle of L (00, 10, 11, 20, 21, 22),
+// 7..15 G row by row (1/T).
 // AS = false: no artificial stress, the only user of the principal frame's
 // axes, so only the principal values are formed (for the damage strain).  The
 // mixed form is instantiated with AS alone, where the parameter decides: its
@@ -833,8 +769,10 @@ __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
   }
   if (A.nact) A.nact[a] = nact;
   if (A.nnb) A.nnb[a] = cnt;
-  if constexpr (MIXED && KEEP_SUMS) {
-    float *o = A.sums;
+  if constexpr (KEEP_SUMS) {
+    R *o;
+    if constexpr (MIXED) o = A.sums;
+    else o = A.sums64;
     const int64_t ld = A.ld;
     o[a] = drho.value();
     for (int i = 0; i < dim; ++i)
@@ -847,19 +785,6 @@ __global__ void SPH_PASSA_BOUNDS k_passA(RhsArgs A) {
 // ---------------------------------------------------------------------------
 // Pass B: momentum and energy
 // ---------------------------------------------------------------------------
-template <class R>
-__device__ __forceinline__ void sym_mv(int dim, const R t[6], const R g[3], R out[3]) {
-  if (dim == 3) {
-    out[0] = t[0] * g[0] + t[3] * g[1] + t[4] * g[2];
-    out[1] = t[3] * g[0] + t[1] * g[1] + t[5] * g[2];
-    out[2] = t[4] * g[0] + t[5] * g[1] + t[2] * g[2];
-  } else {
-    out[0] = t[0] * g[0] + t[2] * g[1];
-    out[1] = t[2] * g[0] + t[1] * g[1];
-    out[2] = R(0);
-  }
-}
-
 template <bool MIXED>
 __device__ __forceinline__ void load_T(const RhsArgs &A, int64_t b, int ns,
                                        typename std::conditional<MIXED, float, double>::type t[6],
@@ -1088,7 +1013,7 @@ __global__ void k_repack_rho(const double *__restrict__ rho, const double *__res
 }
 
 void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &p, const sph_derivs &out,
-                cudaStream_t st, float *sums) {
+                cudaStream_t st, bool adjoint) {
   const int64_t n = s->n;
   if (n == 0) return;
   RhsArgs A;
@@ -1137,18 +1062,10 @@ void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &
   A.prm = p;
   A.err = c->d_err;
   const bool mixed = p.precision == SPH_MIXED;
-  A.sums = mixed ? sums : nullptr;
-  // FP64 passes are bound by each SM's FP64 unit, so what counts for a small n
-  // is that the warps spread evenly over the SMs: one-warp blocks while that
-  // leaves fewer than eight 128-thread blocks per SM.
-  const int T = !mixed && nblk(n, 128) < 8 * c->num_sms ? 32 : c->tune.pass_threads;
-  // With fewer than kLaneWarps warps per SM even that leaves the unit idle
-  // between dependent operations: 2, 4 or 8 lanes then share a particle's
-  // list, and the constitutive update is repeated on each.  Against one lane,
-  // at thresholds of 2, 4 and 8 warps: rings at 4.4k (ten steps) 6.90 -> 5.67,
-  // 5.79, 5.80 ms; a right-hand side at 8k 902 -> 815, 804, 920 us and at 27k
-  // 1078 -> 1080, 1078, 1125 us; RK3 at 14k 3.18 -> 3.18, 2.96, 3.25 ms.
-  while (!mixed && A.lane_shift < 3 && (n << A.lane_shift) < (int64_t)32 * kLaneWarps * c->num_sms) ++A.lane_shift;
+  A.sums = c->adj_sums;
+  A.sums64 = c->adj_inter;
+  const int T = mixed ? c->tune.pass_threads : threads64(n, c->num_sms, c->tune.pass_threads);
+  A.lane_shift = mixed ? 0 : lanes64_shift(n, c->num_sms);
   const int64_t nt = n << A.lane_shift;  // threads of a pass
   int pr = -1;
   const bool d3 = s->dim == 3;
@@ -1167,9 +1084,12 @@ void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &
   }
   pr = prof_begin(c, st, PH_PASSA);
   const bool as = p.eps_s > 0.0;
-  if (mixed && A.sums) {  // the adjoint's forward
-    if (d3) k_passA<true, true, 3, true><<<nblk(n, T), T, 0, st>>>(A);
-    else k_passA<true, true, 2, true><<<nblk(n, T), T, 0, st>>>(A);
+  if (adjoint) {  // pass A alone, keeping its sums
+    const int g = nblk(nt, T);
+    if (mixed && d3) k_passA<true, true, 3, true><<<g, T, 0, st>>>(A);
+    else if (mixed) k_passA<true, true, 2, true><<<g, T, 0, st>>>(A);
+    else if (d3) k_passA<false, false, 3, true><<<g, T, 0, st>>>(A);
+    else k_passA<false, false, 2, true><<<g, T, 0, st>>>(A);
     ++sph::g_launches;
   } else if (mixed) {
     SPH_LAUNCH(k_passA, true, true);
@@ -1178,6 +1098,7 @@ void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &
     else SPH_LAUNCH(k_passA, false, false);
   }
   prof_end(c, st, pr);
+  if (adjoint) return;
   pr = prof_begin(c, st, PH_PASSB);
   if (mixed) {
     if (as) SPH_LAUNCH(k_passB, true, true);

@@ -365,10 +365,11 @@ void refine_partners(sph_ctx *c, const sph_state *s, const unsigned long long *m
 void adapt_h(sph_ctx *c, sph_state *s, double n_des, int tol, int max_iter, int32_t *flags, cudaStream_t st);
 void partners_to_csr(sph_ctx *c, const sph_state *s, int64_t *off, int32_t *idx, int64_t cap, cudaStream_t st);
 // rhs.cu
-// sums: NULL, or (mixed) where pass A also stores its pair sums for the
-// adjoint (16 * cap_n floats, the layout of k_passA's KEEP_SUMS form)
+// adjoint: only pass A (the reverse needs neither dv/dt nor du/dt), which also
+// stores its pair sums, in c->adj_sums (mixed) or the first 16 rows of
+// c->adj_inter (FP64), in the layout of k_passA's KEEP_SUMS form
 void rhs_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &p, const sph_derivs &out,
-                cudaStream_t st, float *sums = nullptr);
+                cudaStream_t st, bool adjoint = false);
 // gravity.cu
 // reuse: the tree was built at earlier positions (pseudo-particles reused)
 void gravity_walk(sph_ctx *c, const sph_state *s, const sph_params &p, double *ax, double *ay, double *az,

@@ -161,11 +161,12 @@ typedef struct sph_ctx sph_ctx;
  * sph_step_rk3 step, the step's first walk; across the steps that share a
  * tree under tree_reuse, the walk of the step that built it), which also
  * records each particle's candidates with (1 - 1/64) h_ab <= r_ab <
- * (1 + 1/64) h_ab (only those are tested again), as long as the
- * summed bound on the largest per-axis displacement of any particle since
- * that walk is at most h_a / (256 sqrt D) for every particle a and no
- * particle has more than 24 such candidates (else they walk); the lists are
- * the same either way.  1 walks the tree at every evaluation
+ * (1 + 1/64) h_ab (only those are tested again), for the particles whose
+ * own summed bound on the largest per-axis displacement since that walk is at
+ * most h_a / (128 sqrt D) and that have no more than 24 such candidates; the
+ * walk groups (up to 32 particles) of the others, and those whose partners
+ * they were or became, are walked; the lists are the same either way.  1 walks
+ * the tree at every evaluation
  * (Sect. 3.5.2 as printed).  iter_cap: 0 (default) bounds each tree walk
  * (partner search and gravity) by the number of tree nodes and each find of
  * the friends-of-friends union by 2^24 pointer steps; a positive value lowers

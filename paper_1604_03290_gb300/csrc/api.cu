@@ -146,7 +146,8 @@ sph_status sph_create(sph_ctx **out, int32_t dim, int64_t max_particles, int32_t
   c->sh_idx = ctx_alloc<int32_t>(c, (int64_t)kMaxShell * N, ok);
   c->sh_cnt = ctx_alloc<int32_t>(c, N, ok);
   c->sh_in = ctx_alloc<int32_t>(c, N, ok);
-  c->need_walk = ctx_alloc<int32_t>(c, 1, ok);
+  c->grp_of = ctx_alloc<int32_t>(c, N, ok);
+  c->redo = ctx_alloc<int32_t>(c, redo_words(T.cap_groups), ok);
   c->tick = ctx_alloc<int32_t>(c, 2, ok);
   c->csr_total = ctx_alloc<int64_t>(c, 1, ok);
   c->hflags = ctx_alloc<int32_t>(c, kMaxHIter + 3, ok);
@@ -189,6 +190,8 @@ sph_status sph_create(sph_ctx **out, int32_t dim, int64_t max_particles, int32_t
   S.dmove = ctx_alloc<unsigned long long>(c, 1, ok);
   S.dbuild = ctx_alloc<unsigned long long>(c, 1, ok);
   S.dgrow = ctx_alloc<unsigned long long>(c, 1, ok);
+  S.disp_s = ctx_alloc<float>(c, N, ok);
+  S.disp_q = ctx_alloc<float>(c, N, ok);
   S.dt = ctx_alloc<double>(c, ci, ok);
   S.gather = ctx_alloc<double>(c, N, ok);
   S.gather_i = ctx_alloc<int32_t>(c, N, ok);
@@ -353,16 +356,16 @@ static void timed_tree(sph_ctx *c, const sph_state *s, const sph_params &p, cuda
 // grow: displacement bound since the tree build (NULL: built at s);
 // greuse: gravity from the pseudo-particles of an earlier build;
 // shell: the walk also records the partner shells (for a later refine);
-// move: refine the partners from the lists and shells of the last walk, which
-// every particle has left by at most *move per axis (NULL: walk)
+// disp: refine the partners from the lists and shells of the last walk, which
+// every particle has left by at most its disp per axis (NULL: walk)
 static void partners_gravity_passes(sph_ctx *c, sph_state *s, const MatTable &mt, const sph_params &p,
                                     const sph_derivs &out, cudaStream_t st,
                                     const unsigned long long *grow = nullptr, bool greuse = false,
-                                    bool shell = false, const unsigned long long *move = nullptr) {
+                                    bool shell = false, const float *disp = nullptr) {
   int pr;
-  if (move) {
+  if (disp) {
     pr = prof_begin(c, st, PH_REFINE);
-    refine_partners(c, s, move, grow, st);
+    refine_partners(c, s, disp, grow, st);
     prof_end(c, st, pr);
     std::swap(c->nb_idx, c->nb_alt);  // the passes read the refined lists
     std::swap(c->nb_cnt, c->nb_cnt_alt);
@@ -377,7 +380,7 @@ static void partners_gravity_passes(sph_ctx *c, sph_state *s, const MatTable &mt
     prof_end(c, st, pr);
   }
   rhs_passes(c, s, mt, p, out, st);
-  if (move) {  // the walk's lists, counts and shells stay for the next refine
+  if (disp) {  // the walk's lists, counts and shells stay for the next refine
     std::swap(c->nb_idx, c->nb_alt);
     std::swap(c->nb_cnt, c->nb_cnt_alt);
   }
@@ -677,13 +680,15 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
       // the lists and shells of the build step's walk stay in place: while
       // the displacement since that walk is within the shell's bound, the
       // partners are refined from them (else a walk over the widened boxes)
-      partners_gravity_passes(c, s, mt, *p, d[0], st, B.dbuild, p->gravity, false, refine ? B.dbuild : nullptr);
+      partners_gravity_passes(c, s, mt, *p, d[0], st, B.dbuild, p->gravity, false, refine ? B.disp_s : nullptr);
     }
     pr = prof_begin(c, st, PH_INTEGRATE);
     timestep_reduce(c, s, *p, d[0], st);
     if (reuse_pred) cudaMemsetAsync(B.dmove, 0, sizeof(unsigned long long), st);
     // on a kept tree the update also writes the predicted state's FP32 views
-    pc_update(c, s, &q, d[0], 0.5, mt, *p, st, reuse_pred ? B.dmove : nullptr, reuse_pred && fuse);
+    Moved moved;
+    if (reuse_pred) moved = Moved{B.dmove, build ? nullptr : B.disp_s, B.disp_q};
+    pc_update(c, s, &q, d[0], 0.5, mt, *p, st, moved, reuse_pred && fuse);
     if (reuse_pred && !build) bound_add(B.dgrow, B.dbuild, B.dmove, st);
     prof_end(c, st, pr);
     if (reuse_pred) {
@@ -695,7 +700,7 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
       // displacement since the walk whose lists are refined: this step's walk
       // at a build, the build step's walk otherwise
       const unsigned long long *since = build ? B.dmove : B.dgrow;
-      partners_gravity_passes(c, &q, mt, *p, d[1], st, since, p->gravity, false, refine ? since : nullptr);
+      partners_gravity_passes(c, &q, mt, *p, d[1], st, since, p->gravity, false, refine ? B.disp_q : nullptr);
     } else {
       rhs_all(c, &q, mt, *p, d[1], st);
     }
@@ -705,7 +710,7 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
       // views of the new state for the next step of this call, if it keeps the tree
       const bool keep = fuse && it + 1 < nsteps && !vh && (age + 1) % R != 0;
       cudaMemsetAsync(B.dmove, 0, sizeof(unsigned long long), st);
-      pc_update(c, s, s, d[1], 1.0, mt, *p, st, B.dmove, keep);
+      pc_update(c, s, s, d[1], 1.0, mt, *p, st, Moved{B.dmove, build ? nullptr : B.disp_s, B.disp_s}, keep);
       bound_add(B.dbuild, B.dbuild, B.dmove, st);
       age = (age + 1) % R;
       packed = keep;
@@ -762,13 +767,13 @@ sph_status sph_step_rk3(sph_ctx *c, sph_state *s, const sph_material *mats, int3
   auto stage = [&](const sph_derivs *const *k, const double *coef, int nd, sph_derivs &out) {
     int pr = prof_begin(c, st, PH_INTEGRATE);
     if (reuse) cudaMemsetAsync(B.dmove, 0, sizeof(unsigned long long), st);
-    combine_update(c, s, &q, k, coef, nd, nullptr, mt, *p, st, reuse ? B.dmove : nullptr);
+    combine_update(c, s, &q, k, coef, nd, nullptr, mt, *p, st, reuse ? Moved{B.dmove, nullptr, B.disp_q} : Moved());
     prof_end(c, st, pr);
     if (reuse) {
       pr = prof_begin(c, st, PH_TREE);
       pack_f32(c, &q, st);
       prof_end(c, st, pr);
-      partners_gravity_passes(c, &q, mt, *p, out, st, B.dmove, false, false, refine ? B.dmove : nullptr);
+      partners_gravity_passes(c, &q, mt, *p, out, st, B.dmove, false, false, refine ? B.disp_q : nullptr);
     } else {
       rhs_all(c, &q, mt, *p, out, st);
     }

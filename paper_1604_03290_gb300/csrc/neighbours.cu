@@ -151,8 +151,38 @@ __device__ __forceinline__ int32_t sort_ranges(WalkScratch &W, int nr, int lane)
   return total;
 }
 
-// OWN_H = false: interaction partners (h_ab), lists and counts, skipped when
-// the flag `done` is given and is 0 (it is then a run-if flag).  OWN_H = true:
+// Groups a refine queues for walking again: two queues (phases), a bit per
+// group in each so that a group is queued once.  Words: the two counts, then
+// the bits; the queues lie in Tree::arrived, free after a build.
+struct Redo {
+  int32_t *w;
+  int32_t *q;
+  int64_t words, cap;  // bit words and entries per queue
+  __device__ __forceinline__ int32_t *queue(int phase) const { return q + (phase - 1) * cap; }
+  __device__ __forceinline__ int count(int phase) const { return w[phase - 1]; }
+  __device__ __forceinline__ int32_t *bits(int phase, int g) const { return w + 4 + (phase - 1) * words + (g >> 5); }
+  __device__ __forceinline__ bool queued(int phase, int g) const {
+    return (*(const volatile int32_t *)bits(phase, g) >> (g & 31)) & 1;
+  }
+  // queue group g, unless it is `own` (or for phase 2 already in phase 1)
+  __device__ __forceinline__ void add(int phase, int g, int own) const {
+    if (g == own || queued(phase, g) || (phase == 2 && queued(1, g))) return;
+    const int32_t bit = (int32_t)(1u << (g & 31));
+    if (atomicOr(bits(phase, g), bit) & bit) return;
+    queue(phase)[atomicAdd(&w[phase - 1], 1)] = g;
+  }
+};
+int64_t redo_words(int64_t cap_groups) { return 4 + 2 * ((cap_groups + 31) / 32); }
+
+// A particle whose own displacement bound since the walk allows the refine
+// (see k_partners_refine): 2 sqrt(D) disp <= kSkin h, in code units; the FP32
+// rounding of h (2^-24) and of the products is in the factor.
+__device__ __forceinline__ bool slow_particle(float disp, float h, int dim) {
+  const float f = dim == 3 ? 2.0f * 1.7320508f * (1.0f + 1e-5f) : 2.0f * 1.4142136f * (1.0f + 1e-5f);
+  return __fmul_ru(f, disp) <= __fmul_rd(kSkinF, h);
+}
+
+// OWN_H = false: interaction partners (h_ab), lists and counts.  OWN_H = true:
 // only the number of particles within each particle's own h (the current h of
 // the state, not the packed one), plus the count of particles whose number
 // lies farther than tol from n_des (*unconverged); the walk is skipped once
@@ -160,7 +190,15 @@ __device__ __forceinline__ int32_t sort_ranges(WalkScratch &W, int nr, int lane)
 // Warps draw their groups from a ticket counter (tick[0]): a fixed stride left
 // half the warps a second group and the others none at 263k particles.  The
 // last warp to find no group left (tick[1] counts them) sets both back to 0.
-template <bool OWN_H, bool SHELL>
+// SELECT (after a refine): only the groups queued for walking again, all their
+// particles.  Phase 1 takes the first queue (groups of particles that could
+// not refine their lists) and, of particles that moved too far, queues the
+// groups of the partners they had and of those they have now; phase 2 takes
+// these where phase 1 has not walked them.  With more than half of the groups
+// in the first queue, or few enough that each warp takes one (the walk then
+// lasts as long as its slowest group), phase 1 walks them all and phase 2
+// none.  SHELL records each particle's group.
+template <bool OWN_H, bool SHELL, bool SELECT>
 __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *__restrict__ x,
                                            const double *__restrict__ y, const double *__restrict__ z,
                                            const double *__restrict__ h, int dim, int kmax,
@@ -169,12 +207,17 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
                                            const Units *__restrict__ U, const int32_t *__restrict__ done,
                                            int32_t *__restrict__ unconverged, double n_des, int tol,
                                            int32_t *__restrict__ sh_idx, int32_t *__restrict__ sh_cnt,
-                                           int32_t *__restrict__ sh_in, int32_t *tick, unsigned long long *ctr) {
-  static_assert(!(OWN_H && SHELL), "shells are partner candidates");
+                                           int32_t *__restrict__ sh_in, int32_t *tick, int32_t *grp_of, Redo R,
+                                           int phase, const float *disp, const int32_t *old_idx,
+                                           const int32_t *old_cnt, unsigned long long *ctr) {
+  static_assert(!(OWN_H && SHELL) && !(SELECT && (OWN_H || SHELL)), "shells are partner candidates");
   if constexpr (OWN_H) {
     if (*done) return;
-  } else {
-    if (done && *done == 0) return;  // done is run_if here
+  }
+  bool every = false;  // SELECT: every group after all
+  if constexpr (SELECT) {
+    every = 2 * R.count(1) > *T.ngroups || *T.ngroups <= (int)(gridDim.x * kNbWarps);
+    if (R.count(phase) == 0 || (phase == 2 && every)) return;
   }
   // the shell widens every test by the factor (1 + kSkin) of its radius
   const float wide = SHELL ? 1.0f + kSkinF : 1.0f;
@@ -182,7 +225,7 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
   WalkScratch &W = scratch[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
-  const int ngroups = *T.ngroups;
+  const int ngroups = SELECT && !every ? R.count(phase) : *T.ngroups;
   // The walk stops at nodes flagged in their box word (at most
   // max(leaf_size, walk_leaf) particles, or depth B; set by the tree build)
   // and culls their whole particle range: any stopping rule gives the same set.
@@ -197,10 +240,28 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
     if (lane == 0) g = atomicAdd(&tick[0], 1);
     g = __shfl_sync(0xffffffffu, g, 0);
     if (g >= ngroups) break;
+    if constexpr (SELECT)
+      if (!every) {
+        g = R.queue(phase)[g];
+        if (phase == 2 && R.queued(1, g)) continue;
+      }
     const int32_t s0 = T.grp_start[g], s1 = T.grp_end[g], inst = T.grp_inst[g];
     const int32_t slot = s0 + lane;
     const bool act = slot < s1;
     const int32_t a = act ? (T.perm_identity ? slot : T.perm[slot]) : -1;
+    if constexpr (SHELL)
+      if (act) grp_of[a] = g;
+    // this lane's particle moved too far: its partners' groups are walked too
+    const bool far = SELECT && act && !every && phase == 1 && !slow_particle(disp[a], pk.px(a).w, dim);
+    if (far) {
+      int last = g;  // neighbouring entries mostly share a group
+      const int k1 = old_cnt[a];
+      for (int k = 0; k < k1; ++k) {
+        const int e = grp_of[old_idx[(int64_t)k * ld + a]];
+        if (e != last) R.add(2, e, g);
+        last = e;
+      }
+    }
     float4 P = act ? pk.px(a) : make_float4(0.f, 0.f, 0.f, 0.f);
     float4 Q = act ? pk.pxl(a) : make_float4(0.f, 0.f, 0.f, 0.f);
     // reference point: lane 0's position
@@ -295,6 +356,8 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
                 if (cnt < kmax) *out = bs[u];
                 out += ld;
               }
+              if constexpr (SELECT)
+                if (far) R.add(2, grp_of[bs[u]], g);
               ++cnt;
             }
             if constexpr (SHELL) {
@@ -480,19 +543,26 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
 }
 
 // Partners at moved positions from the lists and shells of an earlier walk
-// (the Verlet-list idea).  When every particle moved by at most `move` per
-// axis since that walk, a pair's distance changed by at most 2 sqrt(D) move;
-// with 4 sqrt(D) move <= kSkin h_a that is at most kSkin h_ab (h_ab >= h_a / 2).
-// So a partner of the walk closer than (1 - kSkin) h_ab is still one, a
-// non-partner farther than (1 + kSkin) h_ab is still none, and only the shell
-// between the two can change.  The old list and the shell are both ascending,
-// and the shell's partners are also in the list: merged, the candidates are
-// visited in ascending order, the list's members outside the shell are kept
-// as they are (no gather), and each shell member is decided by the walk's
-// predicate (FP32 outside the band, the FP64 definition inside it), so the new
-// list equals that of a walk at the new positions bit for bit.  A particle
-// whose bound does not hold, or whose shell overflowed, sets *need_walk
-// instead, and a walk follows.
+// (the Verlet-list idea).  A particle is slow when 2 sqrt(D) times the bound
+// of its own largest per-axis displacement since that walk is at most kSkin
+// h_a.  The distance of two slow particles changed by at most sqrt(D) (move_a
+// + move_b) <= kSkin h_ab: a partner of the walk closer than (1 - kSkin) h_ab
+// is still one, a non-partner farther than (1 + kSkin) h_ab is still none, and
+// only the shell between the two can change.  The old list and the shell are
+// both ascending, and the shell's partners are also in the list: merged, the
+// candidates are visited in ascending order, the list's members outside the
+// shell are kept as they are (no gather), and each shell member is decided by
+// the walk's predicate (FP32 outside the band, the FP64 definition inside it),
+// so the new list equals that of a walk at the new positions bit for bit.
+// The groups of fast particles (and of those whose shell overflowed) are
+// walked again, and so are those of every slow one whose status with a fast
+// one may differ from what its list and shell say: the fast one's old
+// partners and its new ones, both queued by the walk of its group (unless that
+// takes every group anyway).  A projectile's
+// few fast particles so cost a walk of its surroundings; taking the largest
+// displacement of all particles for each, every evaluation of a batch of
+// impacts walked every group (64 impacts, 8 evaluations: 3.6 of 12.6 ms, now
+// 1.6 of 10.7).
 constexpr int kRefineThreads = 128;
 __global__ void __launch_bounds__(kRefineThreads)
     k_partners_refine(PackedF32 pk, const double *__restrict__ x, const double *__restrict__ y,
@@ -500,17 +570,17 @@ __global__ void __launch_bounds__(kRefineThreads)
                       int kmax, const int32_t *__restrict__ old_idx, const int32_t *__restrict__ old_cnt,
                       const int32_t *__restrict__ sh_idx, const int32_t *__restrict__ sh_cnt,
                       const int32_t *__restrict__ sh_in, int32_t *__restrict__ new_idx,
-                      int32_t *__restrict__ new_cnt,
-                      const unsigned long long *__restrict__ move, int32_t *__restrict__ need_walk, int32_t *err) {
+                      int32_t *__restrict__ new_cnt, const float *__restrict__ disp,
+                      const int32_t *__restrict__ grp_of, Redo R, int32_t *err) {
   // the shell of each thread's particle, staged for the merge
   __shared__ int32_t shs[kMaxShell][kRefineThreads];
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= n) return;
   const int ns = sh_cnt[a];
-  const double sqd = dim == 3 ? 1.7320508075688772 : 1.4142135623730951;  // sqrt(D)
-  const double bound = __dmul_ru(__dmul_ru(4.0 * sqd, bitsd(*move)), 1.0 + 1e-6);
-  if (ns < 0 || !(bound <= __dmul_rd(kSkin, h[a]))) {
-    *need_walk = 1;
+  const bool slow = slow_particle(disp[a], pk.px(a).w, dim);
+  if (ns < 0 || !slow) {
+    const int g = grp_of[a];  // one lane of each group queues it
+    if ((threadIdx.x & 31) == (unsigned)(__ffs(__match_any_sync(__activemask(), g)) - 1)) R.add(1, g, -1);
     return;
   }
   const int t = threadIdx.x;
@@ -586,35 +656,36 @@ static int walk_grid(const sph_ctx *c, int64_t n) {
   return std::min(c->num_sms * c->tune.walk_blocks_per_sm * (4 / kNbWarps), nblk(n, 16 * kNbWarps));
 }
 
-static void walk(sph_ctx *c, const sph_state *s, cudaStream_t st, const unsigned long long *grow, int32_t *idx,
-                 int32_t *cnt, bool shell, const int32_t *run_if) {
-  const int blocks = walk_grid(c, s->n);
-  if (shell)
-    k_partners<false, true><<<blocks, kNbWarps * 32, 0, st>>>(
-        c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h, s->dim, c->kmax, idx, cnt, c->cap_n, c->d_err, grow,
-        c->units, run_if, nullptr, 0.0, 0, c->sh_idx, c->sh_cnt, c->sh_in, c->tick, counters(c));
-  else
-    k_partners<false, false><<<blocks, kNbWarps * 32, 0, st>>>(
-        c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h, s->dim, c->kmax, idx, cnt, c->cap_n, c->d_err, grow,
-        c->units, run_if, nullptr, 0.0, 0, nullptr, nullptr, nullptr, c->tick, counters(c));
+void find_partners(sph_ctx *c, const sph_state *s, cudaStream_t st, const unsigned long long *grow, bool shell) {
+  if (s->n == 0) return;
+  const bool sh = shell && c->sh_idx != nullptr;
+  const auto kern = sh ? k_partners<false, true, false> : k_partners<false, false, false>;
+  kern<<<walk_grid(c, s->n), kNbWarps * 32, 0, st>>>(
+      c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h, s->dim, c->kmax, c->nb_idx, c->nb_cnt, c->cap_n, c->d_err, grow,
+      c->units, nullptr, nullptr, 0.0, 0, c->sh_idx, c->sh_cnt, c->sh_in, c->tick, c->grp_of, Redo(), 0, nullptr,
+      nullptr, nullptr, counters(c));
   ++sph::g_launches;
 }
 
-void find_partners(sph_ctx *c, const sph_state *s, cudaStream_t st, const unsigned long long *grow, bool shell) {
-  if (s->n == 0) return;
-  walk(c, s, st, grow, c->nb_idx, c->nb_cnt, shell && c->sh_idx != nullptr, nullptr);
-}
-
-void refine_partners(sph_ctx *c, const sph_state *s, const unsigned long long *move, const unsigned long long *grow,
+void refine_partners(sph_ctx *c, const sph_state *s, const float *disp, const unsigned long long *grow,
                      cudaStream_t st) {
   const int64_t n = s->n;
   if (n == 0) return;
-  cudaMemsetAsync(c->need_walk, 0, sizeof(int32_t), st);
-  { k_partners_refine<<<nblk(n, kRefineThreads), kRefineThreads, 0, st>>>(c->pk, s->x[0], s->x[1], s->x[2], s->h, s->dim, n, c->cap_n,
-                                                   c->kmax, c->nb_idx, c->nb_cnt, c->sh_idx, c->sh_cnt, c->sh_in, c->nb_alt,
-                                                   c->nb_cnt_alt, move, c->need_walk, c->d_err); ++sph::g_launches; }
-  // returns at once unless a particle set the flag
-  walk(c, s, st, grow, c->nb_alt, c->nb_cnt_alt, false, c->need_walk);
+  // groups hold at least one particle each, so the queues fit n entries
+  const Redo R{c->redo, c->tree.arrived, (c->tree.cap_groups + 31) / 32, c->tree.cap_nodes / 2};
+  cudaMemsetAsync(c->redo, 0, sizeof(int32_t) * redo_words(c->tree.cap_groups), st);
+  { k_partners_refine<<<nblk(n, kRefineThreads), kRefineThreads, 0, st>>>(
+        c->pk, s->x[0], s->x[1], s->x[2], s->h, s->dim, n, c->cap_n, c->kmax, c->nb_idx, c->nb_cnt, c->sh_idx,
+        c->sh_cnt, c->sh_in, c->nb_alt, c->nb_cnt_alt, disp, c->grp_of, R, c->d_err); ++sph::g_launches; }
+  // both return at once unless a group was queued; the resident blocks only, as they usually do
+  const int blocks = std::min(walk_grid(c, n), c->num_sms * SPH_WALK_MIN_BLOCKS);
+  for (int phase = 1; phase <= 2; ++phase) {
+    k_partners<false, false, true><<<blocks, kNbWarps * 32, 0, st>>>(
+        c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h, s->dim, c->kmax, c->nb_alt, c->nb_cnt_alt, c->cap_n, c->d_err,
+        grow, c->units, nullptr, nullptr, 0.0, 0, nullptr, nullptr, nullptr, c->tick, c->grp_of, R, phase, disp,
+        c->nb_idx, c->nb_cnt, counters(c));
+    ++sph::g_launches;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -650,10 +721,10 @@ void adapt_h(sph_ctx *c, sph_state *s, double n_des, int tol, int max_iter, int3
   if (n == 0) return;
   const int blocks = walk_grid(c, n);
   for (int i = 0; i <= max_iter; ++i) {
-    { k_partners<true, false><<<blocks, kNbWarps * 32, 0, st>>>(c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h,
+    { k_partners<true, false, false><<<blocks, kNbWarps * 32, 0, st>>>(c->tree, c->pk, s->x[0], s->x[1], s->x[2], s->h,
                                                                s->dim, c->kmax, c->nb_idx, c->nb_cnt, c->cap_n,
                                                                c->d_err, nullptr, c->units, flags, flags + 2 + i,
-                                                               n_des, tol, nullptr, nullptr, nullptr, c->tick, nullptr); ++sph::g_launches; }
+                                                               n_des, tol, nullptr, nullptr, nullptr, c->tick, nullptr, Redo(), 0, nullptr, nullptr, nullptr, nullptr); ++sph::g_launches; }
     if (i == max_iter) break;
     { k_h_update<<<nblk(n, 256), 256, 0, st>>>(s->h, c->nb_cnt, n, s->dim, n_des, flags + 2 + i, flags,
                                              flags + 1); ++sph::g_launches; }

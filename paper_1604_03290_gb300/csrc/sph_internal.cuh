@@ -143,6 +143,8 @@ struct StepBufs {
   unsigned long long *dmove;   // bits of the predictor's largest per-axis displacement
   unsigned long long *dbuild;  // bits of a bound on every displacement since the last tree build
   unsigned long long *dgrow;   // dbuild + dmove
+  float *disp_s, *disp_q;      // per particle, code units: bounds of the displacement of the state and of
+                               // the state being evaluated since the walk whose lists are refined
   double *dt;                  // per instance
   double *gather;              // reorder scratch (n doubles)
   int32_t *gather_i;
@@ -191,7 +193,8 @@ struct sph_ctx {
   int32_t *sh_cnt;      // their number, -1 when more than kMaxShell
   int32_t *sh_in;       // bit j set when shell entry j was a partner at the walk
   int32_t *tick;        // group tickets of the partner walk: next group, warps done (both 0 between walks)
-  int32_t *need_walk;   // device flag: some particle could not refine its list
+  int32_t *grp_of;      // group of each particle at the walk that recorded the shells
+  int32_t *redo;        // groups a refine has to walk again (Redo, neighbours.cu)
   int64_t *csr_total;   // device scalar for sph_neighbours
   int32_t *hflags;      // variable-h iteration: done, updates, off-target count per pass
   // pass A -> pass B per-particle data
@@ -345,6 +348,7 @@ void prof_end(sph_ctx *c, cudaStream_t st, int idx);
 // writes those of the state in its new order)
 void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cudaStream_t st, bool pack = true);
 int64_t look_words(int64_t max_particles, int64_t cap_nodes);
+int64_t redo_words(int64_t cap_groups);  // size of sph_ctx::redo
 void tree_reorder_state(sph_ctx *c, sph_state *s, cudaStream_t st);
 void pack_f32(sph_ctx *c, const sph_state *s, cudaStream_t st);
 // neighbours.cu
@@ -354,12 +358,13 @@ void pack_f32(sph_ctx *c, const sph_state *s, cudaStream_t st);
 void find_partners(sph_ctx *c, const sph_state *s, cudaStream_t st, const unsigned long long *grow = nullptr,
                    bool shell = false);
 // Partners of s into c->nb_alt / nb_cnt_alt from the lists and shells of the
-// last walk (nb_idx, nb_cnt, sh_idx, sh_cnt; left unchanged), whose positions
-// every particle of s left by at most `move` per axis (device bits); a walk
-// with boxes grown by `grow` recomputes every list when some particle cannot
-// refine its own.  The caller swaps the two list buffers (and the two count
-// arrays) for the passes that read the result.
-void refine_partners(sph_ctx *c, const sph_state *s, const unsigned long long *move, const unsigned long long *grow,
+// last walk (nb_idx, nb_cnt, sh_idx, sh_cnt; left unchanged), which particle a
+// of s left by at most disp[a] per axis (code units) and none by more than
+// `grow` (SI, bits): particles that cannot refine their own list, and those
+// whose partners may have changed because another moved too far, are walked
+// again.  The caller swaps the two list buffers (and the two count arrays) for
+// the passes that read the result.
+void refine_partners(sph_ctx *c, const sph_state *s, const float *disp, const unsigned long long *grow,
                      cudaStream_t st);
 // variable smoothing length iteration; flags: device int32[max_iter + 3]
 void adapt_h(sph_ctx *c, sph_state *s, double n_des, int tol, int max_iter, int32_t *flags, cudaStream_t st);
@@ -390,18 +395,25 @@ void fragments_fof(sph_ctx *c, const sph_state *s, const double *h0, double b, d
                    int64_t *nfrag, cudaStream_t st);
 // step.cu
 void timestep_reduce(sph_ctx *c, const sph_state *s, const sph_params &p, const sph_derivs &d, cudaStream_t st);
-// dmove (device, may be NULL): receives the bits of max over particles and
-// axes of |out.x - base.x|; non-finite output or rho <= 0 then raises the
-// non-finite error bit, as a tree build over `out` would.  pack: also write
-// the FP32 views of out (c->pk, in the units and instance corners of the
-// current tree), as pack_f32 would.
+// Displacement bounds an update reports (device; all NULL: none): the bits of
+// max over particles and axes of |out.x - base.x|, and each particle's own
+// largest per-axis bound in code units, added to `in` (NULL: zero).  With max,
+// non-finite output or rho <= 0 raises the non-finite error bit, as a tree
+// build over `out` would.
+struct Moved {
+  unsigned long long *max = nullptr;
+  const float *in = nullptr;
+  float *out = nullptr;
+};
+// pack: also write the FP32 views of out (c->pk, in the units and instance
+// corners of the current tree), as pack_f32 would.
 void pc_update(sph_ctx *c, const sph_state *base, sph_state *out, const sph_derivs &d, double frac,
-               const MatTable &mt, const sph_params &p, cudaStream_t st, unsigned long long *dmove = nullptr,
+               const MatTable &mt, const sph_params &p, cudaStream_t st, const Moved &moved = Moved(),
                bool pack = false);
 // out = base + dt (coef_0 d_0 + ...), nd <= 3 sets, where mask[inst] (NULL: all)
 void combine_update(sph_ctx *c, const sph_state *base, sph_state *out, const sph_derivs *const *d, const double *coef,
                     int nd, const int32_t *mask, const MatTable &mt, const sph_params &p, cudaStream_t st,
-                    unsigned long long *dmove = nullptr, bool pack = false);
+                    const Moved &moved = Moved(), bool pack = false);
 // embedded Runge-Kutta: step size of the attempt (c->st.dt), error and control
 void rk_set_dt(sph_ctx *c, const sph_state *s, double *dt_io, cudaStream_t st);
 // *out = a + b rounded up (bits of non-negative doubles)

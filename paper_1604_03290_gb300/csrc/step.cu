@@ -338,6 +338,9 @@ struct PcArgs {
   MatTable mt;
   int density_sum;
   unsigned long long *dmove;  // NULL, or max |out.x - base.x| (bits of a non-negative double)
+  // NULL, or each particle's own bound, in code units: disp_out = disp_in (NULL: 0) + |out.x - base.x|
+  const float *disp_in;
+  float *disp_out;
   int32_t *err;
   // pack: also write the FP32 views of out (those k_pack would write)
   int pack;
@@ -422,6 +425,10 @@ __device__ __forceinline__ unsigned long long pc_particle(const PcArgs &A, int64
   if (A.dmove) {
     bad |= !positive_finite_bits(rho_o);
     if (bad) raise_err(A.err, ERR_NONFINITE);
+  }
+  if (A.disp_out) {
+    const float m = to_f32_dir_scaled(bitsd(mv), pow2_exp(A.U->invL), true, A.U->invL);
+    A.disp_out[a] = __fadd_ru(A.disp_in ? A.disp_in[a] : 0.f, m);
   }
   if (A.pack)
     pack_particle(A.pk, a, A.dim, xo[0], xo[1], xo[2], vo[0], vo[1], vo[2], A.h[a], A.m[a], rho_o, A.ilo + 3 * inst,
@@ -517,7 +524,7 @@ static DSet dset_of(const sph_derivs &d) {
 
 void combine_update(sph_ctx *c, const sph_state *base, sph_state *out, const sph_derivs *const *d, const double *coef,
                     int nd, const int32_t *mask, const MatTable &mt, const sph_params &p, cudaStream_t st,
-                    unsigned long long *dmove, bool pack) {
+                    const Moved &moved, bool pack) {
   if (base->n == 0) return;
   PcArgs A;
   memset(&A, 0, sizeof(A));
@@ -554,7 +561,10 @@ void combine_update(sph_ctx *c, const sph_state *base, sph_state *out, const sph
   A.dt = c->st.dt;
   A.mt = mt;
   A.density_sum = p.density_sum;
-  A.dmove = dmove;
+  A.dmove = moved.max;
+  A.disp_in = moved.in;
+  A.disp_out = moved.out;
+  A.U = c->units;
   A.err = c->d_err;
   A.pack = pack ? 1 : 0;
   if (pack) {
@@ -562,15 +572,14 @@ void combine_update(sph_ctx *c, const sph_state *base, sph_state *out, const sph
     A.ilo = c->tree.inst_lo;
     A.h = out->h;
     A.m = out->m;
-    A.U = c->units;
   }
   { k_pc<<<nblk(base->n, 256), 256, 0, st>>>(A); ++sph::g_launches; }
 }
 
 void pc_update(sph_ctx *c, const sph_state *base, sph_state *out, const sph_derivs &d, double frac,
-               const MatTable &mt, const sph_params &p, cudaStream_t st, unsigned long long *dmove, bool pack) {
+               const MatTable &mt, const sph_params &p, cudaStream_t st, const Moved &moved, bool pack) {
   const sph_derivs *dd[1] = {&d};
-  combine_update(c, base, out, dd, &frac, 1, nullptr, mt, p, st, dmove, pack);
+  combine_update(c, base, out, dd, &frac, 1, nullptr, mt, p, st, moved, pack);
 }
 
 // ---------------------------------------------------------------------------

@@ -436,13 +436,20 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
         __syncwarp();
         bool hit = false;
         int nc = 0;
-        int4 rec = make_int4(0, 0, 0, 0);
+        int4 rec = make_int4(0, 0, 0, 0), c0 = make_int4(-1, -1, -1, -1), c1 = c0;
         if (nd >= 0) {
           const float4 bl = __ldg(&T.fbox_lo[nd]), bh = __ldg(&T.fbox_hi[nd]);
           if (reached(bl, bh)) {
             hit = (__float_as_uint(bl.w) >> 31) != 0u;  // the walk stops here
-            if (hit) rec = __ldg(&T.nrec[nd]);
-            else nc = min(T.nchild[nd], 8);
+            if (hit) {
+              rec = __ldg(&T.nrec[nd]);
+            } else {
+              const int4 *ch = reinterpret_cast<const int4 *>(T.child) + 2 * (int64_t)nd;
+              c0 = __ldg(ch);
+              if (dim == 3) c1 = __ldg(ch + 1);
+              nc = (c0.x >= 0) + (c0.y >= 0) + (c0.z >= 0) + (c0.w >= 0) + (c1.x >= 0) + (c1.y >= 0) + (c1.z >= 0) +
+                   (c1.w >= 0);
+            }
           }
         }
         const unsigned hm = __ballot_sync(0xffffffffu, hit);
@@ -462,21 +469,12 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
           fits = false;
           break;
         }
-        const int4 *ch = reinterpret_cast<const int4 *>(T.child) + 2 * (int64_t)nd;
-        const int at = sp + incl - nc;
         if (nc > 0) {
-          const int4 c0 = ch[0];
-          const int32_t k[4] = {c0.x, c0.y, c0.z, c0.w};
+          int at = sp + incl - nc;
+          const int32_t k[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (j < nc) W.stack[at + j] = k[j];
-        }
-        if (nc > 4) {
-          const int4 c1 = ch[1];
-          const int32_t k[4] = {c1.x, c1.y, c1.z, c1.w};
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (4 + j < nc) W.stack[at + 4 + j] = k[j];
+          for (int j = 0; j < 8; ++j)
+            if (k[j] >= 0) W.stack[at++] = k[j];
         }
         sp += push;
         __syncwarp();

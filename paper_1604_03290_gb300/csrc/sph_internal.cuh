@@ -80,7 +80,7 @@ struct Tree {
   int packed_walk;     // fcom_lo.w holds the packed node word (cap_nodes <= kPackedSkip + 1)
   int32_t *nnodes;     // device scalar
   int32_t *first, *end, *skip, *parent, *nchild, *arrived, *level;
-  int32_t *child;      // up to 8 child ids per node, in arrival order
+  int32_t *child;      // child ids per node, a slot per octant (-1: none)
   int4 *nrec;          // (first, end, skip, level) per node, for the walks
   unsigned long long *cell;  // level prefix of the key (instance bits included)
   double *mass, *com;  // com: 3 * cap_nodes, component-major

@@ -98,6 +98,13 @@ struct GravArgs {
   const Units *U;
   int32_t *err;
   int share;  // FP64: 2^share lanes per particle
+  // A node whose cube holds the particle also holds its centre of mass, so r <=
+  // sqrt(D) s there; with D theta^2 < 1 (by a margin far above the rounding of
+  // either test) the opening criterion already rejects it and the containment
+  // test can be skipped: the accepted set is the same.  Decided on the host:
+  // formed in the kernel, the compiler evaluated the comparison again at every
+  // visit (an FP64 instruction each, 37 % of the FP64 unit).
+  int test_inside;
   int reuse;  // the tree was built at earlier positions: locate each particle anew
   unsigned long long *ctr;  // NULL, or the interaction counters
 };
@@ -161,11 +168,6 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
     const float s0f = PACKED ? to_f32_scaled(s0r, pow2_exp(A.U->invL), A.U->invL) : 0.f;
     const double th = A.theta;
     const float th2f = (float)(th * th);
-    // A node whose cube holds the particle also holds its centre of mass, so
-    // r <= sqrt(D) s there; with D theta^2 < 1 (by a margin far above the
-    // rounding of either test) the opening criterion already rejects it and
-    // the containment test can be skipped: the accepted set is the same.
-    const bool test_inside = (double)dim * th * th >= 0.99;
     GravSumF acc;
     int32_t skip_until = -1;
     const int32_t root = T.inst_root[inst];
@@ -194,7 +196,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
       }
       bool open = false, direct = false;
       if (act && nd >= skip_until) {
-        const bool inside = test_inside && (ka >> (dim * (B - lev))) == T.cell[nd];
+        const bool inside = A.test_inside && (ka >> (dim * (B - lev))) == T.cell[nd];
         bool accept = false;
         float mpf = 0.f;
         R d[3] = {R(0), R(0), R(0)}, r2 = R(0);
@@ -364,7 +366,7 @@ __global__ void __launch_bounds__(32, kGrav64Blocks) k_gravity64(GravArgs A) {
   const int64_t cap = T.cap_nodes;
   const double th = A.theta;
   const float th2f = (float)(th * th);
-  const bool test_inside = (double)DIM * th * th >= 0.99;  // see k_gravity
+  const bool test_inside = A.test_inside != 0;
   for (int g = blockIdx.x; g < ngroups; g += gridDim.x) {
     const int32_t s0 = chunks ? g * per : T.grp_start[g];
     const int32_t s1 = chunks ? (int32_t)(((int64_t)s0 + per < T.n) ? (int64_t)s0 + per : T.n) : T.grp_end[g];
@@ -500,6 +502,7 @@ void gravity_walk(sph_ctx *c, const sph_state *s, const sph_params &p, double *a
   A.U = c->units;
   A.err = c->d_err;
   A.reuse = reuse ? 1 : 0;
+  A.test_inside = (double)s->dim * p.theta * p.theta >= 0.99;
   A.ctr = counters(c);
   // One instance: a block per chunk, so that the hardware hands chunks out as
   // warps finish (a persistent grid gave each block every 4864th chunk: at 400k

@@ -12,7 +12,7 @@
 // partners' terms with respect to itself.  No atomics, deterministic order.
 //
 //   k_adj_passB   reverse of the momentum / energy pass -> x, v, T, c_s, rho
-//   k_adj_update  pass-A sums recomputed, reverse of the constitutive update
+//   k_adj_update  from the forward's pass-A sums, reverse of the constitutive update
 //                 (T = sigma/rho^2, damage-reduced stress, Hooke + Jaumann,
 //                 von Mises, EOS, grad v = G C with C = L^-1) -> S, u, rho,
 //                 parameters, and the cotangents of the pass-A sums
@@ -22,6 +22,7 @@
 // gravity.  Branch switches (viscosity on/off, yield on/off, EOS branches,
 // C = I fallback) are held at the forward evaluation's side.
 #include "eos.cuh"
+#include "fpbits.cuh"
 #include "pairs64.cuh"
 #include "sph_internal.cuh"
 
@@ -49,7 +50,59 @@ struct AdjArgs {
   const Units *U;
   const float *sums;  // mixed: the forward pass A's pair sums (16 rows of stride ld)
   int lane_shift;     // FP64: 2^lane_shift lanes share a particle's partner list
+  // mixed: the viscosity parameters in FP32, converted on the host (in the pair
+  // loop the compiler converted them for every pair, three FP64-unit
+  // instructions)
+  float f_alpha, f_beta, f_eps_v;
 };
+
+// Conversions of the mixed reverse on the integer pipe (fpbits.cuh), exact or
+// rounded as the FP64-unit instructions would; F = double passes values through.
+template <class F>
+__device__ __forceinline__ F narrow(double v) {
+  if constexpr (sizeof(F) == 4) return to_f32_scaled(v, 0, 1.0);
+  else return v;
+}
+// v * sc for a power of two sc
+template <class F>
+__device__ __forceinline__ F narrow(double v, double sc) {
+  if constexpr (sizeof(F) == 4) return to_f32_scaled(v, pow2_exp(sc), sc);
+  else return v;
+}
+__device__ __forceinline__ double widen(float v, double sc) { return to_f64_scaled(v, pow2_exp(sc), sc); }
+__device__ __forceinline__ double widen(double v, double) { return v; }
+// N values at once with one fallback branch: a call per value (to_f32_scaled's)
+// would make the compiler save its live registers around each
+template <int N, class F>
+__device__ __forceinline__ void narrow_n(const double *v, double sc, F *out) {
+  if constexpr (sizeof(F) == 4) {
+    const int k = pow2_exp(sc);
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < N; ++i) ok &= f32_rn_scaled(v[i], k, out[i]);
+    if (!ok) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) out[i] = __double2float_rn(v[i] * sc);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) out[i] = v[i];
+  }
+}
+// f *= sc in FP32, sc a power of two: one rounding, of the exact product, as in
+// FP64 and back
+template <int N>
+__device__ __forceinline__ void shift_n(float *f, double sc) {
+  const int k = pow2_exp(sc);
+  if (k >= -126 && k <= 127) {
+    const float fs = bitsf((uint32_t)(k + 127) << 23);
+#pragma unroll
+    for (int i = 0; i < N; ++i) f[i] *= fs;
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) f[i] = __double2float_rn((double)f[i] * sc);
+  }
+}
 
 __device__ __forceinline__ int sidx(int dim, int i, int j) { return symk(dim, i, j); }
 
@@ -144,20 +197,20 @@ struct VPair {
 template <class R>
 __device__ __forceinline__ VPair<R> visc_pair(int dim, const R d[3], const R w[3], R r2, R hab,
                                               R rho_a, R rho_b, R cs_a, R cs_b,
-                                              const sph_params &P) {
+                                              R alpha, R beta, R eps_v) {
   VPair<R> V;
   V.vx = R(0.0);
   for (int i = 0; i < dim; ++i) V.vx += w[i] * d[i];
   V.Pi = V.dPi_dnu = V.dnu_dvx = V.dnu_dr2 = V.dPi_dc = V.dPi_drb = R(0.0);
   if (V.vx < R(0.0)) {
-    const R iQ = R(1.0) / (r2 + R(P.eps_v) * hab * hab);
+    const R iQ = R(1.0) / (r2 + eps_v * hab * hab);
     const R nu = hab * V.vx * iQ;
     const R cb = R(0.5) * (cs_a + cs_b), irb = R(1.0) / (R(0.5) * (rho_a + rho_b));
-    V.Pi = (-R(P.alpha) * cb * nu + R(P.beta) * nu * nu) * irb;
-    V.dPi_dnu = (-R(P.alpha) * cb + R(2.0) * R(P.beta) * nu) * irb;
+    V.Pi = (-alpha * cb * nu + beta * nu * nu) * irb;
+    V.dPi_dnu = (-alpha * cb + R(2.0) * beta * nu) * irb;
     V.dnu_dvx = hab * iQ;
     V.dnu_dr2 = -nu * iQ;
-    V.dPi_dc = -R(P.alpha) * nu * irb;
+    V.dPi_dc = -alpha * nu * irb;
     V.dPi_drb = -V.Pi * irb;
   }
   return V;
@@ -395,9 +448,13 @@ __device__ void eos_scaled(const sph_material &M0, double s, double rho, double 
 // each particle's are scaled by a power of two to order one first and its
 // results scaled back exactly: FP32's exponent range then limits only the
 // state, whose SI values it holds.  FP64: the sums of the FP64 pass A, and the
-// reverse is FP64 throughout (F = double, no scaling).
+// reverse is FP64 throughout (F = double, no scaling).  The mixed form was bound
+// by the FP64 unit (76 % of it) through its conversions; on the integer pipe, and
+// writing pass A's cotangents in code units itself, it and the kernels around it
+// take 0.47 instead of 0.53 ms at 1M (five blocks per SM; 3 % of the call slower
+// at the compiler's 131 registers).
 template <bool MIXED, int DIM>
-__global__ void k_adj_update(AdjArgs A) {
+__global__ void __launch_bounds__(128, MIXED ? 5 : 1) k_adj_update(AdjArgs A) {
   using F = typename std::conditional<MIXED, float, double>::type;
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= A.n) return;
@@ -419,8 +476,8 @@ __global__ void k_adj_update(AdjArgs A) {
     const F *sm;
     if constexpr (MIXED) sm = A.sums;
     else sm = A.inter;
-    const F it = MIXED ? (F)A.U->invT : F(1);
-    srho = MIXED ? (double)sm[c] * A.U->invT : (double)sm[c];
+    const F it = MIXED ? narrow<F>(A.U->invT) : F(1);
+    srho = MIXED ? widen(sm[c], A.U->invT) : (double)sm[c];
     for (int i = 0; i < dim; ++i)
       for (int j = 0; j <= i; ++j) L[i][j] = L[j][i] = sm[(int64_t)(1 + i * (i + 1) / 2 + j) * ld + c];
     for (int i = 0; i < dim; ++i)
@@ -443,7 +500,7 @@ __global__ void k_adj_update(AdjArgs A) {
   const int mi = (mi0 >= 0 && mi0 < A.mt.nmat) ? mi0 : 0;
   const sph_material &M = A.mt.m[mi];
   const double uc = A.u[c];
-  const F mu = (F)M.mu, Y0 = (F)M.Y0;
+  const F mu = narrow<F>(M.mu), Y0 = narrow<F>(M.Y0);
   F p, pr, pu;
   // MIXED: one evaluation in FP32 dual numbers, in the forward's code units,
   // gives p, dp/drho, dp/du and the exact derivatives of c_s in rho and u and
@@ -456,22 +513,28 @@ __global__ void k_adj_update(AdjArgs A) {
     const EosC<ad::Dual3> K = eos_consts<ad::Dual3>(M, U->matf[mi], U);
     ad::Dual3 p3, c3, pr3, pu3;
     eos_eval<ad::Dual3>(M, K, rc, uc, p3, c3, &pr3, &pu3);
-    p = p3.v * (float)U->sig;
-    pr = pr3.v * (float)(U->sig * U->invrho);
-    pu = pu3.v * (float)(U->sig * U->invE);
-    dcr = c3.d[0] * (float)(U->V * U->invrho);
-    dcu = c3.d[1] * (float)(U->V * U->invE);
-    dps = p3.d[2] * (float)U->sig;
-    dcs = c3.d[2] * (float)U->V;
+    const float sig = narrow<float>(U->sig), V = narrow<float>(U->V);
+    p = p3.v * sig;
+    pr = pr3.v * narrow<float>(U->sig, U->invrho);
+    pu = pu3.v * narrow<float>(U->sig, U->invE);
+    dcr = c3.d[0] * narrow<float>(U->V, U->invrho);
+    dcu = c3.d[1] * narrow<float>(U->V, U->invE);
+    dps = p3.d[2] * sig;
+    dcs = c3.d[2] * V;
   } else {
     double cs;
     eos_scaled(M, 1.0, rc, uc, p, cs, &pr, &pu);
   }
   const bool strength = A.S != nullptr && M.strength;
   F S[3][3], St[3][3];
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j)
-      S[i][j] = (strength && i < dim && j < dim) ? (F)A.S[(int64_t)sidx(dim, i, j) * A.n + c] : F(0);
+  {
+    double s64[6];
+    F s6[6];
+    for (int k = 0; k < 6; ++k) s64[k] = strength && k < ns ? A.S[(int64_t)k * A.n + c] : 0.0;
+    narrow_n<6>(s64, 1.0, s6);
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j) S[i][j] = (i < dim && j < dim) ? s6[sidx(dim, i, j)] : F(0);
+  }
   F J2 = F(0);
   for (int i = 0; i < dim; ++i)
     for (int j = 0; j < dim; ++j) J2 += S[i][j] * S[i][j];
@@ -486,37 +549,59 @@ __global__ void k_adj_update(AdjArgs A) {
   const bool damage = A.dmg != nullptr && M.damage;
   F dd = F(0);
   if (damage) {
-    const F del = (F)A.dmg[c];
+    const F del = narrow<F>(A.dmg[c]);
     dd = del * del * del;
   }
   // ---- the cotangents (of T, c_s, dS/dt), scaled (MIXED) ----
   double sc = 1.0, isc = 1.0;
   if constexpr (MIXED) {
-    double mx = fabs(A.csbar[c]);
-    for (int k = 0; k < ns; ++k) mx = fmax(mx, fabs(A.Tbar[(int64_t)k * ld + c]));
+    // the largest magnitude, from the bits (a NaN does not count)
+    const uint64_t inf = 0x7ff0000000000000ULL;
+    uint64_t mx = 0;
+    auto largest = [&](double v) {
+      const uint64_t b = dbits(v) & 0x7fffffffffffffffULL;
+      if (b > mx && b <= inf) mx = b;
+    };
+    largest(A.csbar[c]);
+    for (int k = 0; k < ns; ++k) largest(A.Tbar[(int64_t)k * ld + c]);
     if (A.bdS && strength)
-      for (int k = 0; k < ns; ++k) mx = fmax(mx, fabs(A.bdS[(int64_t)k * A.n + c]));
-    if (mx > 0.0 && mx < INFINITY) {
-      int e;
-      frexp(mx, &e);
-      sc = ldexp(1.0, -e);
-      isc = ldexp(1.0, e);
+      for (int k = 0; k < ns; ++k) largest(A.bdS[(int64_t)k * A.n + c]);
+    const int e = (int)(mx >> 52) - 1022;  // 2^(e-1) <= mx < 2^e for a normal number
+    if (e > -1022 && e < 1024) {
+      sc = bitsd((uint64_t)(1023 - e) << 52);
+      isc = bitsd((uint64_t)(1023 + e) << 52);
+    } else if (mx > 0 && mx < inf) {
+      int es;
+      frexp(bitsd(mx), &es);
+      sc = ldexp(1.0, -es);
+      isc = ldexp(1.0, es);
     }
   }
   // ---- reverse: T = sigma / rho^2 ----
   F Tb[3][3], Tc[6];
   {
-    double t64[6];
-    load_T64(A, c, t64);
-    for (int k = 0; k < 6; ++k) Tc[k] = (F)t64[k];
+    if constexpr (MIXED) {
+      const float4 t0 = A.Tf[c], t1 = A.Tf[ld + c];
+      const float t[6] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y};
+      for (int k = 0; k < 6; ++k) Tc[k] = k < ns ? t[k] : 0.f;
+      shift_n<6>(Tc, A.U->sig * A.U->invrho * A.U->invrho);  // T = sigma / rho^2
+    } else {
+      load_T64(A, c, Tc);
+    }
   }
   F TbT = F(0), trSig = F(0);
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      Tb[i][j] = (i < dim && j < dim) ? (F)(A.Tbar[(int64_t)sidx(dim, i, j) * A.ld + c] * sc) : F(0);
-      if (i < dim && j < dim) TbT += Tb[i][j] * Tc[sidx(dim, i, j)];
-    }
-  const F rcf = (F)rc;
+  {
+    double t64[6];
+    F t6[6];
+    for (int k = 0; k < 6; ++k) t64[k] = k < ns ? A.Tbar[(int64_t)k * ld + c] : 0.0;
+    narrow_n<6>(t64, sc, t6);
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j) {
+        Tb[i][j] = (i < dim && j < dim) ? t6[sidx(dim, i, j)] : F(0);
+        if (i < dim && j < dim) TbT += Tb[i][j] * Tc[sidx(dim, i, j)];
+      }
+  }
+  const F rcf = narrow<F>(rc);
   F rhobar = F(-2) * TbT / rcf;
   const F irc2 = F(1) / (rcf * rcf);  // one division for the nine components below
   F sigbar[3][3];
@@ -531,12 +616,17 @@ __global__ void k_adj_update(AdjArgs A) {
     for (int j = 0; j < 3; ++j) Stbar[i][j] = (F(1) - dd) * sigbar[i][j];
   // ---- reverse: dS = 2 mu (eps_dot - tr/D I) + R S_t - S_t R ----
   F Sdb[3][3];  // full-matrix cotangent of dS (symmetric)
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      const F cst = (A.bdS && strength && i < dim && j < dim) ? (F)(A.bdS[(int64_t)sidx(dim, i, j) * A.n + c] * sc)
-                                                               : F(0);
-      Sdb[i][j] = (i == j) ? cst : F(0.5) * cst;
-    }
+  {
+    double s64[6];
+    F s6[6];
+    for (int k = 0; k < 6; ++k) s64[k] = A.bdS && strength && k < ns ? A.bdS[(int64_t)k * A.n + c] : 0.0;
+    narrow_n<6>(s64, sc, s6);
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j) {
+        const F cst = (i < dim && j < dim) ? s6[sidx(dim, i, j)] : F(0);
+        Sdb[i][j] = (i == j) ? cst : F(0.5) * cst;
+      }
+  }
   F ed[3][3], Rr[3][3], tr = F(0);
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) {
@@ -590,12 +680,12 @@ __global__ void k_adj_update(AdjArgs A) {
         const F wk = k < dim ? F(1) : F(2);
         sb = fY * Stb_st[k] - fjp * wk * S_st[k];
       }
-      A.gS[(int64_t)k * A.n + c] += (double)sb * isc;
+      A.gS[(int64_t)k * A.n + c] += widen(sb, isc);
     }
     if (yielding) Y0bar = proj * F(2) * fY / Y0;
   }
   // ---- reverse: EOS ----
-  const F csbar = (F)(A.csbar[c] * sc);
+  const F csbar = narrow<F>(A.csbar[c], sc);
   F ubar = pbar * pu;
   rhobar += pbar * pr;
   F Kbar = F(0);
@@ -667,20 +757,30 @@ __global__ void k_adj_update(AdjArgs A) {
   }
   // ---- reverse: drho = rho * sum_rho ; dx = v + xsph * xs (FP64, unscaled) ----
   const double bdr = A.bdrho ? A.bdrho[c] : 0.0;
-  A.grho[c] += (double)rhobar * isc + bdr * srho;
-  A.gu[c] += (double)ubar * isc;
+  A.grho[c] += widen(rhobar, isc) + bdr * srho;
+  A.gu[c] += widen(ubar, isc);
   for (int i = 0; i < dim; ++i)
     if (A.bdx[i]) A.gv[i][c] += A.bdx[i][c];
-  double *I = A.inter;
-  I[c] = rc * bdr;
   if constexpr (MIXED) {
+    // the cotangents of the pass-A sums in code units (see ACot): the
+    // continuity sum and G are rates (1/T), L is a number, XSPH a velocity
+    const Units &U = *A.U;
+    float v[24];
     for (int i = 0; i < 3; ++i)
       for (int j = 0; j < 3; ++j) {
-        I[(1 + 3 * i + j) * ld + c] = (double)Lbar[i][j] * isc;
-        I[(10 + 3 * i + j) * ld + c] = (double)Gbar[i][j] * isc;
+        v[1 + 3 * i + j] = Lbar[i][j];
+        v[10 + 3 * i + j] = Gbar[i][j];
       }
-    for (int i = 0; i < 3; ++i) I[(19 + i) * ld + c] = (i < dim && A.bdx[i]) ? P.xsph * A.bdx[i][c] : 0.0;
+    shift_n<9>(v + 1, isc);
+    shift_n<9>(v + 10, isc * U.invT);
+    v[0] = narrow<float>(rc * bdr, U.invT);
+    for (int i = 0; i < 3; ++i) v[19 + i] = (i < dim && A.bdx[i]) ? narrow<float>(P.xsph * A.bdx[i][c], U.V) : 0.f;
+    v[22] = v[23] = 0.f;
+    for (int q = 0; q < 6; ++q)
+      A.Apk[(int64_t)q * ld + c] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
   } else {
+    double *I = A.inter;
+    I[c] = rc * bdr;
     // the layout of k_adj_passA: L's cotangent enters through d^T Lbar d only
     for (int i = 0; i < dim; ++i)
       for (int j = i; j < dim; ++j)
@@ -689,9 +789,9 @@ __global__ void k_adj_update(AdjArgs A) {
       for (int j = 0; j < dim; ++j) I[(7 + 3 * i + j) * ld + c] = Gbar[i][j];
     for (int i = 0; i < dim; ++i) I[(16 + i) * ld + c] = A.bdx[i] ? P.xsph * A.bdx[i][c] : 0.0;
   }
-  A.pbar[c] = strength ? (double)mubar * isc : 0.0;
-  A.pbar[ld + c] = (double)Y0bar * isc;
-  A.pbar[2 * ld + c] = (double)Kbar * isc;
+  A.pbar[c] = strength ? widen(mubar, isc) : 0.0;
+  A.pbar[ld + c] = widen(Y0bar, isc);
+  A.pbar[2 * ld + c] = widen(Kbar, isc);
 }
 
 // ---------------------------------------------------------------------------
@@ -882,7 +982,7 @@ __global__ void k_adj_passA(AdjArgs A) {
 // param_bar[(inst * nmat + mat) * 3 + k], in a fixed order.  Block (inst, j)
 // sums the j-th of gy equal chunks of its instance (a strided loop, then a
 // tree in shared memory); with part set it stores that partial sum, and
-// k_adj_params_final adds the gy partials of each entry in chunk order.  With
+// k_adj_params_final adds the gy partials of each entry.  With
 // part NULL (gy = 1) the block adds its instance's sum to out itself.
 constexpr int kParamThreads = 256;
 constexpr int64_t kParamChunk = 4096;  // particles per block, about
@@ -922,14 +1022,18 @@ __global__ void __launch_bounds__(kParamThreads) k_adj_params(const double *__re
   }
 }
 
+// A warp per entry: lane i adds the partials i, i + 32, ..., then the lanes in a
+// fixed order (a thread per entry, one partial after the other: 23 us at 1M)
 __global__ void k_adj_params_final(const double *__restrict__ part, int64_t m, int gy, double *out) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // entry (inst * nmat + mat) * 3 + k
+  const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // entry (inst * nmat + mat) * 3 + k
   if (t >= m) return;
+  const int lane = threadIdx.x & 31;
   const int64_t q = t / 3;
   const int k = (int)(t - 3 * q);
   double s = 0.0;
-  for (int j = 0; j < gy; ++j) s += part[(q * gy + j) * 3 + k];
-  out[t] += s;
+  for (int j = lane; j < gy; j += 32) s += part[(q * gy + j) * 3 + k];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[t] += s;
 }
 
 // The parameter cotangents of all particles (c->ag, 3 x cap_n) summed into
@@ -945,7 +1049,7 @@ static void adj_params_sum(sph_ctx *c, const int32_t *mat, const int64_t *inst_o
                                                           param_bar); ++sph::g_launches; }
   if (part) {
     const int64_t m = (int64_t)ninst * nmat * 3;
-    { k_adj_params_final<<<nblk(m, 256), 256, 0, st>>>(part, m, gy, param_bar); ++sph::g_launches; }
+    { k_adj_params_final<<<nblk(32 * m, 256), 256, 0, st>>>(part, m, gy, param_bar); ++sph::g_launches; }
   }
 }
 
@@ -954,27 +1058,19 @@ static void adj_params_sum(sph_ctx *c, const int32_t *mat, const int64_t *inst_o
 // and A are differentiated in FP32, in the code units of the forward
 // evaluation (powers of two, so every conversion is exact), on differences of
 // the hi/lo-split positions and velocities as in the forward pass, with
-// Kahan-compensated FP32 sums; the constitutive update (k_adj_update) stays
-// FP64.  A quantity q in SI is q_code * U_q, so its cotangent in SI is the
-// code-unit cotangent divided by U_q, and a given output cotangent enters in
-// code units multiplied by U_q.
+// Kahan-compensated FP32 sums.  A quantity q in SI is q_code * U_q, so its
+// cotangent in SI is the code-unit cotangent divided by U_q, and a given output
+// cotangent enters in code units multiplied by U_q.
 // ---------------------------------------------------------------------------
-// Forward T and c_s back to FP64 SI for k_adj_update; output cotangents of
-// dv/dt and du/dt into code units for pass B.
-__global__ void k_adj_unpack32(AdjArgs A, double *T64, double *cs64) {
+// Output cotangents of dv/dt and du/dt into code units for pass B.
+__global__ void k_adj_pack_cot32(AdjArgs A) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= A.n) return;
   const Units &U = *A.U;
-  const double uT = U.sig * U.invrho * U.invrho;  // T = sigma / rho^2
-  const float4 t0 = A.Tf[c], t1 = A.Tf[A.ld + c];
-  const float t[6] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y};
-  const int ns = nsym(A.dim);
-  for (int k = 0; k < 6; ++k) T64[(int64_t)k * A.ld + c] = k < ns ? (double)t[k] * uT : 0.0;
-  cs64[c] = (double)t1.z * U.V;
   float vb[3] = {0.f, 0.f, 0.f};
   for (int i = 0; i < A.dim; ++i)
-    if (A.bdv[i]) vb[i] = (float)(A.bdv[i][c] * U.acc);
-  const float ub = A.bdu ? (float)(A.bdu[c] * (U.E * U.invT)) : 0.f;
+    if (A.bdv[i]) vb[i] = narrow<float>(A.bdv[i][c], U.acc);
+  const float ub = A.bdu ? narrow<float>(A.bdu[c], U.E * U.invT) : 0.f;
   A.Bpk[c] = make_float4(vb[0], vb[1], vb[2], ub);
 }
 
@@ -1020,7 +1116,7 @@ __global__ void k_adj_passB32(AdjArgs A) {
     float r2 = 0.f;
     for (int i = 0; i < dim; ++i) r2 += d[i] * d[i];
     const KPair<float> K = kernel_pair<float>(dim, sqrtf(r2), hab);
-    const VPair<float> Vs = visc_pair<float>(dim, d, w, r2, hab, Vc.w, Ve.w, csc, cse, A.prm);
+    const VPair<float> Vs = visc_pair<float>(dim, d, w, r2, hab, Vc.w, Ve.w, csc, cse, A.f_alpha, A.f_beta, A.f_eps_v);
     float db[3], wb[3], Bs[6], csh, rh;
     pairB_adj<float>(dim, d, w, K, Vs, Tc, Te, Qe.w, vbc, bc.w, db, wb, Bs, csh, rh);  // c's own term
     for (int i = 0; i < dim; ++i) {
@@ -1049,25 +1145,6 @@ __global__ void k_adj_passB32(AdjArgs A) {
   const double uTinv = U.rho * U.rho * U.invsig;
   for (int q = 0; q < 6; ++q) A.Tbar[(int64_t)q * A.ld + c] = q < ns ? Tb[q].value() * uTinv : 0.0;
   A.csbar[c] = csb.value() * U.invV;
-}
-
-// Cotangents of the pass-A sums (FP64 SI, from k_adj_update) into code units:
-// the continuity sum and G are rates (1/T), L is a number, XSPH a velocity.
-__global__ void k_adj_pack_acot32(AdjArgs A) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= A.n) return;
-  const Units &U = *A.U;
-  const double *I = A.inter;
-  const int64_t ld = A.ld;
-  float v[24];
-  v[0] = (float)(I[c] * U.invT);
-  for (int k = 0; k < 9; ++k) {
-    v[1 + k] = (float)I[(1 + k) * ld + c];
-    v[10 + k] = (float)(I[(10 + k) * ld + c] * U.invT);
-  }
-  for (int i = 0; i < 3; ++i) v[19 + i] = (float)(I[(19 + i) * ld + c] * U.V);
-  v[22] = v[23] = 0.f;
-  for (int q = 0; q < 6; ++q) A.Apk[(int64_t)q * ld + c] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
 }
 
 __device__ __forceinline__ ACot<float> load_acot32(const AdjArgs &A, int64_t a) {
@@ -1188,12 +1265,10 @@ void rhs_adjoint(sph_ctx *c, const sph_state *s, const MatTable &mt, const sph_p
     A.Apk = c->adj32 + c->cap_n;
     A.U = c->units;
     A.sums = c->adj_sums;
-    // FP64 SI copies of T and c_s for the constitutive reverse (the third
-    // derivative set of the step buffers is free here)
-    double *T64 = c->st.d_S[2], *cs64 = c->st.d_cs[2];
-    A.T = T64;
-    A.cs = cs64;
-    { k_adj_unpack32<<<nblk(n, 256), 256, 0, st>>>(A, T64, cs64); ++sph::g_launches; }
+    A.f_alpha = (float)p.alpha;
+    A.f_beta = (float)p.beta;
+    A.f_eps_v = (float)p.eps_v;
+    { k_adj_pack_cot32<<<nblk(n, 256), 256, 0, st>>>(A); ++sph::g_launches; }
     if (s->dim == 3) {
       { k_adj_passB32<3><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
       { k_adj_update<true, 3><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
@@ -1201,7 +1276,6 @@ void rhs_adjoint(sph_ctx *c, const sph_state *s, const MatTable &mt, const sph_p
       { k_adj_passB32<2><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
       { k_adj_update<true, 2><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
     }
-    { k_adj_pack_acot32<<<nblk(n, 256), 256, 0, st>>>(A); ++sph::g_launches; }
     if (s->dim == 3) { k_adj_passA32<3><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
     else { k_adj_passA32<2><<<nblk(n, T), T, 0, st>>>(A); ++sph::g_launches; }
   } else {

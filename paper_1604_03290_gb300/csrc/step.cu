@@ -36,15 +36,23 @@ struct DtArgs {
 
 // FP32 view of a double for screening, built from its bits on the integer
 // pipe: the top 23 mantissa bits (truncated: relative error below 2^-23).
-// Outside 2^-60 <= |v| <= 2^60 (zero excepted) the view is not trusted and
-// `risky` is set; squares and quotients of trusted views stay in FP32's
-// normal range.
-__device__ __forceinline__ float screen_f32(double v, bool &risky) {
+// Squares and quotients of views with 2^-60 <= |v| <= 2^60 stay in FP32's
+// normal range.  Above that the view is not trusted and `risky` is set; below
+// (zero excepted) the view is `tiny` and `low` is set: 0 for a numerator, 2^-60
+// for a denominator, so that the limit formed from it is a lower bound.  (A
+// state at rest holds many derivatives of rounding size; taken as not trusted,
+// each cost an FP64 division, 0.17 instead of 0.08 ms for 832k particles.)
+constexpr float kTinyDen = 8.67361737988403547e-19f;  // 2^-60
+__device__ __forceinline__ float screen_f32(double v, bool &risky, bool &low, float tiny) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
   if ((b << 1) == 0ULL) return 0.f;
   const unsigned hi = (unsigned)(b >> 32);
   const int e = (int)((hi >> 20) & 0x7ffu);
-  if (e < 1023 - 60 || e > 1023 + 60) {
+  if (e < 1023 - 60) {
+    low = true;
+    return tiny;
+  }
+  if (e > 1023 + 60) {
     risky = true;
     return 0.f;
   }
@@ -68,8 +76,9 @@ static __device__ __noinline__ double accel_limit(int dim, double h, double a0, 
 // is first estimated in FP32 (within about 1e-6 relative); the FP64 expression
 // is then evaluated only for limits whose estimate lies within 2^-12 of the
 // smallest estimate of the block (of the warp or the lane, when those span
-// several instances: `scope` 2, 1, 0), or whose inputs the FP32 view does not
-// trust.  Any limit skipped is larger than the one that attains that minimum,
+// several instances: `scope` 2, 1, 0; a lower bound does not count as an
+// estimate, but is held against the smallest), or whose inputs the FP32 view
+// does not trust.  Any limit skipped is larger than the one that attains that minimum,
 // so the minimum over the scope equals the all-FP64 minimum bit for bit, at
 // about one FP64 division per block.  The result for one thread is only
 // meaningful through that minimum.
@@ -78,67 +87,73 @@ __device__ double particle_dt(const DtArgs &A, int64_t a_in, bool valid, int sco
   const int64_t a = valid ? a_in : A.n - 1;  // lanes past the end read the last particle, then drop out
   const float inf = __int_as_float(0x7f800000);
   float est[11];
-  unsigned risky = 0;
+  unsigned risky = 0, low = 0;  // per limit: view not trusted; est a lower bound
   const double h = A.h[a], cs = A.cs[a];
-  bool r = false;
-  const float hf = screen_f32(h, r);
+  bool r = false, rl = false;
+  const float hf = screen_f32(h, r, rl, 0.f);
   {
-    bool rc = r;
-    const float csf = screen_f32(cs, rc);
+    bool rc = r, l = rl;
+    const float csf = screen_f32(cs, rc, l, kTinyDen);
     est[0] = (long long)__double_as_longlong(cs) > 0 ? A.f_courant * hf * __frcp_rn(csf) : inf;
     if (rc) risky |= 1u;
+    if (l) low |= 1u;
   }
   double dvd[3] = {0.0, 0.0, 0.0};
   {
-    bool ra = r, any = false;
+    bool ra = r, l = rl, any = false;
     float a2 = 0.f;
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
       if (ax >= A.dim) break;
       dvd[ax] = A.dv[ax][a];
-      const float f = screen_f32(dvd[ax], ra);
+      const float f = screen_f32(dvd[ax], ra, l, kTinyDen);
       a2 += f * f;
       any |= bits_nonzero(dvd[ax]);
     }
     est[1] = any ? A.f_accel * sqrtf(hf) * rsqrtf(sqrtf(a2)) : inf;
     if (ra) risky |= 2u;
+    if (l) low |= 2u;
   }
   const double drho = A.drho[a], rho = A.rho[a];
   {
-    bool rr = false;
-    const float q = fabsf(screen_f32(rho, rr)), d = fabsf(screen_f32(drho, rr));
+    bool rr = false, l = false;
+    const float q = fabsf(screen_f32(rho, rr, l, 0.f)), d = fabsf(screen_f32(drho, rr, l, kTinyDen));
     est[2] = (!P.density_sum && bits_nonzero(drho)) ? A.f_quantity * q * __frcp_rn(d) : inf;
     if (rr) risky |= 4u;
+    if (l) low |= 4u;
   }
   const double du = A.du[a], u = A.u[a];
   {
-    bool rr = false;
-    const float q = fabsf(screen_f32(u, rr)), d = fabsf(screen_f32(du, rr));
+    bool rr = false, l = false;
+    const float q = fabsf(screen_f32(u, rr, l, 0.f)), d = fabsf(screen_f32(du, rr, l, kTinyDen));
     est[3] = bits_nonzero(du) ? A.f_quantity * (q + A.f_u_floor) * __frcp_rn(d) : inf;
     if (rr) risky |= 8u;
+    if (l) low |= 8u;
   }
   const int ns = nsym(A.dim);
   const bool has_S = A.S && A.dS;
   for (int k = 0; k < 6; ++k) {
     est[4 + k] = inf;
     if (has_S && k < ns) {
-      bool rr = false;
+      bool rr = false, l = false;
       const double q = A.S[(int64_t)k * A.n + a], dq = A.dS[(int64_t)k * A.n + a];
-      const float qf = fabsf(screen_f32(q, rr)), df = fabsf(screen_f32(dq, rr));
+      const float qf = fabsf(screen_f32(q, rr, l, 0.f)), df = fabsf(screen_f32(dq, rr, l, kTinyDen));
       if (bits_nonzero(dq)) est[4 + k] = A.f_quantity * (qf + A.f_S_floor) * __frcp_rn(df);
       if (rr) risky |= 16u << k;
+      if (l) low |= 16u << k;
     }
   }
   est[10] = inf;
   const bool has_d = A.dmg && A.ddmg;
   double dd = 0.0, dq = 0.0;
   if (has_d) {
-    bool rr = false;
+    bool rr = false, l = false;
     dq = A.ddmg[a];
     dd = A.dmg[a];
-    const float qf = fabsf(screen_f32(dd, rr)), df = screen_f32(dq, rr);
+    const float qf = fabsf(screen_f32(dd, rr, l, 0.f)), df = screen_f32(dq, rr, l, kTinyDen);
     if ((long long)__double_as_longlong(dq) > 0) est[10] = A.f_quantity * (qf + A.f_dmg_floor) * __frcp_rn(df);
     if (rr) risky |= 1024u;
+    if (l) low |= 1024u;
   }
   if (!valid) {
     risky = 0;
@@ -148,7 +163,7 @@ __device__ double particle_dt(const DtArgs &A, int64_t a_in, bool valid, int sco
   float best = A.f_dt_max;
 #pragma unroll
   for (int i = 0; i < 11; ++i)
-    if (!((risky >> i) & 1u)) best = fminf(best, est[i]);
+    if (!(((risky | low) >> i) & 1u)) best = fminf(best, est[i]);
   if (scope >= 1)
     for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
   if (scope == 2) {

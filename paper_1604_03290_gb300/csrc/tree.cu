@@ -344,6 +344,7 @@ __device__ __forceinline__ int32_t block_excl_scan(int32_t v, int32_t *total) {
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kLookWin = 8;
 constexpr int kSortWarps = kSortThreads / 32;
 
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const unsigned long long *__restrict__ keys, int64_t n,
@@ -414,12 +415,12 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_pass(const unsigned long 
   *mine = own | (tile == 0 ? kLookIncl : kLookOwn);
   uint32_t before = 0;
   bool known = tile == 0;
-  for (int q = tile - 1; q >= 0 && !known; q -= 8) {
-    uint32_t v[8];
+  for (int q = tile - 1; q >= 0 && !known; q -= kLookWin) {
+    uint32_t v[kLookWin];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = q - u >= 0 ? look_load(&state[(int64_t)(q - u) * 256 + t]) : kLookIncl;
+    for (int u = 0; u < kLookWin; ++u) v[u] = q - u >= 0 ? look_load(&state[(int64_t)(q - u) * 256 + t]) : kLookIncl;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < kLookWin; ++u) {
       if (known) continue;
       int polls = 0;
       while ((v[u] >> 30) == 0u && ++polls < kLookPolls) {
@@ -447,12 +448,75 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_pass(const unsigned long 
   }
 }
 
+// The same sort for n <= kSmallSort in one launch: a pair's place is the number
+// of pairs before it in (key, index) order, counted against every key.  A
+// block places 32 pairs, a lane each; its warps share out the keys, read from
+// shared memory two at a time.  n^2 comparisons of about four instructions over
+// the whole chip, against a launch per digit with a few tiles at 7.5 us each.
+// A 3D tree and partner lists, with and without it: 4.1k particles 279 / 349 us,
+// 8.0k 289 / 354, 13.9k 316 / 353, 22k 385 / 371, 33k 512 / 400; so the line is
+// drawn at 16k.  (The digits in one block's shared memory: 39 us for six digits
+// of 4.4k keys, against 6 us here.)
+constexpr int kRankThreads = 512, kRankTile = 2048;
+constexpr int64_t kSmallSort = 16384;
+
+__global__ void __launch_bounds__(kRankThreads) k_sort_small(const unsigned long long *__restrict__ kin,
+                                                             const int32_t *__restrict__ vin,
+                                                             unsigned long long *__restrict__ kout,
+                                                             int32_t *__restrict__ vout, int n) {
+  constexpr int W = kRankThreads / 32;
+  __shared__ __align__(16) unsigned long long sk[kRankTile];
+  __shared__ int red[W][32];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int i0 = blockIdx.x * 32, i = i0 + lane;
+  const unsigned long long ki = i < n ? kin[i] : 0ULL;
+  int cnt = 0;
+  for (int j0 = 0; j0 < n; j0 += kRankTile) {
+    const int m = min(kRankTile, n - j0), share = ((m + 2 * W - 1) / (2 * W)) * 2;
+    __syncthreads();
+    // past the end: a key that counts for none (m is odd only when n - j0 is)
+    for (int k = t; k < ((m + 1) & ~1); k += kRankThreads) sk[k] = k < m ? kin[j0 + k] : ~0ULL;
+    __syncthreads();
+    const int a = min(w * share, (m + 1) & ~1), b = min(a + share, (m + 1) & ~1);
+    // keys before the block's own pairs, among them, after them
+    const int own = min(max(i0 - j0, a), b), past = min(max(i0 + 32 - j0, a), b);
+    const ulonglong2 *s2 = (const ulonglong2 *)sk;
+#pragma unroll 8
+    for (int k = a; k < own; k += 2) {
+      const ulonglong2 q = s2[k >> 1];
+      cnt += q.x <= ki ? 1 : 0;
+      cnt += q.y <= ki ? 1 : 0;
+    }
+    for (int k = own; k < past; ++k) cnt += (sk[k] < ki || (sk[k] == ki && j0 + k < i)) ? 1 : 0;
+#pragma unroll 8
+    for (int k = past; k < b; k += 2) {
+      const ulonglong2 q = s2[k >> 1];
+      cnt += q.x < ki ? 1 : 0;
+      cnt += q.y < ki ? 1 : 0;
+    }
+  }
+  red[w][lane] = cnt;
+  __syncthreads();
+  if (w > 0 || i >= n) return;
+  int pos = 0;
+#pragma unroll
+  for (int k = 0; k < W; ++k) pos += red[k][lane];
+  kout[pos] = ki;
+  vout[pos] = vin[i];
+}
+
 static int sort_passes(int bits) { return (bits + 7) / 8; }
 
-// The passes; Tree::look zeroed, its histograms filled
+// The passes; above kSmallSort with Tree::look zeroed and its histograms filled
 static void sort_run(sph_ctx *c, int64_t n, int bits, cudaStream_t st) {
   Tree &T = c->tree;
   const int tiles = nblk(n, kSortTile), passes = sort_passes(bits);
+  if (n <= kSmallSort) {
+    { k_sort_small<<<nblk(n, 32), kRankThreads, 0, st>>>(T.keys[0], T.vals[0], T.keys[1], T.vals[1], (int)n); ++sph::g_launches; }
+    T.skey = T.keys[1];
+    T.perm = T.vals[1];
+    return;
+  }
   int src = 0;
   for (int p = 0; p < passes; ++p) {
     k_sort_pass<<<tiles, kSortThreads, 0, st>>>(T.keys[src], T.vals[src], T.keys[src ^ 1], T.vals[src ^ 1], n, 8 * p,
@@ -474,6 +538,10 @@ void sort_pairs(sph_ctx *c, int64_t n, int bits, cudaStream_t st) {
   if (n <= 0) {
     T.skey = T.keys[0];
     T.perm = T.vals[0];
+    return;
+  }
+  if (n <= kSmallSort) {
+    sort_run(c, n, bits, st);
     return;
   }
   const int passes = sort_passes(bits);
@@ -1016,7 +1084,7 @@ void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cu
   if (n > 0) {
     { k_keys<<<std::min(nblk(n, 256), 8 * c->num_sms), 256, 0, st>>>(
           s->x[0], s->x[1], s->x[2], s->v[0], s->v[1], s->v[2], s->h, s->m, s->rho, n, dim, max_depth, s->inst_off,
-          ninst, passes, pack, c->pk, c->units, T); ++sph::g_launches; }
+          ninst, n <= kSmallSort ? 0 : passes, pack, c->pk, c->units, T); ++sph::g_launches; }
     sort_run(c, n, bits, st);
   } else {
     T.skey = T.keys[0];

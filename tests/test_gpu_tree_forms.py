@@ -30,7 +30,7 @@ def _keys(x, off, depth):
     return key
 
 
-@pytest.mark.parametrize("n", [1, 2, 255, 256, 257, 2047, 2048, 2049, 4095, 4097, 70001])
+@pytest.mark.parametrize("n", [1, 2, 255, 256, 257, 1023, 1025, 2047, 2048, 2049, 4095, 4097, 16383, 16385, 70001])
 @pytest.mark.parametrize("dim,parts,depth", [(3, 1, 20), (2, 1, 21), (3, 5, 18)])
 def test_permutation_is_the_stable_sort(n, dim, parts, depth):
     from paper_1604_03290_gb300 import sph

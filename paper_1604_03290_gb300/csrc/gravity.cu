@@ -73,6 +73,13 @@ struct GravSumF {
     pz += fz;
     if (++n == kFlushTerms) flush();
   }
+  // the term g d; the fused form is written out, so that every instance of the walk rounds alike
+  __device__ __forceinline__ void add_scaled(float g, const float d[3]) {
+    px = __fmaf_rn(g, d[0], px);
+    py = __fmaf_rn(g, d[1], py);
+    pz = __fmaf_rn(g, d[2], pz);
+    if (++n == kFlushTerms) flush();
+  }
   __device__ __forceinline__ void value(double &x, double &y, double &z) {
     flush();
     x = kx.value();
@@ -80,6 +87,11 @@ struct GravSumF {
     z = kz.value();
   }
 };
+
+// x^2 + y^2 + z^2, its fused operations written out as well
+__device__ __forceinline__ float norm2(float x, float y, float z) {
+  return __fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y)));
+}
 
 // 1 / q^(3/2) from the reciprocal square root in FP32 (a few ulps, far below
 // the mixed form's tolerance)
@@ -126,12 +138,16 @@ __device__ __forceinline__ double r2_fp64(const double xa[3], double cx, double 
 // (the node's member range only when some lane sums it directly), and the
 // node edge s0 / 2^level is the instance's FP32 edge shifted by the level:
 // the same value k_node_finish stores otherwise.
-template <int DIM, bool PACKED>
+// INSIDE, COUNT: with the containment test, with the interaction counters.  Each
+// costs a few instructions and registers at every visit, so the packed form
+// has instances without them: 2M cloud step (neither) 34.1 -> 33.0 ms, 400k pair
+// window (containment only) 19.3 -> 18.7 ms, 1 % of it from leaving the warp's
+// second vote out at inner nodes.
+template <int DIM, bool PACKED, bool INSIDE, bool COUNT>
 __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(GravArgs A) {
   using R = float;
   __shared__ float4 sh_hi[kGrWarps][kMaxLeaf];  // (x_hi, y_hi, z_hi, G m_b) of leaf members
   __shared__ float4 sh_lo[kGrWarps][kMaxLeaf];
-  __shared__ int32_t sh_b[kGrWarps][kMaxLeaf];
   const Tree &T = A.T;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // Warps take groups of particles; acceptance is per particle, so any
@@ -153,12 +169,13 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
     const int32_t slot = s0 + lane;
     const bool act = slot < s1;
     const int32_t a = act ? (T.perm_identity ? slot : T.perm[slot]) : 0;  // identity: state in tree order
-    double xa[3] = {0, 0, 0};
-    for (int ax = 0; ax < dim; ++ax) xa[ax] = A.x[ax][a];
     // the cell of the particle's current position (the key of the build
     // unless the tree is reused); node cubes are those of the build
+    double xa[3] = {0, 0, 0};
+    if (INSIDE && act)
+      for (int ax = 0; ax < dim; ++ax) xa[ax] = A.x[ax][a];
     const unsigned long long ka =
-        !act ? 0ULL
+        !INSIDE || !act ? 0ULL
              : (A.reuse ? morton_key(xa, dim, B, inst, T.inst_lo, T.inst_s0[inst], T.inst_rs0[inst]) : T.skey[slot]);
     const float4 Pa = A.pk.px(a), Qa = A.pk.pxl(a);
     const double e = A.eps * (double)Pa.w;
@@ -169,7 +186,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
     const double th = A.theta;
     const float th2f = (float)(th * th);
     GravSumF acc;
-    int32_t skip_until = -1;
+    int32_t skip_until = act ? -1 : 0x7fffffff;  // an idle lane meets no node
     const int32_t root = T.inst_root[inst];
     const int32_t stop = root >= 0 ? T.skip[root] : root;
     int iter = 0;
@@ -195,8 +212,8 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
         leaf = (e1 - f <= L) || lev == B;
       }
       bool open = false, direct = false;
-      if (act && nd >= skip_until) {
-        const bool inside = A.test_inside && (ka >> (dim * (B - lev))) == T.cell[nd];
+      if (nd >= skip_until) {
+        const bool inside = INSIDE && A.test_inside && (ka >> (dim * (B - lev))) == T.cell[nd];
         bool accept = false;
         float mpf = 0.f;
         R d[3] = {R(0), R(0), R(0)}, r2 = R(0);
@@ -208,7 +225,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
           d[0] = (Pa.x - ch.x) + (Qa.x - cl.x);
           d[1] = (Pa.y - ch.y) + (Qa.y - cl.y);
           d[2] = (Pa.z - ch.z) + (Qa.z - cl.z);
-          r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+          r2 = norm2(d[0], d[1], d[2]);
           mpf = ch.w;
           const float sf = PACKED ? __int_as_float(__float_as_int(s0f) - (lev << 23)) : cl.w;
           const float lhs = sf * sf, rhs = th2f * r2;
@@ -224,9 +241,9 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
         if (accept) {
           const R mp = mpf;
           const R gq = -G * mp * inv_q32(r2 + eps2);
-          acc.add(gq * d[0], gq * d[1], dim == 3 ? gq * d[2] : R(0));
+          acc.add_scaled(gq, d);
           skip_until = sk;
-          ++nacc;
+          if constexpr (COUNT) ++nacc;
         } else if (leaf) {
           direct = true;
           skip_until = sk;
@@ -234,11 +251,16 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
           open = true;
         }
       }
-      const bool any_open = __any_sync(0xffffffffu, open);
+      if (!leaf) {  // no lane sums it directly
+        nd = __any_sync(0xffffffffu, open) ? nd + 1 : sk;
+        continue;
+      }
       const unsigned dmask = __ballot_sync(0xffffffffu, direct);
+      const int32_t node = nd;
+      nd = sk;
       if (dmask) {
         if constexpr (PACKED) {
-          const int4 rec = T.nrec[nd];
+          const int4 rec = T.nrec[node];
           f = rec.x;
           e1 = rec.y;
         }
@@ -252,7 +274,6 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
             qb = A.pk.pxl(bm);
             sh_hi[w][lane] = make_float4(pb.x, pb.y, pb.z, -(float)G * qb.w);  // qb.w = m as float
             sh_lo[w][lane] = make_float4(qb.x, qb.y, qb.z, qb.w);
-            sh_b[w][lane] = bm;
           }
           __syncwarp();
           const bool transposed = __popc(dmask) * kTransposedCost < c * kSerialCost;
@@ -274,7 +295,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
               if (lane < c && bm != ai) {
                 const float dx = (ax - pb.x) + (lx - qb.x), dy = (ay - pb.y) + (ly - qb.y),
                             dz = (az - pb.z) + (lz - qb.z);
-                const float q = dx * dx + dy * dy + dz * dz + e2i;
+                const float q = norm2(dx, dy, dz) + e2i;
                 if (q > 0.f) {
                   const float gq = gmk * inv_q32(q);
                   fx = gq * dx;
@@ -291,34 +312,32 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
               const unsigned okm = __ballot_sync(0xffffffffu, ok);
               if (lane == i) {
                 acc.add((R)fx, (R)fy, dim == 3 ? (R)fz : R(0));
-                nterm += __popc(okm);
+                if constexpr (COUNT) nterm += __popc(okm);
               }
             }
           } else if (direct) {
             for (int k = 0; k < c; ++k) {
-              const int32_t b = sh_b[w][k];
-              if (b == a) continue;
+              if (base + k == slot) continue;  // the particle itself
               R d[3], gm;  // gm = -G m_b
               const float4 ph = sh_hi[w][k], pl = sh_lo[w][k];
               d[0] = (Pa.x - ph.x) + (Qa.x - pl.x);
               d[1] = (Pa.y - ph.y) + (Qa.y - pl.y);
               d[2] = (Pa.z - ph.z) + (Qa.z - pl.z);
               gm = ph.w;
-              const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+              const R r2 = norm2(d[0], d[1], d[2]);
               const R q = r2 + eps2;
               if (!(q > R(0))) continue;
               const R gq = gm * inv_q32(q);
-              acc.add(gq * d[0], gq * d[1], dim == 3 ? gq * d[2] : R(0));
-              ++nterm;
+              acc.add_scaled(gq, d);
+              if constexpr (COUNT) ++nterm;
             }
           }
           __syncwarp();
         }
       }
-      nd = any_open ? nd + 1 : sk;
     }
     if (iter > nnodes) raise_err(A.err, ERR_TIMEOUT);
-    if (A.ctr) {
+    if (COUNT && A.ctr) {
       warp_count(A.ctr + CTR_GRAV_NODES, nacc);
       warp_count(A.ctr + CTR_GRAV_TERMS, nterm);
       if (lane == 0) atomicAdd(A.ctr + CTR_GRAV_VISITS, (unsigned long long)iter);
@@ -482,6 +501,15 @@ __global__ void __launch_bounds__(32, kGrav64Blocks) k_gravity64(GravArgs A) {
   }
 }
 
+template <int DIM>
+static void gravity_mixed(const GravArgs &A, bool packed, int blocks, cudaStream_t st) {
+  const int threads = kGrWarps * 32;
+  if (!packed) k_gravity<DIM, false, true, true><<<blocks, threads, 0, st>>>(A);
+  else if (A.ctr) k_gravity<DIM, true, true, true><<<blocks, threads, 0, st>>>(A);
+  else if (A.test_inside) k_gravity<DIM, true, true, false><<<blocks, threads, 0, st>>>(A);
+  else k_gravity<DIM, true, false, false><<<blocks, threads, 0, st>>>(A);
+}
+
 void gravity_walk(sph_ctx *c, const sph_state *s, const sph_params &p, double *ax, double *ay, double *az,
                   cudaStream_t st, bool reuse) {
   if (s->n == 0) return;
@@ -521,12 +549,10 @@ void gravity_walk(sph_ctx *c, const sph_state *s, const sph_params &p, double *a
   const bool packed = mixed && c->tree.packed_walk;
   const int blocks64 = c->tree.ninst <= 1 ? nblk(s->n << A.share, 32) : c->num_sms * kGrav64Blocks;
   if (s->dim == 3) {
-    if (packed) k_gravity<3, true><<<blocks, kGrWarps * 32, 0, st>>>(A);
-    else if (mixed) k_gravity<3, false><<<blocks, kGrWarps * 32, 0, st>>>(A);
+    if (mixed) gravity_mixed<3>(A, packed, blocks, st);
     else k_gravity64<3><<<blocks64, 32, 0, st>>>(A);
   } else {
-    if (packed) k_gravity<2, true><<<blocks, kGrWarps * 32, 0, st>>>(A);
-    else if (mixed) k_gravity<2, false><<<blocks, kGrWarps * 32, 0, st>>>(A);
+    if (mixed) gravity_mixed<2>(A, packed, blocks, st);
     else k_gravity64<2><<<blocks64, 32, 0, st>>>(A);
   }
   ++sph::g_launches;

@@ -54,3 +54,50 @@ def test_permutation_is_the_stable_sort(n, dim, parts, depth):
     sph.build_tree(ctx, ds, leaf_size=8, max_depth=depth, reorder=True)
     np.testing.assert_array_equal(ds.id.cpu().numpy(), want)
     np.testing.assert_array_equal(ds.x.cpu().numpy(), x[:, want])
+
+
+def _nodes(key, dim, depth, leaf, off):
+    """(level, count) of every node in pre-order, cell by cell from the sorted keys."""
+    out = []
+
+    def cell(a, b, level):
+        out.append((level, b - a))
+        if b - a <= leaf or level == depth:
+            return
+        pre = key[a:b] >> (dim * (depth - level - 1))
+        cuts = [a] + [a + 1 + int(c) for c in np.nonzero(pre[1:] != pre[:-1])[0]] + [b]
+        for lo, hi in zip(cuts[:-1], cuts[1:]):
+            cell(lo, hi, level + 1)
+
+    for lo, hi in zip(off[:-1], off[1:]):
+        if hi > lo:
+            cell(int(lo), int(hi), 0)
+    return np.array(out).T
+
+
+@pytest.mark.parametrize("n,dim,leaf,parts,kind", [
+    (1, 3, 16, 1, "uniform"), (17, 3, 16, 1, "uniform"), (5000, 3, 1, 1, "uniform"), (5000, 2, 2, 1, "uniform"),
+    (20000, 3, 16, 1, "uniform"), (20000, 3, 32, 7, "uniform"), (20000, 2, 8, 3, "grid"), (20000, 3, 16, 1, "clusters"),
+    (3000, 3, 16, 2, "twins"), (40, 3, 16, 1, "twins")])
+def test_nodes_are_the_cells_that_split(n, dim, leaf, parts, kind):
+    from paper_1604_03290_gb300 import sph
+    rng = np.random.default_rng(n + leaf)
+    x = rng.uniform(0.0, 1.0, (dim, n))
+    if kind == "grid":
+        x = np.round(30 * x) / 30
+    if kind == "clusters":  # a long tail of nested cells
+        x = x * 0.5 ** rng.integers(0, 14, n)
+    if kind == "twins":  # full-depth leaves with more than `leaf` members
+        x[:, : n // 2] = x[:, :1]
+    depth = 17
+    ps = wl.lattice_block(nx=n, ny=1, nz=1, dim=dim)
+    ps.x = np.ascontiguousarray(x)
+    off = np.linspace(0, n, parts + 1).astype(np.int64)
+    if parts > 1:
+        ps.inst_off = off
+    ctx = sph.Context(dim, n, max_instances=parts, max_neighbours=4, leaf_size=leaf)
+    sph.build_tree(ctx, sph.DeviceState(ps), leaf_size=leaf, max_depth=depth)
+    nodes = sph.tree_nodes(ctx, 8 * n + 8192)
+    want = _nodes(np.sort(_keys(x, off, depth).astype(np.int64)), dim, depth, leaf, off)
+    np.testing.assert_array_equal(nodes["level"].cpu().numpy(), want[0])
+    np.testing.assert_array_equal(nodes["count"].cpu().numpy(), want[1])

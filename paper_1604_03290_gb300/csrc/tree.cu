@@ -675,39 +675,55 @@ __device__ __forceinline__ int first_node_level(const KeyLevels &K, int64_t i, i
 // nodes are the levels from its first to the first that does not split, which
 // one comparison of keys L slots apart tells: searching each cell's end took
 // 11 us for 4.4k particles (now 5.6), 71 us for 1M (now 57).
+// IT slots per thread: four shorten the look-back's chain of tiles, at small n
+// one spreads the slots over more SMs.  One, four, eight: a tree and partner
+// lists of 4.1k particles 272, 275, 283 us, 33k 397, 396, 400, 111k 528, 523,
+// 527, 263k 794, 786, 790; the mixed adjoint at 1M 4452, 4426, 4437 us.
+template <int IT>
 __global__ void __launch_bounds__(256) k_node_scan(KeyLevels K, int64_t n, int L, const int64_t *__restrict__ inst_off,
                                                    int ninst, Tree T, uint32_t *state, int32_t *err) {
   __shared__ int tile_s;
   __shared__ uint32_t before_s;
   if (threadIdx.x == 0) tile_s = (int)atomicAdd(&T.look[LK_NODES], 1u);
   __syncthreads();
-  const int64_t i = (int64_t)tile_s * 256 + threadIdx.x;
-  int k = 0;
-  if (i < n) {
-    int64_t seg_lo, seg_hi;
-    slot_segment(inst_off, ninst, n, i, seg_lo, seg_hi);
-    const int split = K.split_level(i, L, n), l0 = first_node_level(K, i, seg_lo, seg_hi, L, split);
-    if (l0 <= K.B) k = min(max(l0, split + 1), K.B) - l0 + 1;
+  const int64_t first = ((int64_t)tile_s * 256 + threadIdx.x) * IT;
+  int nodes[IT], sum = 0;
+#pragma unroll
+  for (int j = 0; j < IT; ++j) {
+    const int64_t i = first + j;
+    nodes[j] = 0;
+    if (i < n) {
+      int64_t seg_lo, seg_hi;
+      slot_segment(inst_off, ninst, n, i, seg_lo, seg_hi);
+      const int split = K.split_level(i, L, n), l0 = first_node_level(K, i, seg_lo, seg_hi, L, split);
+      if (l0 <= K.B) nodes[j] = min(max(l0, split + 1), K.B) - l0 + 1;
+    }
+    sum += nodes[j];
   }
   int32_t tot;
-  int32_t off = block_excl_scan(k, &tot);
+  int32_t off = block_excl_scan(sum, &tot);
   if (threadIdx.x < 32) {
     const uint32_t b = look_back_warp(state, tile_s, (uint32_t)tot, err);
     if (threadIdx.x == 0) before_s = b;
   }
   __syncthreads();
   off += (int32_t)before_s;
-  if (i > n) return;
-  T.nstart[i] = off;
-  if (i == n) {
-    *T.nnodes = off <= T.cap_nodes ? off : (int32_t)T.cap_nodes;
-    if (off > T.cap_nodes) raise_err(err, ERR_NODE_OVERFLOW);
-    return;
-  }
   int4 *child = reinterpret_cast<int4 *>(T.child);
-  for (int64_t id = off; id < off + k && id < T.cap_nodes; ++id) {
-    T.nchild[id] = T.arrived[id] = 0;
-    child[2 * id] = child[2 * id + 1] = make_int4(-1, -1, -1, -1);
+#pragma unroll
+  for (int j = 0; j < IT; ++j) {
+    const int64_t i = first + j;
+    if (i > n) return;
+    T.nstart[i] = off;
+    if (i == n) {
+      *T.nnodes = off <= T.cap_nodes ? off : (int32_t)T.cap_nodes;
+      if (off > T.cap_nodes) raise_err(err, ERR_NODE_OVERFLOW);
+      return;
+    }
+    for (int64_t id = off; id < off + nodes[j] && id < T.cap_nodes; ++id) {
+      T.nchild[id] = T.arrived[id] = 0;
+      child[2 * id] = child[2 * id + 1] = make_int4(-1, -1, -1, -1);
+    }
+    off += nodes[j];
   }
 }
 
@@ -1061,7 +1077,8 @@ void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cu
   int ibits = 0;
   while ((1 << ibits) < ninst) ++ibits;
   const int bits = dim * max_depth + ibits, passes = sort_passes(bits);
-  const int node_tiles = nblk(n + 1, 256), group_tiles = nblk(T.cap_nodes, 256);
+  const bool wide = n >= 65536;  // see k_node_scan
+  const int node_tiles = nblk(n + 1, wide ? 1024 : 256), group_tiles = nblk(T.cap_nodes, 256);
   uint32_t *node_state = T.look + kLookFixed + (int64_t)passes * nblk(n, kSortTile) * 256;
   uint32_t *group_state = node_state + node_tiles;
   const int64_t words = group_state + group_tiles - T.look;
@@ -1097,7 +1114,9 @@ void tree_build(sph_ctx *c, const sph_state *s, int leaf_size, int max_depth, cu
     T.perm = T.vals[0];
   }
   KeyLevels K{T.skey, dim, max_depth};
-  { k_node_scan<<<node_tiles, 256, 0, st>>>(K, n, leaf_size, s->inst_off, ninst, T, node_state, c->d_err); ++sph::g_launches; }
+  if (wide) k_node_scan<4><<<node_tiles, 256, 0, st>>>(K, n, leaf_size, s->inst_off, ninst, T, node_state, c->d_err);
+  else k_node_scan<1><<<node_tiles, 256, 0, st>>>(K, n, leaf_size, s->inst_off, ninst, T, node_state, c->d_err);
+  ++sph::g_launches;
   { k_node_emit<<<nblk(std::max<int64_t>(n, 1), 256), 256, 0, st>>>(K, n, leaf_size, s->inst_off, ninst, T.nstart, T); ++sph::g_launches; }
   const int mblocks = nblk(std::max<int64_t>(n, 1), 16);  // a leaf holds at least one particle
   if (dim == 3) k_moments<3><<<mblocks, 128, 0, st>>>(T, s->x[0], s->x[1], s->x[2], s->m, s->h);

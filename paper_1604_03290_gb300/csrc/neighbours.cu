@@ -1,13 +1,11 @@
 // Interaction partners (Sect. 3.5.2), GB300 form.
 //
 // The paper walks the tree once per particle from the root.  Here a warp
-// walks it once for 32 consecutive sorted particles (one "group"): the tree
-// is stored in pre-order, so the walk is a single loop over node ids that
-// either enters a node (id + 1) or jumps over its subtree (skip[id]) - no
-// stack, and every lane follows the same path.  A node is entered when its
-// particle box comes within (h_group + h_node,max)/2 of the group's box,
-// which can only keep more candidates than the paper's test; the set itself
-// is decided per lane by the exact predicate.
+// walks it once for a group of up to 32 particles of sibling cells, 32 nodes
+// at a time, a lane each.  A node is entered when its particle box comes
+// within (h_group + h_node,max)/2 of the group's box, which can only keep
+// more candidates than the paper's test; the set itself is decided per lane
+// by the exact predicate.
 //
 // Predicate: b is a partner of a iff ((dx^2 + dy^2) + dz^2) < h_ab^2 with
 // h_ab = (h_a + h_b)/2, all in FP64 without fused multiply-add.  On GB300

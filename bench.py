@@ -123,14 +123,14 @@ class ClockSampler:
 # now, the figures are stale and are not used (the kernel is then reported
 # against HBM alone, with traffic null).
 NCU_PER_PARTICLE = {
-    "partners": {"inst": 862.46, "dram": 356.52, "fp32_pipe": 0.274, "issue": 0.683, "l1": 0.328,
-                 "src": ("neighbours.cu", "9347fbb88607e52e")},
-    "refine": {"inst": 10.60, "dram": 67.06, "fp32_pipe": 0.095, "issue": 0.228, "l1": 0.290,
-               "src": ("neighbours.cu", "9347fbb88607e52e")},
-    "passA": {"inst": 315.03, "dram": 499.16, "fp32_pipe": 0.384, "issue": 0.582, "l1": 0.695,
-              "src": ("rhs.cu", "34f6a376fba94640")},
-    "passB": {"inst": 336.22, "dram": 347.92, "fp32_pipe": 0.416, "issue": 0.567, "l1": 0.889,
-              "src": ("rhs.cu", "34f6a376fba94640")},
+    "partners": {"inst": 627.26, "dram": 287.12, "fp32_pipe": 0.245, "issue": 0.674, "l1": 0.334,
+                 "src": ("neighbours.cu", "dba6e566e49e559a")},
+    "refine": {"inst": 10.13, "dram": 63.07, "fp32_pipe": 0.111, "issue": 0.247, "l1": 0.340,
+               "src": ("neighbours.cu", "dba6e566e49e559a")},
+    "passA": {"inst": 315.03, "dram": 498.36, "fp32_pipe": 0.388, "issue": 0.588, "l1": 0.699,
+              "src": ("rhs.cu", "9072f1f39261b8d3")},
+    "passB": {"inst": 336.25, "dram": 347.75, "fp32_pipe": 0.417, "issue": 0.574, "l1": 0.892,
+              "src": ("rhs.cu", "9072f1f39261b8d3")},
 }
 
 

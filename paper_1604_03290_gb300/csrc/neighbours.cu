@@ -314,7 +314,9 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
     };
     // 3. the kept candidates against every lane's particle, four at a time
     // (one round of shared loads, four independent distances); the buffer is
-    // padded with candidates out of everyone's reach
+    // padded with candidates out of everyone's reach and of index -2, which
+    // never count: a lane with a position that is not a number or an infinite
+    // h cannot tell them from its partners by distance
     auto test = [&](int nc) {
       const int np = (nc + 3) & ~3;
       if (lane < np - nc) {
@@ -343,7 +345,7 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
           if (unsure) {  // rare: the FP64 predicate
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-              if ((unsure >> u) & 1u)
+              if (((unsure >> u) & 1u) && bs[u] >= 0)
                 in[u] = OWN_H ? exact_within_own_h(x, y, z, h, dim, a, bs[u]) : exact_partner(x, y, z, h, dim, a, bs[u]);
           }
 #pragma unroll
@@ -360,7 +362,7 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
             }
             if constexpr (SHELL) {
               // near the support radius on either side
-              if (other && r2[u] >= h2[u] * kInner2 && r2[u] <= h2[u] * kShell2) {
+              if (other && r2[u] >= h2[u] * kInner2 && r2[u] <= h2[u] * kShell2 && bs[u] >= 0) {
                 if (scnt < kMaxShell) {
                   *sout = bs[u];
                   sin |= (uint32_t)in[u] << scnt;

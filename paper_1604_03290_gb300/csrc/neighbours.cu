@@ -749,14 +749,13 @@ constexpr int kCsrShort = 128;
 constexpr int kCsrWarps = 8;
 __global__ void __launch_bounds__(32 * kCsrWarps) k_csr_fill(const int32_t *__restrict__ nb_idx,
                                                             const int32_t *__restrict__ nb_cnt, int64_t ld,
-                                                            const int32_t *__restrict__ start, int64_t n, int64_t *off,
-                                                            int32_t *idx, int64_t cap, int32_t *err) {
+                                                            const int64_t *__restrict__ off, int64_t n, int32_t *idx,
+                                                            int64_t cap, int32_t *err) {
   __shared__ __align__(16) int32_t lists[kCsrWarps][kCsrShort];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t a = (int64_t)blockIdx.x * kCsrWarps + w;
   if (a > n) return;
-  const int64_t o = start[a];
-  if (lane == 0) off[a] = o;
+  const int64_t o = off[a];
   if (a == n) {
     if (lane == 0 && o > cap) raise_err(err, ERR_CSR_OVERFLOW);
     return;
@@ -804,13 +803,13 @@ __global__ void __launch_bounds__(32 * kCsrWarps) k_csr_fill(const int32_t *__re
   }
 }
 
-void scan_counts(sph_ctx *c, const int32_t *in, int32_t *out, int64_t m, cudaStream_t st);
+void scan_counts(sph_ctx *c, const int32_t *in, int64_t *out, int64_t m, cudaStream_t st);
 
 void partners_to_csr(sph_ctx *c, const sph_state *s, int64_t *off, int32_t *idx, int64_t cap, cudaStream_t st) {
   int64_t n = s->n;
   { k_cnt_copy<<<nblk(n + 1, 256), 256, 0, st>>>(c->nb_cnt, c->tree.ncount, n); ++sph::g_launches; }
-  scan_counts(c, c->tree.ncount, c->tree.nstart, n + 1, st);
-  { k_csr_fill<<<nblk(n + 1, kCsrWarps), 32 * kCsrWarps, 0, st>>>(c->nb_idx, c->nb_cnt, c->cap_n, c->tree.nstart, n, off, idx, cap,
+  scan_counts(c, c->tree.ncount, off, n + 1, st);
+  { k_csr_fill<<<nblk(n + 1, kCsrWarps), 32 * kCsrWarps, 0, st>>>(c->nb_idx, c->nb_cnt, c->cap_n, off, n, idx, cap,
                                                c->d_err); ++sph::g_launches; }
 }
 

@@ -276,59 +276,73 @@ __global__ void k_pack(const double *__restrict__ x, const double *__restrict__ 
 // the order their blocks start, so a tile only ever waits for blocks that
 // are running.  Every wait is bounded; one that runs out raises the timeout
 // bit and goes on with the sum so far, which every later access tolerates.
-// State word: count in the low 30 bits, then 1 = the tile's own count, 2 =
-// inclusive.
+// State word W (one store, one load): its two top bits are 1 = the tile's own
+// count, 2 = inclusive, the rest the count.  32 bits hold 2^30 - 1: enough for
+// the particles of a digit and for walk groups, and for nodes, whose sums stop
+// there and so exceed any node capacity that fits the device (236 bytes a node).
+// Counts of other things than particles (k_scan) take 64 bits.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kLookOwn = 1u << 30, kLookIncl = 2u << 30, kLookVal = kLookOwn - 1u;
+template <class W>
+struct Look {
+  static constexpr int kShift = 8 * sizeof(W) - 2;
+  static constexpr W kOwn = (W)1 << kShift, kIncl = (W)2 << kShift, kVal = kOwn - 1;
+};
+constexpr uint32_t kLookOwn = Look<uint32_t>::kOwn, kLookIncl = Look<uint32_t>::kIncl, kLookVal = Look<uint32_t>::kVal;
 constexpr int kLookPolls = 1 << 22;
 
-__device__ __forceinline__ uint32_t look_load(const uint32_t *p) { return *(const volatile uint32_t *)p; }
+template <class W>
+__device__ __forceinline__ W look_load(const W *p) {
+  return *(const volatile W *)p;
+}
 
 // Sum of the tiles before `tile` for one counter; called by a whole warp,
 // lane i reading the i-th tile back.  Publishes the inclusive sum.
-__device__ __forceinline__ uint32_t look_back_warp(uint32_t *state, int tile, uint32_t own, int32_t *err) {
+template <class W>
+__device__ __forceinline__ W look_back_warp(W *state, int tile, W own, int32_t *err) {
+  using K = Look<W>;
   const int lane = threadIdx.x & 31;
-  if (lane == 0) *(volatile uint32_t *)&state[tile] = own | (tile == 0 ? kLookIncl : kLookOwn);
-  uint32_t before = 0;
+  if (lane == 0) *(volatile W *)&state[tile] = own | (tile == 0 ? K::kIncl : K::kOwn);
+  W before = 0;
   for (int t = tile - 1; t >= 0; t -= 32) {
     const int mine = t - lane;
-    uint32_t v = kLookIncl;  // before the first tile: nothing, known
+    W v = K::kIncl;  // before the first tile: nothing, known
     if (mine >= 0) {
       int polls = 0;
-      while (((v = look_load(&state[mine])) >> 30) == 0u && ++polls < kLookPolls) __nanosleep(20);
+      while (((v = look_load(&state[mine])) >> K::kShift) == 0 && ++polls < kLookPolls) __nanosleep(20);
       if (polls >= kLookPolls) raise_err(err, ERR_TIMEOUT);
     }
-    const unsigned incl = __ballot_sync(0xffffffffu, (v >> 30) != 1u);
+    const unsigned incl = __ballot_sync(0xffffffffu, (v >> K::kShift) != 1);
     const int last = incl ? __ffs(incl) - 1 : 31;
-    uint32_t sum = lane <= last ? v & kLookVal : 0u;
+    W sum = lane <= last ? v & K::kVal : (W)0;
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    before += sum;
+    before = min(before + sum, (W)K::kVal);
     if (incl) break;
   }
-  if (lane == 0 && tile > 0) *(volatile uint32_t *)&state[tile] = (before + own) | kLookIncl;
+  if (lane == 0 && tile > 0) *(volatile W *)&state[tile] = min(before + own, (W)K::kVal) | K::kIncl;
   return before;
 }
 
-__device__ __forceinline__ int32_t block_excl_scan(int32_t v, int32_t *total) {
-  __shared__ int32_t ws[32];
+template <class T>
+__device__ __forceinline__ T block_excl_scan(T v, T *total) {
+  __shared__ T ws[32];
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  int32_t s = v;
+  T s = v;
   for (int o = 1; o < 32; o <<= 1) {
-    int32_t t = __shfl_up_sync(0xffffffffu, s, o);
+    T t = __shfl_up_sync(0xffffffffu, s, o);
     if (lane >= o) s += t;
   }
   if (lane == 31) ws[w] = s;
   __syncthreads();
   if (w == 0) {
-    int32_t t = lane < nw ? ws[lane] : 0;
+    T t = lane < nw ? ws[lane] : 0;
     for (int o = 1; o < 32; o <<= 1) {
-      int32_t u = __shfl_up_sync(0xffffffffu, t, o);
+      T u = __shfl_up_sync(0xffffffffu, t, o);
       if (lane >= o) t += u;
     }
     ws[lane] = t;
   }
   __syncthreads();
-  int32_t res = s - v + (w > 0 ? ws[w - 1] : 0);
+  T res = s - v + (w > 0 ? ws[w - 1] : 0);
   *total = ws[nw - 1];
   __syncthreads();
   return res;
@@ -555,45 +569,57 @@ void sort_pairs(sph_ctx *c, int64_t n, int bits, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// Exclusive scan of int32 counts (length m), one pass
+// Exclusive scan of non-negative int32 counts (length m), one pass.  Sums are
+// kept in 64 bits (partners and flaws number more than 2^30 well within the
+// device's memory); O holds the offsets.
 // ---------------------------------------------------------------------------
 constexpr int kScanThreads = 256, kScanItems = 16, kScanTile = kScanThreads * kScanItems;
 
-__global__ void __launch_bounds__(kScanThreads) k_scan(const int32_t *in, int32_t *out,  // may be the same
-                                                       int64_t m, uint32_t *ticket, uint32_t *state, int32_t *err) {
+template <class O>
+__global__ void __launch_bounds__(kScanThreads) k_scan(const int32_t *in, O *out,  // may be the same
+                                                       int64_t m, uint32_t *ticket, uint64_t *state, int32_t *err) {
   __shared__ int tile_s;
-  __shared__ uint32_t before_s;
+  __shared__ uint64_t before_s;
   if (threadIdx.x == 0) tile_s = (int)atomicAdd(ticket, 1u);
   __syncthreads();
   const int64_t at = (int64_t)tile_s * kScanTile + (int64_t)threadIdx.x * kScanItems;
   int32_t v[kScanItems];
-  int32_t s = 0;
+  int64_t s = 0;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
     v[k] = (at + k < m) ? in[at + k] : 0;
     s += v[k];
   }
-  int32_t tot;
-  int32_t off = block_excl_scan(s, &tot);
+  int64_t tot;
+  int64_t off = block_excl_scan(s, &tot);
   if (threadIdx.x < 32) {
-    const uint32_t b = look_back_warp(state, tile_s, (uint32_t)tot, err);
+    const uint64_t b = look_back_warp(state, tile_s, (uint64_t)tot, err);
     if (threadIdx.x == 0) before_s = b;
   }
   __syncthreads();
-  off += (int32_t)before_s;
+  off += (int64_t)before_s;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
-    if (at + k < m) out[at + k] = off;
+    if (at + k < m) out[at + k] = (O)off;
     off += v[k];
   }
 }
 
-void scan_counts(sph_ctx *c, const int32_t *in, int32_t *out, int64_t m, cudaStream_t st) {
+template <class O>
+static void scan_run(sph_ctx *c, const int32_t *in, O *out, int64_t m, cudaStream_t st) {
+  static_assert(kLookFixed % 2 == 0, "64-bit state words");
   Tree &T = c->tree;
   const int tiles = nblk(m, kScanTile);
-  cudaMemsetAsync(T.look, 0, sizeof(uint32_t) * (kLookFixed + tiles), st);
-  k_scan<<<tiles, kScanThreads, 0, st>>>(in, out, m, T.look, T.look + kLookFixed, c->d_err);
+  cudaMemsetAsync(T.look, 0, sizeof(uint32_t) * (kLookFixed + 2 * (int64_t)tiles), st);
+  k_scan<<<tiles, kScanThreads, 0, st>>>(in, out, m, T.look, (uint64_t *)(T.look + kLookFixed), c->d_err);
   ++sph::g_launches;
+}
+// 32-bit offsets: the caller's total is at most 2^31 - 1
+void scan_counts(sph_ctx *c, const int32_t *in, int32_t *out, int64_t m, cudaStream_t st) {
+  scan_run(c, in, out, m, st);
+}
+void scan_counts(sph_ctx *c, const int32_t *in, int64_t *out, int64_t m, cudaStream_t st) {
+  scan_run(c, in, out, m, st);
 }
 
 // Words of Tree::look a context for N particles and `cap` nodes needs: a

@@ -62,9 +62,11 @@ __device__ __forceinline__ double slope64(double q) {
   const double a1 = in ? 1.0 : -1.0, b1 = in ? 0.0 : 1.0, c1 = in ? 3.0 : 1.0, d1 = in ? -2.0 : -1.0;
   return fma(a1, q, b1) * fma(c1, q, d1);
 }
-// (h^D / sigma) W: 1 + 6 q^2 (q - 1), or 2 (1 - q)^3
+// (h^D / sigma) W: 1 + 6 q^2 (q - 1), or 2 (1 - q)^3.  The q of a partner (r^2 <
+// h^2) may round above 1, where W is 0: a negative value would give NaN under a
+// non-integer power (artificial stress).  The sign of 1 - q is tested on its bits.
 __device__ __forceinline__ double value64(double q) {
-  const double t = below_half(q) ? q : 1.0 - q, t2 = t * t;
+  const double e = 1.0 - q, t = below_half(q) ? q : ((int64_t)dbits(e) < 0 ? 0.0 : e), t2 = t * t;
   return below_half(q) ? fma(6.0 * t2, t - 1.0, 1.0) : 2.0 * t2 * t;
 }
 

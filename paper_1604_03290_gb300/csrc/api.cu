@@ -578,13 +578,14 @@ static sph_status check_continue(sph_ctx *c, const sph_state *s, const sph_param
 }
 
 // Keeps what a later call needs to continue the tree window of this one.
-static void keep_window(sph_ctx *c, const sph_state *s, const sph_params *p, int age, cudaStream_t st) {
+static void keep_window(sph_ctx *c, const sph_state *s, const sph_params *p, int age, bool lists, cudaStream_t st) {
   StepBufs &B = c->st;
   const int64_t n = s->n;
   for (int k = 0; k < s->dim; ++k) cudaMemcpyAsync(B.snap[k], s->x[k], sizeof(double) * n, cudaMemcpyDeviceToDevice, st);
   cudaMemcpyAsync(B.snap[3], s->h, sizeof(double) * n, cudaMemcpyDeviceToDevice, st);
   c->win_valid = true;
   c->win_age = age;
+  c->win_lists = lists;
   c->win_R = p->tree_reuse;
   c->win_n = n;
   c->win_ninst = s->ninst > 0 ? s->ninst : 1;
@@ -642,12 +643,16 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
   // last walk, the step's first one or, on a reused tree, the build step's
   // (a walk follows only where the particles moved too far since it)
   const bool refine = reuse_pred && c->tune.walk_every_eval == 0;
+  // the lists, shells and groups in the context are those of the walk that a
+  // refine starts from: the build's, recorded with shells, and no walk since
+  bool lists = false;
   // a window of R steps on one tree may span calls (params.tree_continue)
   const bool window = R > 0 && !(p->n_des > 0.0);
   int age = 0;
   if (window && p->tree_continue) {
     if ((r = check_continue(c, s, p, st)) != SPH_OK) return r;
     age = c->win_age;
+    lists = c->win_lists;
   }
   // the FP32 views hold s already: the last corrector wrote them (the first
   // step of a call packs, as the state may have been changed between calls)
@@ -671,6 +676,7 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
       prof_end(c, st, pr);
       if (R > 0) cudaMemsetAsync(B.dbuild, 0, sizeof(unsigned long long), st);
       partners_gravity_passes(c, s, mt, *p, d[0], st, nullptr, false, refine);
+      lists = refine;
     } else {
       if (!packed) {
         pr = prof_begin(c, st, PH_TREE);
@@ -679,8 +685,10 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
       }
       // the lists and shells of the build step's walk stay in place: while
       // the displacement since that walk is within the shell's bound, the
-      // partners are refined from them (else a walk over the widened boxes)
-      partners_gravity_passes(c, s, mt, *p, d[0], st, B.dbuild, p->gravity, false, refine ? B.disp_s : nullptr);
+      // partners are refined from them (else a walk over the widened boxes,
+      // which takes their place for the rest of the window)
+      lists = lists && refine;
+      partners_gravity_passes(c, s, mt, *p, d[0], st, B.dbuild, p->gravity, false, lists ? B.disp_s : nullptr);
     }
     pr = prof_begin(c, st, PH_INTEGRATE);
     timestep_reduce(c, s, *p, d[0], st);
@@ -700,7 +708,7 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
       // displacement since the walk whose lists are refined: this step's walk
       // at a build, the build step's walk otherwise
       const unsigned long long *since = build ? B.dmove : B.dgrow;
-      partners_gravity_passes(c, &q, mt, *p, d[1], st, since, p->gravity, false, refine ? B.disp_q : nullptr);
+      partners_gravity_passes(c, &q, mt, *p, d[1], st, since, p->gravity, false, lists ? B.disp_q : nullptr);
     } else {
       rhs_all(c, &q, mt, *p, d[1], st);
     }
@@ -720,7 +728,7 @@ sph_status sph_step(sph_ctx *c, sph_state *s, const sph_material *mats, int32_t 
     prof_end(c, st, pr);
   }
   if (dt && nsteps > 0) cudaMemcpyAsync(dt, B.dt, sizeof(double) * ninst, cudaMemcpyDeviceToDevice, st);
-  if (window) keep_window(c, s, p, age, st);
+  if (window) keep_window(c, s, p, age, lists, st);
   return finish(c, p, st, "sph_step");
 }
 

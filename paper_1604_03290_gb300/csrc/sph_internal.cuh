@@ -223,6 +223,7 @@ struct sph_ctx {
   // tree window of sph_step (tree_reuse) that a later call may continue:
   // valid only while no other call has touched the tree or the lists
   bool win_valid, win_was;
+  bool win_lists;  // a refine may start from the lists, shells and groups of the window's build walk
   int win_age, win_R, win_ninst, win_leaf, win_depth, win_gravity;
   int64_t win_n;
   // allocation list

@@ -1002,13 +1002,19 @@ __global__ void __launch_bounds__(128) k_moments(Tree T, const double *__restric
   int32_t node = sub == 0 ? leaf : -1;  // finished, its parent to be told by this lane
   // upwards: of the nodes finished in a round, those that complete a parent
   while (__any_sync(all, node >= 0)) {
-    __threadfence();
+    // the lane that counts up the parent fences after the warp's barrier, so
+    // that the stores of all its team's lanes come before its count; the lanes
+    // that read children likewise come after a barrier past the last one's fence
     __syncwarp();
+    __threadfence();
     const int32_t p = node >= 0 ? T.parent[node] : -1;
     const bool win = p >= 0 && atomicAdd(&T.arrived[p], 1) == T.nchild[p] - 1;
     node = win ? p : -1;
     unsigned todo = __ballot_sync(all, win);
-    if (todo) __threadfence();
+    if (todo) {
+      __threadfence();
+      __syncwarp();
+    }
     while (todo) {
       unsigned pick = todo;  // team t takes the t-th parent left
       for (int t = 0; t < team; ++t) pick &= pick - 1;

@@ -9,8 +9,10 @@
 // leaves a relative error of the order of the rounding of its last operation:
 //   1/x:        e = 1 - x y,    y (1 + e + e^2)             error e^3
 //   1/sqrt(x):  e = 1 - x y^2,  y (1 + e/2 + 3 e^2 / 8)     error (5/16) e^3
-// in three and five FP64 instructions.  tests/test_gpu_fp64_forms.py bounds
-// both by two units in the last place.  Operands outside 2^-959..2^961 (where
+// in three and five FP64 instructions.  The errors are at most 0.51 and 1.02
+// units in the last place (0.5 and 1.5 for the correctly rounded division and
+// for a division by a correctly rounded root), which
+// tests/test_gpu_fp64_reciprocals.py derives and holds them to.  Operands outside 2^-959..2^961 (where
 // the seed could flush or overflow), zero, negatives, infinities and NaN take
 // the correctly rounded operations, out of line.  Divisions outside the pair
 // loops keep the language's operator.

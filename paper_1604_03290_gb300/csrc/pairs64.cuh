@@ -45,7 +45,7 @@ struct Lanes64 {
     n = 1 << shift;
     const int lane = threadIdx.x & 31;
     sub = lane & (n - 1);
-    mask = (n == 32 ? ~0u : (1u << n) - 1u) << (lane - sub);
+    mask = ((1u << n) - 1u) << (lane - sub);  // n <= 8
   }
   __device__ __forceinline__ double sum(double v) const {
     for (int o = 1; o < n; o <<= 1) v += __shfl_xor_sync(mask, v, o);
@@ -105,7 +105,9 @@ __device__ __forceinline__ void radial64(const Support64<DIM> &H, double r2, dou
 // over the SMs' FP64 units: one-warp blocks while that leaves fewer than eight
 // 128-thread blocks per SM; and with fewer than kLaneWarps warps per SM even
 // that leaves the unit idle between dependent operations, so 2, 4 or 8 lanes
-// share a particle's list (the particle's own update is repeated on each).
+// share a particle's list.  After the sums only the first lane of each group goes
+// on to the particle's own update, which a warp then runs with 4 to 16 lanes
+// active; the measured thresholds include that.
 // Against one lane, at thresholds of 2, 4 and 8 warps: rings at 4.4k (ten
 // steps) 6.90 -> 5.67, 5.79, 5.80 ms; a right-hand side at 8k 902 -> 815, 804,
 // 920 us and at 27k 1078 -> 1080, 1078, 1125 us; RK3 at 14k 3.18 -> 3.18, 2.96,

@@ -297,7 +297,9 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
     // relative coordinates carry an error of a few 1e-7 of the group's extent + h
     const float rslack = 1e-5f * (fmaxf(fmaxf(rh[0] - rl[0], rh[1] - rl[1]), rh[2] - rl[2]) + hg);
     const int32_t root = T.inst_root[inst];
-    int cnt = 0, scnt = 0;
+    // a square of the support that FP32 cannot hold (h infinite, or not a number)
+    // tells no candidate from the padding of the test: no shell, always walked
+    int cnt = 0, scnt = SHELL && !(hha * hha * kShell2 < INFINITY) ? kMaxShell + 1 : 0;
     uint32_t sin = 0;  // shell entries that are partners (bit per entry)
     unsigned ntest = 0;  // candidates this lane tested (counters)
     int32_t *out = nb_idx + a, *sout = SHELL ? sh_idx + a : nullptr;  // a = -1 writes nothing
@@ -362,7 +364,7 @@ __global__ void SPH_WALK_BOUNDS k_partners(Tree T, PackedF32 pk, const double *_
             }
             if constexpr (SHELL) {
               // near the support radius on either side
-              if (other && r2[u] >= h2[u] * kInner2 && r2[u] <= h2[u] * kShell2 && bs[u] >= 0) {
+              if (other && r2[u] >= h2[u] * kInner2 && r2[u] <= h2[u] * kShell2) {
                 if (scnt < kMaxShell) {
                   *sout = bs[u];
                   sin |= (uint32_t)in[u] << scnt;

@@ -123,10 +123,10 @@ class ClockSampler:
 # now, the figures are stale and are not used (the kernel is then reported
 # against HBM alone, with traffic null).
 NCU_PER_PARTICLE = {
-    "partners": {"inst": 627.26, "dram": 287.12, "fp32_pipe": 0.245, "issue": 0.674, "l1": 0.334,
-                 "src": ("neighbours.cu", "dba6e566e49e559a")},
-    "refine": {"inst": 10.13, "dram": 63.07, "fp32_pipe": 0.111, "issue": 0.247, "l1": 0.340,
-               "src": ("neighbours.cu", "dba6e566e49e559a")},
+    "partners": {"inst": 627.21, "dram": 288.43, "fp32_pipe": 0.244, "issue": 0.675, "l1": 0.335,
+                 "src": ("neighbours.cu", "b16454c1fb107cce")},
+    "refine": {"inst": 10.13, "dram": 63.07, "fp32_pipe": 0.109, "issue": 0.244, "l1": 0.334,
+               "src": ("neighbours.cu", "b16454c1fb107cce")},
     "passA": {"inst": 315.03, "dram": 498.36, "fp32_pipe": 0.388, "issue": 0.588, "l1": 0.699,
               "src": ("rhs.cu", "9072f1f39261b8d3")},
     "passB": {"inst": 336.25, "dram": 347.75, "fp32_pipe": 0.417, "issue": 0.574, "l1": 0.892,

@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kGrWarps * 32, SPH_GRAV_MIN_BLOCKS) k_gravity(
 //  - a term takes 17 FP64 instructions, with rsqrt64 in place of a square root
 //    and a division, and G applied to the sums.
 // A lane's terms are summed in the order of its own walk, whatever the warp.
-// 50k cloud, the whole call: 9.05 -> 3.14 ms (before: acceptance and terms in FP64
+// 50k cloud, the whole call: 9.05 -> 2.57 ms (before: acceptance and terms in FP64
 // at the node, about 45 instructions each).
 // ---------------------------------------------------------------------------
 constexpr int kList64 = 64;  // entries per lane: a leaf's 32 members fit while 32 wait

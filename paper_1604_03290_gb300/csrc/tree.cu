@@ -700,7 +700,7 @@ __device__ __forceinline__ int first_node_level(const KeyLevels &K, int64_t i, i
 // slot's nodes also get their children and arrival counts cleared.  A slot's
 // nodes are the levels from its first to the first that does not split, which
 // one comparison of keys L slots apart tells: searching each cell's end took
-// 11 us for 4.4k particles (now 5.6), 71 us for 1M (now 57).
+// 11 us for 4.4k particles (now 5.6), 71 us for 1M (now 43).
 // IT slots per thread: four shorten the look-back's chain of tiles, at small n
 // one spreads the slots over more SMs.  One, four, eight: a tree and partner
 // lists of 4.1k particles 272, 275, 283 us, 33k 397, 396, 400, 111k 528, 523,
